@@ -269,12 +269,13 @@ int dm_batch_latency(dm_ctx *ctx, double *out_ms, int32_t n);
  * step; <= 0 = none). */
 int dm_set_tuning(dm_ctx *ctx, int autotune, double hash_load_factor, double heavy_rows);
 
-/* on = 1: counted matches (DM_COUNT, dm_match_shard) on the device-driven path run their
- * plan's last two joins as one kernel when both map 1 to 4 new vertices: the survivors of the
- * second-to-last join are joined and counted in shared memory, so the table between the two
+/* on = 1: counted matches (DM_COUNT, dm_match_shard) that run a launch per join on the device-driven
+ * path run their plan's last two joins as one kernel when both map 1 to 4 new vertices: the survivors
+ * of the second-to-last join are joined and counted in shared memory, so the table between the two
  * joins (the largest of a path-like plan) is never written to or read from device memory.
- * on = 0 (the default) runs every join as its own launch (Alg. 1 step by step). Results are
- * identical either way. No counterpart in the paper (its joins are library calls). */
+ * on = 0 (the default) runs every such join as its own launch. Plans that suit it run several steps
+ * a launch either way (graphs of at most 65 534 vertices, key groups of similar size; csrc/chain.cu).
+ * Results are identical in every case. No counterpart in the paper (its joins are library calls). */
 int dm_set_fusion(dm_ctx *ctx, int on);
 
 /* Block shape of dm_match_batch when autotuning is off (no counterpart in the paper):
@@ -460,11 +461,13 @@ typedef struct dm_stats {
     int32_t n_steps;                  /* join steps of the last dm_match / dm_score_topk */
     int64_t rows[DM_MAX_STEPS];       /* rows of the intermediate table after each step */
     int64_t candidates[DM_MAX_STEPS]; /* joined rows before filtering, per step */
-    int64_t chunks;                   /* join launches (> n_steps when streaming) */
-    int64_t max_rows;                 /* largest intermediate table held at once */
+    int64_t chunks;                   /* join steps run (> n_steps when streaming, or when a launch of
+                                         several steps left part of its input to another one) */
+    int64_t max_rows;                 /* most rows of a step but the last, or of a chunk when streaming */
     double join_ms;                   /* device time of the join kernels (CUDA events) */
-    int64_t join_launches;
-    double join_bytes;                /* algorithmic bytes of the join launches */
+    int64_t join_launches;            /* join steps launched (a launch may run several) */
+    double join_bytes;                /* algorithmic bytes of the join launches: tables that stay in
+                                         shared memory between the steps of a launch count nothing */
     double total_ms;                  /* host wall time of the call */
     int64_t kernel_launches;          /* launches of the library's own kernels during the call */
 } dm_stats;

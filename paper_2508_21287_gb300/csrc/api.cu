@@ -60,6 +60,11 @@ struct DevGraph {
   // every edge and vertex weight is >= 0, so a partial score never exceeds a full one and
   // top-k may drop rows whose partial score is above the current k-th best
   bool nonneg_weights = true;
+  // what decides which pairs of pattern vertices can collide (chain.cu): a lower bound of the
+  // girth, and whether every cycle is even
+  int32_t girth = 3;
+  bool bipartite = false;
+  double edge_deg = 0;  // mean degree of the vertices that edges lead to
   std::map<int, DevTable> motifs;
   std::map<std::tuple<int, int, int, int>, Index> indices;  // (motif, key position 0, 1, sort-merge)
 };
@@ -83,6 +88,8 @@ struct dm_ctx {
   // arena of the device-driven path: two halves alternate as the input and output of a step
   unsigned char *arena = nullptr;
   size_t arena_bytes = 0;
+  void *tabs = nullptr;  // candidate tables of the plan that runs (chain.cu)
+  int64_t tab_bytes = 0;
   unsigned long long *d_ctr_steps = nullptr;  // CTR_N counters per step
   unsigned long long *h_ctr_steps = nullptr;
   struct BatchState *batch = nullptr;  // cached device image of the last batch of plans
@@ -228,6 +235,27 @@ bool connected(const HostCSR &g, int32_t n) {
       }
   }
   return cnt == n;
+}
+
+// Whether a connected graph has no odd cycle.
+bool two_colourable(const HostCSR &g, int32_t n) {
+  std::vector<signed char> col(n, -1);
+  std::vector<int32_t> st{0};
+  col[0] = 0;
+  while (!st.empty()) {
+    const int32_t u = st.back();
+    st.pop_back();
+    for (int32_t k = g.rp[u]; k < g.rp[u + 1]; k++) {
+      const int32_t v = g.ci[k];
+      if (col[v] < 0) {
+        col[v] = 1 - col[u];
+        st.push_back(v);
+      } else if (col[v] == col[u]) {
+        return false;
+      }
+    }
+  }
+  return true;
 }
 
 // ------------------------------------------------------------------ sorting ------------
@@ -441,6 +469,15 @@ struct StepRT {
   int64_t max_group = 1;
   int64_t motif_bytes = 0;
 };
+
+// Launches of several steps (chain.cu): shared memory of an SM, warps it holds at most, the most bytes
+// of candidate tables; and what cuts a plan into launches: the cost of a launch (its start, the first
+// loads of every step, the uneven end), of a row at full occupancy (a 24-vertex path on 16 082 vertices:
+// 149 M rows in 2.2 ms), and of a byte of a table between launches.
+constexpr int CHAIN_SM_BYTES = 224 * 1024;
+constexpr int CHAIN_WARPS = 16;
+constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20;
+constexpr double CHAIN_LAUNCH_NS = 15000, CHAIN_ROW_NS = 0.015, CHAIN_BYTE_NS = 0.0002;
 
 struct Exec {
   dm_ctx *c;
@@ -873,6 +910,510 @@ struct Exec {
     return sink->take(c, t);
   }
 
+  // How the plan runs in launches of several steps each (chain.cu).
+  struct Chain {
+    std::vector<dmk::ChainArgs> launch;
+    dmk::ChainTables tab;                // what the candidates bring
+    int n_tab = 0;
+    std::vector<int64_t> tab_off;        // place of each table in the context's buffer
+    std::vector<int64_t> ids, extra;     // per step: 1 + place of its tables (0: none)
+    int64_t tab_bytes = 0;
+    bool needs_arena = false;
+  };
+
+  // Estimated rows after each step, for the cut into launches only. A new vertex next to a mapped one
+  // with k mapped neighbours finds about D - k places, D the mean degree met along an edge; an edge that
+  // closes a cycle is there for about one row in eight (lattices: 1/7 to 1/9 of the rows of a 12-cycle).
+  std::vector<double> chain_rows() const {
+    const int np = p->n_p;
+    std::vector<std::vector<int>> adj(np);
+    std::vector<char> in(np, 0);
+    std::vector<double> rows;
+    double r = (double)st[0].seed_table->n;
+    for (size_t j = 0; j < p->steps.size(); j++) {
+      const StepSpec &s = p->steps[j];
+      MotifDef md;
+      motif_def(s.motif, &md);
+      auto join = [&](int a, int b) {
+        adj[a].push_back(b);
+        adj[b].push_back(a);
+      };
+      std::vector<char> used(md.edges.size(), 0);
+      for (bool more = true; more && j;) {  // edges of the motif that reach a new vertex
+        more = false;
+        for (size_t e = 0; e < md.edges.size(); e++) {
+          int a = s.slice[md.edges[e].first], b = s.slice[md.edges[e].second];
+          if (used[e] || in[a] == in[b]) continue;
+          if (in[b]) std::swap(a, b);
+          r *= std::max(0.3, g->edge_deg - (double)adj[a].size());
+          join(a, b);
+          in[b] = 1;
+          used[e] = 1;
+          more = true;
+        }
+      }
+      for (size_t e = 0; e < md.edges.size(); e++) {
+        const int a = s.slice[md.edges[e].first], b = s.slice[md.edges[e].second];
+        if (used[e]) continue;
+        if (j) r *= 0.125;
+        join(a, b);
+        in[a] = in[b] = 1;
+      }
+      for (int i = 0; i < s.n_be; i++) {
+        r *= 0.125;
+        join(s.be_vtx[i][0], s.be_vtx[i][1]);
+      }
+      in[s.slice[0]] = 1;
+      rows.push_back(r);
+    }
+    return rows;
+  }
+
+  // Lay the plan out for chain.cu; false when it is not one of those it takes. It needs 16-bit ids,
+  // the adjacency bitmap, steps of at most CH_NEW new vertices and further keys, rows of at most
+  // CH_CHUNKS chunks, and groups that suit one row a lane: a step whose longest key group is
+  // over four times the mean would leave most lanes idle; such plans stay with the per-step kernel,
+  // which deals candidates out evenly.
+  bool chain_layout(Chain &C) const {
+    const int S = (int)st.size(), np = p->n_p;
+    if (S < 2 || S > 64 || g->V > 65534 || !g->adj || p->induced || p->join_algo == DM_JOIN_SORTMERGE) return false;
+    const bool count_mode = mode == DM_COUNT;
+    for (int j = 1; j < S; j++) {
+      const StepSpec &s = p->steps[j];
+      const StepRT &r = st[j];
+      if (s.n_keys < 1 || s.n_be > 8 || !r.ix || r.ix->keys || r.ix->v.n > dmk::CH_MAX_ROWS) return false;
+      const int64_t groups = std::max<int64_t>(1, r.ix->distinct);
+      if (r.max_group > 4 * ((r.ix->v.n + groups - 1) / groups) || r.max_group > dmk::CH_MAX_GROUP) return false;
+      const int further = s.n_keys - r.ix->v.nkeys;
+      if (s.n_new + further > dmk::CH_NEW || further > 4) return false;
+    }
+    const StepSpec &s0 = p->steps[0];
+    if (s0.n_be > 8) return false;
+    for (int i = 0; i < s0.n_new; i++)
+      if (s0.new_mpos[i] != i) return false;  // column i of the first table is its position i
+
+    // the columns each new vertex is compared with, from the pattern edges enforced up to its step,
+    // and the columns each step reads
+    std::vector<std::vector<int>> adj(np);
+    auto enforce = [&](const StepSpec &s) {
+      MotifDef md;
+      motif_def(s.motif, &md);
+      auto add = [&](int a, int b) {
+        adj[a].push_back(b);
+        adj[b].push_back(a);
+      };
+      for (auto &e : md.edges) add(s.slice[e.first], s.slice[e.second]);
+      for (int i = 0; i < s.n_be; i++) add(s.be_vtx[i][0], s.be_vtx[i][1]);
+    };
+    enforce(s0);
+    std::vector<std::vector<std::vector<int>>> ck(S);
+    std::vector<std::vector<int>> ex(S);  // one key, one new vertex: mapped pattern neighbours of the key
+    std::vector<std::vector<char>> need(S + 1, std::vector<char>(MAXW, 0));  // by steps >= j
+    for (int j = 1; j < S; j++) {
+      const StepSpec &s = p->steps[j];
+      if (s.n_keys == 1 && s.n_new == 1)
+        for (int v : adj[p->col_vertex[s.key_col[0]]])
+          for (int col = 0; col < s.w_in && ex[j].size() < 2; col++)
+            if (p->col_vertex[col] == v && std::find(ex[j].begin(), ex[j].end(), col) == ex[j].end()) ex[j].push_back(col);
+      enforce(s);
+      ck[j].resize(s.n_new);
+      for (int i = 0; i < s.n_new; i++) {
+        std::vector<int> dist(np, -1), q{(int)s.slice[s.new_mpos[i]]};
+        dist[q[0]] = 0;
+        for (size_t h = 0; h < q.size(); h++)
+          for (int v : adj[q[h]])
+            if (dist[v] < 0) {
+              dist[v] = dist[q[h]] + 1;
+              q.push_back(v);
+            }
+        for (int col = 0; col < s.w_in; col++) {
+          const int v = p->col_vertex[col], d = dist[v];
+          bool in_slice = false;
+          for (int m = 0; m < s.k; m++) in_slice |= s.slice[m] == v;
+          if (in_slice || d == 1 || (d > 2 && (d < g->girth || (g->bipartite && (d & 1))))) continue;
+          ck[j][i].push_back(col);
+          need[j][col] = 1;
+        }
+      }
+      for (int i = 0; i < s.n_keys; i++) need[j][s.key_col[i]] = 1;
+      for (int i = 0; i < s.n_be; i++)
+        for (int h = 0; h < 2; h++)
+          if (s.be_col[i][h] < s.w_in) need[j][s.be_col[i][h]] = 1;
+    }
+    if (!count_mode)  // every column is handed over in the end
+      for (int col = 0; col < np; col++) need[S][col] = 1;
+    for (int j = S - 1; j >= 1; j--)
+      for (int col = 0; col < np; col++) need[j][col] |= need[j + 1][col];
+
+    // a place in the row for every column: the first free one of its colour class
+    std::vector<int> cls(np, -1);
+    bool two = g->bipartite;
+    if (two) {
+      std::vector<int> q{(int)s0.slice[0]};
+      cls[q[0]] = 0;
+      for (size_t h = 0; h < q.size(); h++)
+        for (int v : adj[q[h]]) {
+          if (cls[v] < 0) {
+            cls[v] = 1 - cls[q[h]];
+            q.push_back(v);
+          } else if (cls[v] == cls[q[h]]) {
+            two = false;  // an odd cycle: no embedding, but the plan runs as any other
+          }
+        }
+    }
+    std::vector<int> place(MAXW, -1), nc(S + 1, 0);
+    std::vector<int> held;  // columns that hold a place in the tile of step j
+    auto place_new = [&](int j, int first, int n) {  // columns first .. first + n - 1 enter tile j
+      std::vector<char> used(4 * dmk::CH_CHUNKS, 0);
+      std::vector<int> keep;
+      for (int col : held)
+        if (need[j][col]) {
+          keep.push_back(col);
+          used[place[col]] = 1;
+        }
+      for (int col = first; col < first + n; col++) {
+        if (!need[j][col]) continue;
+        int h = 0;
+        while (h < (int)used.size() && (used[h] || (two && ((h >> 2) & 1) != cls[p->col_vertex[col]]))) h++;
+        if (h == (int)used.size()) return false;
+        place[col] = h;
+        used[h] = 1;
+        keep.push_back(col);
+      }
+      held = keep;
+      for (int col : held) nc[j] = std::max(nc[j], (place[col] >> 2) + 1);
+      if (two) nc[j] = (nc[j] + 1) / 2 * 2;
+      return true;
+    };
+    // place[] of a column is final when it enters, so a step's offsets can be taken afterwards; a
+    // column's place is free for the new vertices of the step that reads it last
+    std::vector<std::vector<int>> at(S + 1);  // tile j: place of each column, -1 if not held
+    for (int j = 1; j <= S; j++) {
+      const StepSpec &s = p->steps[j - 1];
+      if (!place_new(j, s.w_in, s.n_new)) return false;
+      at[j].assign(MAXW, -1);
+      for (int col : held) at[j][col] = place[col];
+    }
+    auto off = [](int h) { return (uint16_t)((h >> 2) * 512 + (h & 3) * 2); };
+
+    // launches: a deep stack of tiles leaves an SM few warps, a cut costs a launch and a table that is
+    // written and read; the cheapest cuts by the estimated rows
+    const int last_tile = count_mode ? S - 1 : S;
+    auto bytes = [&](int a, int b) {  // tiles a .. b (tile b is the output tile unless the launch counts)
+      int t = 0;
+      for (int j = a; j <= b; j++) t += dmk::chain_tile_bytes(nc[j]);
+      return t;
+    };
+    const std::vector<double> rows = chain_rows();
+    std::vector<double> cost(S + 1, 1e300);  // steps 1 .. j done, tile j + 1 written
+    std::vector<int> from(S + 1, -1);
+    cost[0] = 0;
+    for (int j = 1; j < S; j++) {
+      double work = 0;
+      for (int i = j - 1; i >= 0; i--) {  // one launch of steps i + 1 .. j
+        const bool end = j == S - 1;
+        const int need_smem = bytes(i + 1, end ? last_tile : j + 1) * dmk::CH_CTA_WARPS;
+        work += rows[i + 1];
+        if (j - i > dmk::CH_STEPS || need_smem > dmk::CH_SMEM_MAX) break;
+        const double warps = std::min(CHAIN_WARPS, CHAIN_SM_BYTES / need_smem * dmk::CH_CTA_WARPS);
+        const double x = cost[i] + CHAIN_LAUNCH_NS + CHAIN_ROW_NS * work * CHAIN_WARPS / warps +
+                         (end ? 0.0 : CHAIN_BYTE_NS * 16.0 * (nc[j + 1] + 1) * rows[j]);
+        if (x < cost[j]) {
+          cost[j] = x;
+          from[j] = i;
+        }
+      }
+    }
+    if (cost[S - 1] >= 1e300) return false;
+    std::vector<int> cuts;
+    for (int j = S - 1; j > 0; j = from[j]) cuts.push_back(j);
+    std::reverse(cuts.begin(), cuts.end());
+
+    std::vector<int> opos(MAXW, 0);  // working column -> output position
+    const JoinArgs &la = st[S - 1].base, &a0 = st[0].base;
+    for (int q = 0; q < la.wo; q++) opos[la.src_col[q]] = q;
+    C.launch.assign(cuts.size(), dmk::ChainArgs());
+    C.ids.assign(S, 0);
+    C.extra.assign(S, 0);
+    memset(&C.tab, 0, sizeof(C.tab));
+    C.tab.mode = count_mode ? 1 : 0;
+    C.tab.qerr = a0.qerr;
+    for (size_t i = 0; i < cuts.size(); i++) {
+      dmk::ChainArgs &A = C.launch[i];
+      memset(&A, 0, sizeof(A));
+      const int first = i ? cuts[i - 1] : 0, last = cuts[i];  // steps first + 1 .. last
+      const bool end = i + 1 == cuts.size();
+      A.n_steps = last - first;
+      A.mode = count_mode ? 1 : 0;
+      A.two = two ? 1 : 0;
+      A.out_kind = !end ? 2 : count_mode ? 0 : 1;
+      A.wo = la.wo;
+      A.adj = g->adj;
+      A.adj_words = g->adj_words;
+      A.row_ptr = g->row_ptr;
+      A.col_idx = g->col_idx;
+      A.eerr = g->eerr;
+      A.qerr = a0.qerr;
+      A.scored = a0.scored;
+      A.limit = 1u << 20;  // a warp's candidates: about 2.5e9 a launch, tens of milliseconds
+      int o = 0;
+      std::vector<int> tile(last + 2, 0);
+      for (int j = first + 1; j <= (end ? last_tile : last + 1); j++) {
+        tile[j] = o;
+        o += dmk::chain_tile_bytes(nc[j]);
+      }
+      A.warp_bytes = (o + 15) / 16 * 16;
+      for (int j = first + 1; j <= last; j++) {
+        const StepSpec &s = p->steps[j];
+        const JoinArgs &a = st[j].base;
+        dmk::ChainStep &t = A.st[j - first];
+        const bool counted = end && count_mode && j == last;
+        t.offsets = a.ix.offsets;
+        t.slots = a.ix.slots;
+        t.log2cap = a.ix.log2cap;
+        t.in_off = (uint16_t)(tile[j] / 8);
+        t.out_off = counted ? 0 : (uint16_t)(tile[j + 1] / 8);
+        t.nkeys = (uint8_t)a.ix.nkeys;
+        t.n_new = (uint8_t)s.n_new;
+        t.n_chk = (uint8_t)(s.n_keys - a.ix.nkeys);
+        t.units = s.n_new + t.n_chk <= 4 ? 1 : 2;
+        t.nc_in = (uint8_t)nc[j];
+        t.nc_out = counted ? 0 : (uint8_t)nc[j + 1];
+        for (int x = 0; x < a.ix.nkeys; x++) t.key_off[x] = off(at[j][s.key_col[x]]);
+        for (int x = 0; x < t.n_chk; x++) t.chk_off[x] = off(at[j][s.key_col[a.ix.nkeys + x]]);
+        // one key and 1 or 3 new vertices (M2, M4): room for the longest group at every key, and of
+        // three new vertices two of one colour class first
+        std::vector<int> ord(s.n_new);
+        for (int x = 0; x < s.n_new; x++) ord[x] = x;
+        auto cl = [&](int x) { return two ? cls[s.slice[s.new_mpos[x]]] : 0; };
+        if (a.ix.nkeys == 1 && t.n_chk == 0 && !(counted && s.n_be) &&
+            (s.n_new == 3 || (s.n_new == 1 && st[j].max_group <= 4))) {
+          t.group = (int32_t)st[j].max_group;
+          for (int col : ex[j])
+            if (s.k == 2 && t.n_ex + 1 < t.group) t.ex_off[t.n_ex++] = off(at[j][col]);
+          if (s.n_new == 3 && cl(0) != cl(1)) std::swap(ord[cl(0) == cl(2) ? 1 : 0], ord[2]);
+          t.q = (uint8_t)cl(ord[0]);
+          t.same = s.n_new == 3 && cl(ord[2]) == cl(ord[0]);
+        }
+        std::vector<int> rank(s.n_new);  // new vertex -> its place in the record
+        for (int x = 0; x < s.n_new; x++) rank[ord[x]] = x;
+        t.n_be = (uint8_t)s.n_be;
+        for (int x = 0; x < s.n_be; x++)
+          for (int h = 0; h < 2; h++) {
+            const int col = s.be_col[x][h];
+            (h ? t.be_b : t.be_a)[x] = col < s.w_in ? off(at[j][col]) : (uint16_t)(0x8000 + rank[col - s.w_in]);
+          }
+        for (int x = 0; x < s.n_new; x++) {
+          const int v = ord[x];
+          for (int col : ck[j][v]) t.cm[x] |= (uint8_t)(1u << (at[j][col] >> 2));
+          const int h = counted ? -1 : at[j + 1][s.w_in + v];
+          t.new_off[x] = h >= 0 ? off(h) : dmk::CH_DEAD;
+        }
+        dmk::ChainTables::Tab r{};
+        r.rows = a.ix.rows;
+        r.score = a0.scored ? a.ix.score : nullptr;
+        r.offsets = a.ix.offsets;
+        r.mw = a.ix.mw;
+        r.n_new = s.n_new + t.n_chk;
+        r.units = t.units;
+        for (int x = 0; x < s.n_new; x++) {
+          r.mpos[x] = (uint8_t)s.new_mpos[ord[x]];
+          r.npos[x] = (uint8_t)(opos[s.w_in + ord[x]] + 1);
+        }
+        for (int x = 0; x < t.n_chk; x++) r.mpos[s.n_new + x] = (uint8_t)s.key_mpos[a.ix.nkeys + x];
+        auto add = [&](int kind, int64_t entries, int64_t bytes) {  // its place in the buffer, from 1
+          r.kind = kind;
+          dmk::ChainTables &R = C.tab;
+          if (kind == dmk::CH_TAB_ID || kind == dmk::CH_TAB_ID3)  // ids alone: steps may share them
+            for (int y = 0; y < C.n_tab; y++)
+              if (R.tab[y].kind == kind && R.tab[y].rows == r.rows && !memcmp(R.tab[y].mpos, r.mpos, sizeof(r.mpos)))
+                return C.tab_off[y] + 1;
+          if (C.n_tab == dmk::CH_TABS) return (int64_t)0;
+          R.total += entries;
+          r.end = R.total;
+          C.tab_off.push_back(C.tab_bytes);
+          C.tab_bytes += (bytes + 255) / 256 * 256;
+          R.tab[C.n_tab++] = r;
+          return C.tab_off.back() + 1;
+        };
+        if (t.group) {
+          const bool one = s.n_new == 1;
+          r.group = one ? 4 : (t.group + 3) / 4 * 4;
+          t.stride = one ? 1 : r.group;
+          const int64_t n = (int64_t)g->V * r.group;
+          C.ids[j] = add(one ? dmk::CH_TAB_ID : dmk::CH_TAB_ID3, n, n * (one ? 2 : 8));
+          if (!C.ids[j]) return false;
+          if (count_mode ? !one : a0.scored != 0) {
+            C.extra[j] = add(count_mode ? dmk::CH_TAB_SUM : dmk::CH_TAB_SCORE, n, n * (count_mode ? 8 : 4));
+            if (!C.extra[j]) return false;
+          }
+          const uint64_t pos = (uint64_t)opos[s.w_in] + 1;
+          t.mul = (pos << 32) * 0xBF58476D1CE4E5B9ull;
+          t.pos2 = (uint32_t)(pos << 2);
+        } else {
+          C.extra[j] = add(dmk::CH_TAB_REC, a.ix.n, a.ix.n * 16 * t.units);
+          if (!C.extra[j]) return false;
+        }
+        if (counted && t.group) A.count_new = s.n_new;
+      }
+      if (i == 0) {
+        A.seed_rows = a0.ix.rows;
+        A.seed_score = a0.ix.score;
+        A.seed_mw = a0.ix.mw;
+        A.seed_k = s0.n_new;
+        A.seed_nbe = s0.n_be;
+        for (int x = 0; x < s0.n_be; x++)
+          for (int h = 0; h < 2; h++) A.seed_be[x][h] = (uint8_t)s0.be_col[x][h];
+        A.shard = shard;
+        A.n_shards = n_shards;
+        for (int x = 0; x < s0.n_new; x++) {
+          A.seed_off[x] = at[1][x] >= 0 ? off(at[1][x]) : dmk::CH_DEAD;
+          A.seed_npos[x] = (uint8_t)(opos[x] + 1);
+        }
+      }
+      if (end && !count_mode)
+        for (int q = 0; q < la.wo; q++) A.out_off[q] = off(at[S][la.src_col[q]]);
+    }
+    C.needs_arena = C.launch.size() > 1 || !count_mode;
+    return C.tab_bytes <= CHAIN_TAB_BYTES;
+  }
+
+  int ensure_tables(int64_t bytes) {
+    if (c->tab_bytes >= bytes) return DM_OK;
+    dfree(c, c->tabs);  // in stream order: behind what still reads it
+    c->tabs = nullptr;
+    c->tab_bytes = 0;
+    RET(dalloc(c, &c->tabs, (size_t)bytes));
+    c->tab_bytes = bytes;
+    return DM_OK;
+  }
+
+  // Run the launches of a laid-out plan. A launch is bounded in work: what it leaves of its input
+  // is taken up by another round of launches. *fits is false when a table or the rows overflow the
+  // arena (nothing is delivered then).
+  int run_chain(Chain &C, bool *fits) {
+    const int S = (int)st.size();
+    *fits = false;
+    const int64_t n0 = st[0].seed_table->n;
+    unsigned char *tabs = (unsigned char *)c->tabs;
+    for (int y = 0; y < C.n_tab; y++) C.tab.tab[y].out = tabs + C.tab_off[y];
+    C.tab.ctr = c->d_ctr_steps;
+    C.tab.n_ctr = (int64_t)CTR_N * S;
+    const size_t half = C.launch.size() > 1 ? (c->arena_bytes / 2) / 256 * 256 : c->arena_bytes;
+    int ends = 0;  // plan steps up to the launch
+    std::vector<int> grid(C.launch.size());
+    for (size_t i = 0; i < C.launch.size(); i++) {
+      dmk::ChainArgs &A = C.launch[i];
+      grid[i] = dmk::chain_grid(A, c->num_sms);
+      const int before = ends;
+      for (int l = 1; l <= A.n_steps; l++) {
+        dmk::ChainStep &t = A.st[l];
+        const int j = before + l;
+        t.ids = C.ids[j] ? (const uint2 *)(tabs + C.ids[j] - 1) : nullptr;
+        t.extra = C.extra[j] ? tabs + C.extra[j] - 1 : nullptr;
+        t.rec = (const uint4 *)t.extra;
+      }
+      ends += A.n_steps;
+      A.ctr_last = c->d_ctr_steps + (size_t)ends * CTR_N;
+      A.prune = prune;
+      unsigned char *buf = C.needs_arena ? c->arena + (i & 1) * half : nullptr;
+      if (A.out_kind == 1) {
+        const int64_t rb = 4ll * A.wo + (A.scored ? 4 : 0);
+        A.out_cap = std::max<int64_t>(1, ((int64_t)half - 512) / rb);
+        A.out = (int32_t *)buf;
+        A.outs = A.scored ? (float *)(buf + ((size_t)A.out_cap * A.wo * 4 + 255) / 256 * 256) : nullptr;
+      } else if (A.out_kind == 2) {
+        const int64_t bb = (A.st[A.n_steps].nc_out + 1) * 256;
+        A.out_cap = std::max<int64_t>(1, ((int64_t)half - 512) / (bb + 4));
+        A.out = (int32_t *)buf;
+        A.out_rows = (int32_t *)(buf + A.out_cap * bb);
+      }
+      if (i) {
+        const dmk::ChainArgs &P = C.launch[i - 1];
+        A.in = (const unsigned char *)P.out;
+        A.in_rows = P.out_rows;
+        A.in_blocks = c->d_ctr_steps + (size_t)before * CTR_N + CTR_BLOCKS;
+        A.in_cap = P.out_cap;
+      }
+    }
+    dmk::ChainArgs &F = C.launch[0];
+    // a few items a warp, so that dealing them out evens the warps' loads
+    F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, n0 / (8ll * grid[0] * dmk::CH_CTA_WARPS)));
+    F.seed_n = n0;
+    float ms = 0.f;
+    int64_t run_steps = 0;
+    for (bool more = true, first = true; more; first = false) {
+      if (c->timing) CK(cudaEventRecord(c->ev0, c->stream));
+      if (first) CK(dmk::launch_chain_tables(C.tab, c->stream));
+      std::vector<int> blocks(grid);
+      for (size_t i = 0; i < C.launch.size(); i++) {
+        dmk::ChainArgs &A = C.launch[i];
+        if (!A.in) {
+          const int64_t items = (n0 - A.lo + A.chunk - 1) / A.chunk;
+          blocks[i] = (int)std::min<int64_t>(grid[i], (items + dmk::CH_CTA_WARPS - 1) / dmk::CH_CTA_WARPS);
+          if (blocks[i] == 0) continue;  // the first table is used up
+        }
+        if (!first) CK(cudaMemsetAsync(A.ctr_last + CTR_ITEM, 0, sizeof(unsigned long long), c->stream));
+        CK(dmk::launch_chain(A, blocks[i], c->stream));
+        run_steps += A.n_steps + (A.in ? 0 : 1);
+      }
+      if (c->timing) CK(cudaEventRecord(c->ev1, c->stream));
+      CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * S,
+                         cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+      if (c->timing) {
+        float t = 0.f;
+        CK(cudaEventElapsedTime(&t, c->ev0, c->ev1));
+        ms += t;
+      }
+      for (int j = 0; j < S; j++)
+        if (c->h_ctr_steps[(size_t)j * CTR_N + CTR_OVF]) return DM_OK;
+      more = false;
+      for (size_t i = 0; i < C.launch.size(); i++) {  // every warp's first item and those the counter gave out are done
+        dmk::ChainArgs &A = C.launch[i];
+        const unsigned long long *h = c->h_ctr_steps + (A.ctr_last - c->d_ctr_steps);
+        const int64_t n_in = A.in ? (int64_t)c->h_ctr_steps[A.in_blocks - c->d_ctr_steps] : n0;
+        // (a table of few blocks is always joined to its end)
+        const int64_t warps = (int64_t)blocks[i] * dmk::CH_CTA_WARPS;
+        const int64_t done = A.in && n_in - A.lo < 8 * warps ? n_in : warps + (blocks[i] ? (int64_t)h[CTR_ITEM] : 0);
+        A.lo = std::min<int64_t>(n_in, A.lo + done * (A.in ? 1 : A.chunk));
+        more |= A.lo < n_in;
+      }
+    }
+    *fits = true;
+    c->stats.join_ms += ms;
+    c->stats.join_launches += run_steps;
+    c->stats.chunks += run_steps;
+    for (int j = 0; j < S; j++) {
+      const unsigned long long *h = c->h_ctr_steps + (size_t)j * CTR_N;
+      c->stats.join_bytes += (double)st[j].motif_bytes;
+      c->stats.rows[j] += (int64_t)h[CTR_ROWS];
+      c->stats.candidates[j] += (int64_t)h[CTR_CAND];
+      if (j + 1 < S) c->stats.max_rows = std::max(c->stats.max_rows, (int64_t)h[CTR_ROWS]);
+    }
+    ends = 0;
+    for (auto &A : C.launch) {  // tables between launches: written once, read once
+      ends += A.n_steps;
+      if (A.out_kind == 2)
+        c->stats.join_bytes += 2.0 * 8.0 * (A.st[A.n_steps].nc_out + 1) * (double)c->h_ctr_steps[(size_t)ends * CTR_N + CTR_ROWS];
+    }
+    const unsigned long long *hl = c->h_ctr_steps + (size_t)(S - 1) * CTR_N;
+    if (mode == DM_COUNT) {
+      count += hl[CTR_ROWS];
+      checksum += hl[CTR_SUM];
+      return DM_OK;
+    }
+    const dmk::ChainArgs &A = C.launch.back();
+    c->stats.join_bytes += (double)hl[CTR_ROWS] * (4.0 * A.wo + (A.scored ? 4 : 0));
+    DevTable t;
+    t.rows = A.out;
+    t.score = A.outs;
+    t.n = (int64_t)hl[CTR_ROWS];
+    t.w = A.wo;
+    t.borrowed = true;
+    return sink->take(c, t);
+  }
+
   int ensure_arena(size_t bytes) {
     if (c->arena_bytes >= bytes) return DM_OK;
     if (c->arena) {
@@ -894,14 +1435,21 @@ struct Exec {
     const int S = (int)st.size();
     c->stats.n_steps = S;
     if (chunk_rows == 0 && max_rows == 0 && p->join_algo != DM_JOIN_SORTMERGE && st[0].seed_table->n > 0) {
-      // device-driven path first; grow the arena (up to the budget) while a step overflows
+      // launches of several steps where the plan allows it (a count in one launch needs no
+      // arena), else a launch a step; grow the arena (up to the budget) while a step overflows
+      Chain C;
+      const bool chain = chain_layout(C) && ensure_tables(C.tab_bytes) == DM_OK;
+      if (chain && !C.needs_arena) {
+        bool fits = false;
+        return run_chain(C, &fits);
+      }
       size_t want = std::max<size_t>(c->arena_bytes, (size_t)4 << 30);
       while (true) {
         want = std::min<size_t>(want, (size_t)c->budget);
         if (ensure_arena(want) != DM_OK) break;
         bool fits = false;
         dm_stats saved = c->stats;
-        RET(run_fast(&fits));
+        RET(chain ? run_chain(C, &fits) : run_fast(&fits));
         if (fits) return DM_OK;
         c->stats = saved;
         if (want >= (size_t)c->budget) break;
@@ -1906,6 +2454,7 @@ int dm_destroy(dm_ctx *c) {
   if (c->d_ctr_steps) cudaFree(c->d_ctr_steps);
   if (c->h_ctr_steps) cudaFreeHost(c->h_ctr_steps);
   if (c->arena) cudaFree(c->arena);
+  dfree(c, c->tabs);
   cudaFree(c->m_params);
   cudaFree(c->m_grads);
   cudaFree(c->m_m);
@@ -1956,6 +2505,9 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
   for (int32_t u = 0; u < n; u++) md = std::max(md, h.rp[u + 1] - h.rp[u]);
   g->max_deg = md;
   g->avg_deg = (double)g->nnz / n;
+  double deg2 = 0;
+  for (int32_t u = 0; u < n; u++) deg2 += (double)(h.rp[u + 1] - h.rp[u]) * (h.rp[u + 1] - h.rp[u]);
+  g->edge_deg = g->nnz ? deg2 / (double)g->nnz : 0.0;
   g->nonneg_weights = nonneg;
   auto up = [&](void **dst, const void *src, size_t bytes) -> int {
     if (cudaMalloc(dst, std::max<size_t>(bytes, 16)) != cudaSuccess) return DM_E_NOMEM;
@@ -1978,7 +2530,17 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
     else if (dmk::launch_bitmap(g->row_ptr, g->col_idx, n, g->nnz, g->adj_words, g->adj, c->stream) != cudaSuccess)
       r = DM_E_CUDA;
   }
+  if (r == DM_OK) {  // the girth, through a counter slot that no other work of the context uses now
+    int32_t *d = (int32_t *)c->d_ctr, *h_girth = (int32_t *)c->h_ctr;
+    *h_girth = dmk::GIRTH_MAX;
+    if (cudaMemcpyAsync(d, h_girth, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+        dmk::launch_girth(g->row_ptr, g->col_idx, n, d, c->stream) != cudaSuccess ||
+        cudaMemcpyAsync(h_girth, d, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
+      r = DM_E_CUDA;
+    g->bipartite = two_colourable(h, n);
+  }
   if (r == DM_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) r = DM_E_CUDA;
+  if (r == DM_OK) g->girth = *(int32_t *)c->h_ctr;
   if (r == DM_OK) r = ensure_motif(c, g, 2);
   if (r != DM_OK) {  // a graph that failed to load is neither registered nor kept
     cudaGetLastError();

@@ -130,7 +130,7 @@ struct IndexView {
                                    // offsets and slots are unused)
 };
 
-enum { CTR_ROWS = 0, CTR_NEXT = 1, CTR_SUM = 2, CTR_OVF = 3, CTR_CAND = 4, CTR_N = 8 };
+enum { CTR_ROWS = 0, CTR_NEXT = 1, CTR_SUM = 2, CTR_OVF = 3, CTR_CAND = 4, CTR_ITEM = 5, CTR_BLOCKS = 6, CTR_N = 8 };
 
 struct JoinArgs {
   // input table R (row-major, width w); R == nullptr with w == 0 seeds from the motif table

@@ -79,6 +79,53 @@ cudaError_t launch_bitmap(const int32_t *row_ptr, const int32_t *col_idx, int32_
   return cudaGetLastError();
 }
 
+// One thread a vertex v: breadth-first search from v, which meets an edge between two visited vertices
+// first on a cycle no longer than the shortest one through v allows: after the vertices at depth d - 1
+// have been expanded, every cycle through v of at most 2 d edges has been seen, and the smallest length
+// met over all v is the girth. A thread whose search outgrows GIRTH_LIST vertices reports what it has
+// seen in full, plus one: the result never exceeds the girth (up to GIRTH_MAX, which stands for "at
+// least that"). On lattices a search ends within 40 vertices.
+constexpr int GIRTH_LIST = 96;
+__global__ void k_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth) {
+  const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= V) return;
+  int32_t list[GIRTH_LIST];
+  uint8_t from[GIRTH_LIST], depth[GIRTH_LIST];  // place of the vertex it was found from, distance from v
+  list[0] = v;
+  from[0] = depth[0] = 0;
+  int n = 1, best = GIRTH_MAX;
+  for (int h = 0; h < n; h++) {
+    const int d = depth[h];
+    // what is left to see has at least 2 d + 1 edges
+    if (2 * d + 1 >= best || (h && depth[h - 1] != d && *(volatile int32_t *)girth <= 2 * d + 1)) break;
+    const int32_t u = list[h], parent = list[from[h]];
+    for (int32_t k = __ldg(row_ptr + u); k < __ldg(row_ptr + u + 1); k++) {
+      const int32_t w = __ldg(col_idx + k);
+      if (w == parent && h) continue;
+      int at = 0;
+      while (at < n && list[at] != w) at++;
+      if (at < n) {
+        best = min(best, d + depth[at] + 1);
+      } else if (n < GIRTH_LIST) {
+        list[n] = w;
+        from[n] = (uint8_t)h;
+        depth[n++] = (uint8_t)(d + 1);
+      } else {
+        atomicMin(girth, min(best, 2 * d + 1));
+        return;
+      }
+    }
+  }
+  if (best < GIRTH_MAX) atomicMin(girth, best);
+}
+
+cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth, cudaStream_t s) {
+  if (V <= 0) return cudaSuccess;
+  g_launches++;
+  k_girth<<<(V + 127) / 128, 128, 0, s>>>(row_ptr, col_idx, V, girth);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ scan ---------------
 static_assert(SCAN_TILE == SCAN_BLK * SCAN_ITEMS, "scan tile");
 

@@ -53,9 +53,102 @@ int wjoin_grid(const dmi::JoinArgs &a, int num_sms);
 bool fused_ok(const dmi::JoinArgs &a, const dmi::JoinArgs &b);
 cudaError_t launch_fused(const dmi::JoinArgs &a, const dmi::JoinArgs &b, int num_sms, cudaStream_t s, bool pdl);
 
+// Several steps of a plan, often all of them, in one launch (chain.cu).
+constexpr int CH_STEPS = 24;          // steps of a launch besides the seed, at most
+constexpr int CH_NEW = 8;             // new vertices and further keys of a step, at most
+constexpr int CH_CHUNKS = 8;          // chunks of four ids in a row, at most
+constexpr uint16_t CH_DEAD = 0xFFFF;  // a new vertex that no later step reads
+constexpr int CH_SMEM_MAX = 220 * 1024;
+constexpr int CH_CTA_WARPS = 4;
+constexpr int CH_MAX_GROUP = 255;     // longest key group, and rows of a motif table: what the
+constexpr int64_t CH_MAX_ROWS = (1 << 24) - 1;  // state of an interrupted step holds
+// A warp's tile of 64 rows of nc chunks: checksum sums or scores, state of an interrupted step, rows.
+constexpr int chain_tile_bytes(int nc) { return 64 * 8 + 32 * 4 + nc * 512; }
+struct ChainStep {
+  // steps of grouped candidates (one key, 1 or 3 new vertices; group > 0: candidates of a key, at
+  // most): the ids, `stride` words of 8 bytes a key, and what else a candidate brings (three new
+  // vertices: sum of the checksum terms; scored rows: part of the score)
+  const uint2 *ids;
+  const void *extra;
+  unsigned long long mul;        // one new vertex: its checksum term's constants (ch_term)
+  uint32_t pos2;
+  int32_t group, stride;
+  uint8_t n_ex;                  // one new vertex: columns that are the key's pattern neighbours
+  uint16_t ex_off[2];
+  uint8_t q, same;               // colour class of new vertices 0 and 1, and whether 2 is of it too
+  // any other step: one record a motif row in index order
+  uint8_t units;
+  uint8_t nkeys, n_new, n_chk, n_be, nc_in, nc_out;
+  uint8_t cm[CH_NEW];            // chunks new vertex i is compared with
+  const uint4 *rec;
+  const int32_t *offsets;        // nkeys == 1
+  const dmi::HashSlot *slots;    // nkeys == 2
+  uint32_t log2cap;
+  uint16_t in_off, out_off;      // its tile and the next one, in 8-byte words of the warp's memory
+  uint16_t key_off[2], chk_off[4], new_off[CH_NEW];  // byte offsets from a row's first chunk
+  uint16_t be_a[8], be_b[8];     // byte offset, or 0x8000 + index of the new vertex
+};
+struct ChainArgs {
+  ChainStep st[CH_STEPS + 1];    // 1 .. n_steps; st[0] is the seed or the input table
+  int32_t n_steps, mode, wo, warp_bytes;
+  int32_t two;                   // two colour classes: chunk 2 k + class
+  int32_t count_new;             // 1 or 3: new vertices of a counted last step that ch_count takes, else 0
+  int32_t out_kind;              // 0: count and checksum, 1: packed rows, 2: table for another launch
+  const unsigned long long *adj;
+  int32_t adj_words;
+  const int32_t *row_ptr, *col_idx;
+  const float *eerr, *qerr;
+  int32_t scored;
+  float prune;
+  const int32_t *seed_rows;
+  const float *seed_score;
+  int32_t seed_mw, seed_k, seed_nbe, shard, n_shards;
+  int64_t seed_n, chunk;         // chunk <= 32 rows of the first table are one work item
+  int64_t lo;                    // input already joined by earlier launches: rows of the first table, or blocks
+  uint8_t seed_npos[dmi::MAXM], seed_be[8][2];
+  uint16_t seed_off[dmi::MAXM];
+  const unsigned char *in;       // instead of the seed: blocks of up to 32 rows, in_rows[b] rows in block b
+  const int32_t *in_rows;
+  const unsigned long long *in_blocks;
+  int64_t in_cap;
+  unsigned limit;                // candidates after which a warp takes no further items
+  unsigned long long *ctr_last;  // CTR_N counters of the launch's last step, behind those of its others
+  int32_t *out;                  // packed rows in pattern-vertex order, or blocks
+  float *outs;
+  int32_t *out_rows;
+  int64_t out_cap;               // rows, or blocks
+  uint16_t out_off[dmi::MAXW];   // output position -> byte offset in the last tile's rows
+};
+int chain_grid(const ChainArgs &a, int num_sms);  // blocks of a full launch
+cudaError_t launch_chain(const ChainArgs &a, int grid, cudaStream_t s);
+// What the candidates of a plan's steps bring, and n_ctr zeroed counters. Kinds of tables: records (per
+// motif row, `units` of 16 bytes), and per place of a grouped step an id, three ids and the group's
+// length, the sum of checksum terms, the part of the score.
+enum { CH_TAB_REC = 0, CH_TAB_ID = 1, CH_TAB_ID3 = 2, CH_TAB_SUM = 3, CH_TAB_SCORE = 4 };
+constexpr int CH_TABS = 96;
+struct ChainTables {
+  struct Tab {
+    const int32_t *rows;
+    const float *score;
+    const int32_t *offsets;
+    void *out;
+    int64_t end;                 // entries of the tables up to this one
+    int32_t kind, group, mw, n_new, units;
+    uint8_t mpos[CH_NEW], npos[CH_NEW];  // npos: 1 + output position (0: a further key, not a new vertex)
+  } tab[CH_TABS];
+  int64_t total, n_ctr;
+  unsigned long long *ctr;
+  const float *qerr;
+  int32_t mode;
+};
+cudaError_t launch_chain_tables(const ChainTables &r, cudaStream_t s);
+
 // Data-graph preparation.
 cudaError_t launch_csr_to_m2(const int32_t *row_ptr, const int32_t *col_idx, const float *eerr,
                              int32_t V, int64_t nnz, int32_t *rows, float *score, cudaStream_t s);
+// *girth = min(*girth, a lower bound of the graph's girth); the caller sets it to GIRTH_MAX before.
+constexpr int GIRTH_MAX = 32;
+cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth, cudaStream_t s);
 cudaError_t launch_vertex_table(int32_t V, int32_t *rows, float *score, cudaStream_t s);
 cudaError_t launch_bitmap(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int64_t nnz,
                           int32_t words, unsigned long long *adj, cudaStream_t s);

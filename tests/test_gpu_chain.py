@@ -1,0 +1,106 @@
+"""Plans that run several steps a launch (chain.cu) against the oracle: graphs that decide which pairs
+of vertices are compared (girth, odd cycles), groups of every size the records take, tiles that fill
+and drain at every remainder, and the edge of 16-bit ids. Counts, checksums and rows are exact."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2508_21287_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2508_21287_gb300 import build
+    build.build()
+    from paper_2508_21287_gb300 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.Context(0)
+    yield c
+    c.close()
+
+
+def strip(n):
+    """Triangles in a row: odd cycles, girth 3."""
+    return I.from_edges(n, [(i, i + 1) for i in range(n - 1)] + [(i, i + 2) for i in range(n - 2)])
+
+
+def bipartite(a, b):
+    return I.from_edges(a + b, [(i, a + j) for i in range(a) for j in range(b)])
+
+
+def torus(a, b):
+    return I.from_edges(a * b, sorted({tuple(sorted((r * b + c, q))) for r in range(a) for c in range(b)
+                                       for q in (((r + 1) % a) * b + c, r * b + (c + 1) % b)}))
+
+
+def caterpillar(n):
+    """A path with 0, 1 or 2 leaves a vertex: groups of uneven size, no cycle."""
+    e, k = [(i, i + 1) for i in range(n - 1)], n
+    for i in range(n):
+        for _ in range(i % 3):
+            e.append((i, k))
+            k += 1
+    return I.from_edges(k, e)
+
+
+GRAPHS = {
+    "strip": (strip(37), [4, 7, 9]),
+    "k7": (I.complete(7), [3, 5, 7]),
+    "k33": (bipartite(3, 3), [4, 6]),
+    "k45": (bipartite(4, 5), [5, 7]),
+    "torus5x7": (torus(5, 7), [6, 9]),
+    "torus6x6": (torus(6, 6), [6, 9]),
+    "ring13": (I.cycle(13), [5, 12, 13]),
+    "ring12": (I.cycle(12), [5, 11, 12]),
+    "caterpillar": (caterpillar(23), [6, 11]),
+    "heavyhex": (I.heavy_hex(2, 3), [13, 18]),
+    "rr3": (I.random_regular3(64, 3), [7, 10]),
+}
+
+
+@pytest.mark.parametrize("name", sorted(GRAPHS))
+def test_every_form_equals_the_oracle(ctx, B, name):
+    g, lens = GRAPHS[name]
+    g = I.lognormal_weights(g, 5, qubits=True)
+    gid = ctx.load(g)
+    pats = [I.path(k) for k in lens] + [I.star(3), I.cycle(4), I.cycle(6), I.random_tree(8, 2), I.random_tree(9, 7)]
+    for p in pats:
+        if p.n > g.n:
+            continue
+        ref = oracle.enumerate(g, p, threads=8)
+        want = oracle.scores(g, p, ref.rows)
+        for motifs in (None, [2], [4, 2], [104, 2]):
+            plan = ctx.plan(gid, p, motifs=motifs)
+            assert plan.count() == (ref.count, ref.checksum), (name, p.name, motifs)
+            shards = [B.dm_match_shard(ctx.h, plan.h, i, 3) for i in range(3)]
+            assert sum(c for c, _ in shards) == ref.count and sum(s for _, s in shards) % 2 ** 64 == ref.checksum
+            rows, scores, cnt, cs = plan.all()
+            assert (cnt, cs) == (ref.count, ref.checksum) and np.array_equal(rows, ref.rows), (name, p.name, motifs)
+            # at most 16 FP32 additions of non-negative terms: relative error below 17 * 2^-24 ~ 1e-6
+            if ref.count:
+                np.testing.assert_allclose(scores, want, rtol=2e-6, atol=0)
+            # the general form (a launch a step, sorted keys) sees the same rows step by step
+            stats = ctx.stats()
+            ctx.plan(gid, p, motifs=motifs, join_algo=B.DM_JOIN_SORTMERGE).all()
+            other = ctx.stats()
+            assert stats["rows"] == other["rows"] and stats["candidates"] == other["candidates"], (name, p.name, motifs)
+
+
+@pytest.mark.parametrize("n", [65533, 65534, 65535])
+def test_edge_of_16_bit_ids(ctx, n):
+    # a path: 2 (n - k + 1) embeddings of the path of k vertices; ids up to n - 1
+    gid = ctx.load(I.path(n))
+    for k in (3, 7, 12):
+        plan = ctx.plan(gid, I.path(k))
+        count, checksum = plan.count()
+        rows, _, cnt, cs = plan.all()
+        assert count == cnt == 2 * (n - k + 1) and checksum == cs
+        first = np.arange(n - k + 1)[:, None] + np.arange(k)
+        want = np.concatenate([first, first[:, ::-1]])
+        assert np.array_equal(rows, want[np.lexsort(want.T[::-1])])
