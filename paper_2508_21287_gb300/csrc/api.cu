@@ -88,6 +88,9 @@ struct dm_ctx {
   // arena of the device-driven path: two halves alternate as the input and output of a step
   unsigned char *arena = nullptr;
   size_t arena_bytes = 0;
+  void *sel_work = nullptr, *sel_out = nullptr;  // top-k selection (select.cu)
+  size_t sel_out_bytes = 0;
+  bool sel_dirty = false;  // its histogram holds counts that no selection has cleared
   void *tabs = nullptr;  // candidate tables of the plan that runs (chain.cu)
   int64_t tab_bytes = 0;
   unsigned long long *d_ctr_steps = nullptr;  // CTR_N counters per step
@@ -460,6 +463,14 @@ struct Sink {
   virtual ~Sink() {}
   // Takes ownership of a table of final rows (pattern-vertex order, unsorted).
   virtual int take(dm_ctx *c, DevTable t) = 0;
+  // Called before the stream is waited for, for a table that will be the only one if it fits: t.n is
+  // the most rows it can have, *n_dev receives how many it has. Work enqueued here is void when the
+  // table turns out not to fit; otherwise take() follows.
+  virtual int ahead(dm_ctx *, const DevTable &, const unsigned long long *) { return DM_OK; }
+  virtual void forget() {}  // the table did not fit, or others follow it
+  // k > 0: only the k best rows are wanted, and rows whose partial score is above the k-th best of those
+  // seen may be dropped; hist receives where the joins count the scores of what they write
+  virtual int64_t best_only(dm_ctx *, dmk::SelHist **) { return 0; }
 };
 
 struct StepRT {
@@ -1337,7 +1348,25 @@ struct Exec {
       }
     }
     dmk::ChainArgs &F = C.launch[0];
-    // a few items a warp, so that dealing them out evens the warps' loads
+    // a few items a warp, so that dealing them out evens the warps' loads; where there are not even as
+    // many rows as warps, several warps share a row's first candidates
+    const int64_t warps0 = (int64_t)grid[0] * dmk::CH_CTA_WARPS;
+    F.parts = F.n_steps < 2 || 2 * n0 > warps0 ? 1 : (int32_t)std::min<int64_t>(4, warps0 / n0);
+    for (auto &A : C.launch) {
+      A.sel = nullptr;
+      A.sel_k = 0;
+      A.parts = std::max(1, A.parts);
+    }
+    if (mode == DM_ALL && sink) {
+      dmk::SelHist *h = nullptr;
+      const int64_t k = sink->best_only(c, &h);
+      if (k < 0) return (int)k;
+      if (k > 0)
+        for (auto &A : C.launch) {
+          A.sel = h;
+          A.sel_k = (int32_t)k;
+        }
+    }
     F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, n0 / (8ll * grid[0] * dmk::CH_CTA_WARPS)));
     F.seed_n = n0;
     float ms = 0.f;
@@ -1349,7 +1378,7 @@ struct Exec {
       for (size_t i = 0; i < C.launch.size(); i++) {
         dmk::ChainArgs &A = C.launch[i];
         if (!A.in) {
-          const int64_t items = (n0 - A.lo + A.chunk - 1) / A.chunk;
+          const int64_t items = (n0 - A.lo + A.chunk - 1) / A.chunk * A.parts;
           blocks[i] = (int)std::min<int64_t>(grid[i], (items + dmk::CH_CTA_WARPS - 1) / dmk::CH_CTA_WARPS);
           if (blocks[i] == 0) continue;  // the first table is used up
         }
@@ -1358,6 +1387,14 @@ struct Exec {
         run_steps += A.n_steps + (A.in ? 0 : 1);
       }
       if (c->timing) CK(cudaEventRecord(c->ev1, c->stream));
+      if (first && mode == DM_ALL) {
+        DevTable t;
+        t.rows = C.launch.back().out;
+        t.score = C.launch.back().outs;
+        t.n = C.launch.back().out_cap;
+        t.w = C.launch.back().wo;
+        RET(sink->ahead(c, t, C.launch.back().ctr_last + CTR_ROWS));
+      }
       CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * S,
                          cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
@@ -1367,7 +1404,10 @@ struct Exec {
         ms += t;
       }
       for (int j = 0; j < S; j++)
-        if (c->h_ctr_steps[(size_t)j * CTR_N + CTR_OVF]) return DM_OK;
+        if (c->h_ctr_steps[(size_t)j * CTR_N + CTR_OVF]) {
+          if (sink) sink->forget();
+          return DM_OK;
+        }
       more = false;
       for (size_t i = 0; i < C.launch.size(); i++) {  // every warp's first item and those the counter gave out are done
         dmk::ChainArgs &A = C.launch[i];
@@ -1376,9 +1416,11 @@ struct Exec {
         // (a table of few blocks is always joined to its end)
         const int64_t warps = (int64_t)blocks[i] * dmk::CH_CTA_WARPS;
         const int64_t done = A.in && n_in - A.lo < 8 * warps ? n_in : warps + (blocks[i] ? (int64_t)h[CTR_ITEM] : 0);
-        A.lo = std::min<int64_t>(n_in, A.lo + done * (A.in ? 1 : A.chunk));
+        A.lo = std::min<int64_t>(n_in, A.lo + (A.in ? done : done / A.parts * A.chunk));
         more |= A.lo < n_in;
       }
+      if (more && sink) sink->forget();
+      for (auto &A : C.launch) A.sel = nullptr;  // what was counted went with the first round's selection
     }
     *fits = true;
     c->stats.join_ms += ms;
@@ -1531,7 +1573,10 @@ int deliver(dm_ctx *c, const DevTable &t, int flags, dm_chunk_cb cb, void *user,
 struct TopkSink;
 int topk_take(dm_ctx *c, TopkSink *t, DevTable tab);
 bool topk_small_enough(const TopkSink *t);
-int topk_into_host(dm_ctx *c, TopkSink *t, const DevTable &sorted, int32_t *rows, float *scores, int64_t *n);
+int64_t topk_k(const TopkSink *t);
+int topk_enqueue(dm_ctx *c, int64_t k, const DevTable &t, const unsigned long long *n_dev, bool sorted,
+                 bool counted = false);
+bool topk_enqueued(dm_ctx *c, int64_t k, int64_t n, int32_t w, int32_t *rows, float *scores);
 
 struct AllSink : Sink {
   TopkSink *tap = nullptr;  // also feeds every final chunk to a top-k accumulator
@@ -1555,13 +1600,17 @@ struct AllSink : Sink {
     CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(unsigned long long) * CTR_N, c->stream));
     RET(sort_canonical(c, t, bits, c->d_ctr));
     const bool fast_topk = last && tap && final_rows && topk_small_enough(tap);
-    if (fast_topk) RET(topk_into_host(c, tap, t, final_rows, final_scores, &final_n));
+    const int64_t k = fast_topk ? topk_k(tap) : 0;
+    if (fast_topk && t.n > 0) RET(topk_enqueue(c, k, t, nullptr, true));
     RET(read_ctr(c));
-    final_done = fast_topk;
+    if (fast_topk) {
+      final_n = std::min(k, t.n);
+      final_done = t.n == 0 || topk_enqueued(c, k, t.n, t.w, final_rows, final_scores);
+    }
     count += (uint64_t)t.n;
     checksum += c->h_ctr[CTR_SUM];
     int r = deliver(c, t, flags, cb, user, true);
-    if (r == DM_OK && tap && !fast_topk) return topk_take(c, tap, t);  // the tap takes ownership
+    if (r == DM_OK && tap && !final_done) return topk_take(c, tap, t);  // the tap takes ownership
     free_table(c, t);
     return r;
   }
@@ -1648,27 +1697,79 @@ int topk_table(dm_ctx *c, DevGraph *g, const DevTable &t, int64_t k, DevTable *o
   return DM_OK;
 }
 
-// k best of a canonically sorted table (rows in pattern order + scores), in (score, row)
-// order; consumes t.
-int topk_of_sorted(dm_ctx *c, DevGraph *g, DevTable &t, int64_t k, DevTable *out) {
-  if (k > 1024) {  // large k: select by radix on the order-preserving score keys, then sort the candidates
-    RET(topk_table(c, g, t, k, out));
-    free_table(c, t);
-    return DM_OK;
+// The k best rows of t by (score, row), k <= SEL_K, enqueued with their copy to the head of the pinned
+// staging buffer (select.cu). The caller synchronises, then topk_enqueued hands them over.
+int select_work(dm_ctx *c) {
+  if (c->sel_work && !c->sel_dirty) return DM_OK;
+  if (!c->sel_work) RET(dalloc(c, &c->sel_work, (size_t)dmk::select_work_bytes()));
+  CK(cudaMemsetAsync(c->sel_work, 0, (size_t)dmk::select_work_bytes(), c->stream));
+  const int32_t none = dmk::SEL_NO_BOUND;
+  CK(cudaMemcpyAsync(&((dmk::SelHist *)c->sel_work)->bound, &none, sizeof(none), cudaMemcpyHostToDevice, c->stream));
+  c->sel_dirty = false;
+  return DM_OK;
+}
+
+int topk_enqueue(dm_ctx *c, int64_t k, const DevTable &t, const unsigned long long *n_dev, bool sorted,
+                 bool counted) {
+  const size_t bytes = (size_t)dmk::select_out_bytes(k, t.w);
+  if (!counted) RET(select_work(c));
+  if (c->sel_out_bytes < bytes) {
+    dfree(c, c->sel_out);
+    c->sel_out = nullptr;
+    c->sel_out_bytes = 0;
+    RET(dalloc(c, &c->sel_out, bytes));
+    c->sel_out_bytes = bytes;
   }
-  DevTable o;
-  o.w = t.w;
-  o.n = std::min<int64_t>(k, t.n);
-  RET(dalloc_t(c, &o.rows, (size_t)std::max<int64_t>(1, o.n) * t.w));
-  RET(dalloc_t(c, &o.score, std::max<int64_t>(1, o.n)));
-  if (o.n > 0) {
-    void *tmp = nullptr;
-    RET(dalloc(c, &tmp, (size_t)dmk::topk_tmp_bytes(t.n)));
-    CK(dmk::topk_sorted(t.rows, t.score, t.n, t.w, (int32_t)k, tmp, o.rows, o.score, c->stream));
-    dfree(c, tmp);
+  dmk::SelectArgs a{};
+  a.rows = t.rows;
+  a.sc = t.score;
+  a.n = t.n;
+  a.n_dev = n_dev;
+  a.w = t.w;
+  a.k = (int32_t)k;
+  a.sorted = sorted;
+  a.counted = counted;
+  a.work = c->sel_work;
+  a.out = (unsigned char *)c->sel_out;
+  CK(dmk::topk_select(a, c->num_sms, c->stream));
+  c->sel_dirty = false;  // it leaves the histogram zeroed
+  CK(cudaMemcpyAsync(c->h_stage, c->sel_out, bytes, cudaMemcpyDeviceToHost, c->stream));
+  return DM_OK;
+}
+
+// After topk_enqueue on a table of n rows and a synchronisation: the min(k, n) rows and scores (nullable)
+// into host buffers. False when the selection gave up (too many rows near the k-th score).
+bool topk_enqueued(dm_ctx *c, int64_t k, int64_t n, int32_t w, int32_t *rows, float *scores) {
+  const unsigned char *h = (const unsigned char *)c->h_stage;
+  if (*(const uint32_t *)h > (uint32_t)dmk::SEL_CAP) return false;
+  const size_t m = (size_t)std::min(k, n);
+  if (scores) memcpy(scores, h + 16, 4 * m);
+  memcpy(rows, h + 16 + 4 * k, 4 * m * w);
+  return true;
+}
+
+// k best of a table, canonically sorted or not, in (score, row) order; consumes t.
+int topk_of(dm_ctx *c, DevGraph *g, DevTable &t, int64_t k, bool sorted, DevTable *out) {
+  if (t.n > 0 && k <= dmk::SEL_K) {
+    RET(topk_enqueue(c, k, t, nullptr, sorted));
+    CK(cudaStreamSynchronize(c->stream));
+    if (*(const uint32_t *)c->h_stage <= (uint32_t)dmk::SEL_CAP) {
+      DevTable o;
+      o.w = t.w;
+      o.n = std::min<int64_t>(k, t.n);
+      RET(dalloc_t(c, &o.rows, (size_t)o.n * t.w));
+      RET(dalloc_t(c, &o.score, o.n));
+      const float *sc = (const float *)((const unsigned char *)c->sel_out + 16);
+      CK(cudaMemcpyAsync(o.score, sc, sizeof(float) * o.n, cudaMemcpyDeviceToDevice, c->stream));
+      CK(cudaMemcpyAsync(o.rows, sc + k, sizeof(int32_t) * o.n * t.w, cudaMemcpyDeviceToDevice, c->stream));
+      free_table(c, t);
+      *out = o;
+      return DM_OK;
+    }
   }
+  // large k, or scores that many rows share: select by radix on the score keys, sort the candidates
+  RET(topk_table(c, g, t, k, out));
   free_table(c, t);
-  *out = o;
   return DM_OK;
 }
 
@@ -1679,24 +1780,41 @@ struct TopkSink : Sink {
   DevTable best;              // current best min(k, seen) rows, (score, row) order
   bool have = false;
   float *prune_ptr = nullptr;
+  bool tried = false;         // the first table's selection is enqueued (ahead)
+  bool on_host = false;       // ... and its result is in the staging buffer: best stays empty
+  int ahead(dm_ctx *c, const DevTable &t, const unsigned long long *n_dev) override {
+    if (input_sorted || have || k > dmk::SEL_K || !t.score) return DM_OK;
+    RET(topk_enqueue(c, k, t, n_dev, false, counted));
+    counted = false;
+    tried = true;
+    return DM_OK;
+  }
+  void forget() override { tried = false; }
+  bool counted = false;       // the joins count the scores and lower the bound (best_only)
+  int64_t best_only(dm_ctx *c, dmk::SelHist **hist) override {
+    if (!prune_ptr || input_sorted || have || k > dmk::SEL_K) return 0;
+    RET(select_work(c));
+    *hist = (dmk::SelHist *)c->sel_work;
+    c->sel_dirty = true;  // until the selection that follows has run
+    counted = true;
+    return k;
+  }
   int take(dm_ctx *c, DevTable t) override {
-    DevTable tk;
-    if (!input_sorted && t.n > 16384) {
-      // a large unsorted table: select by score first and sort only the candidates, instead
-      // of sorting every row into canonical order
-      RET(topk_table(c, g, t, k, &tk));
+    if (tried && *(const uint32_t *)c->h_stage <= (uint32_t)dmk::SEL_CAP) {  // the only table there is
+      on_host = true;
+      best.n = std::min<int64_t>(k, t.n);
+      best.w = t.w;
       free_table(c, t);
-    } else {
-      if (!input_sorted || t.borrowed) RET(sort_canonical(c, t, graph_bits(g)));
-      RET(topk_of_sorted(c, g, t, k, &tk));
+      return DM_OK;
     }
+    DevTable tk;
+    RET(topk_of(c, g, t, k, input_sorted && !t.borrowed, &tk));
     if (have) {
       CollectSink cs;
       cs.parts = {best, tk};
       DevTable both;
       RET(cs.concat(c, tk.w, true, &both));
-      RET(sort_canonical(c, both, graph_bits(g)));
-      RET(topk_of_sorted(c, g, both, k, &best));
+      RET(topk_of(c, g, both, k, false, &best));
     } else {
       best = tk;
       have = true;
@@ -1736,28 +1854,8 @@ struct DirectedSink : Sink {
   }
 };
 
-bool topk_small_enough(const TopkSink *t) { return !t->have && t->k <= 1024; }
-
-// Top-k of a canonically sorted table straight into the caller's host buffers (enqueued on
-// the stream; the caller synchronises); the table stays with the caller.
-int topk_into_host(dm_ctx *c, TopkSink *t, const DevTable &sorted, int32_t *rows, float *scores, int64_t *n) {
-  const int64_t m = std::min<int64_t>(t->k, sorted.n);
-  *n = m;
-  if (m <= 0) return DM_OK;
-  DevTable o;
-  o.w = sorted.w;
-  o.n = m;
-  RET(dalloc_t(c, &o.rows, (size_t)m * sorted.w));
-  RET(dalloc_t(c, &o.score, m));
-  void *tmp = nullptr;
-  RET(dalloc(c, &tmp, (size_t)dmk::topk_tmp_bytes(sorted.n)));
-  CK(dmk::topk_sorted(sorted.rows, sorted.score, sorted.n, sorted.w, (int32_t)t->k, tmp, o.rows, o.score, c->stream));
-  dfree(c, tmp);
-  CK(cudaMemcpyAsync(rows, o.rows, sizeof(int32_t) * m * o.w, cudaMemcpyDeviceToHost, c->stream));
-  if (scores) CK(cudaMemcpyAsync(scores, o.score, sizeof(float) * m, cudaMemcpyDeviceToHost, c->stream));
-  free_table(c, o);
-  return DM_OK;
-}
+bool topk_small_enough(const TopkSink *t) { return !t->have && t->k <= dmk::SEL_K; }
+int64_t topk_k(const TopkSink *t) { return t->k; }
 
 int ensure_motif(dm_ctx *c, DevGraph *g, int id);
 
@@ -2455,6 +2553,8 @@ int dm_destroy(dm_ctx *c) {
   if (c->h_ctr_steps) cudaFreeHost(c->h_ctr_steps);
   if (c->arena) cudaFree(c->arena);
   dfree(c, c->tabs);
+  dfree(c, c->sel_work);
+  dfree(c, c->sel_out);
   cudaFree(c->m_params);
   cudaFree(c->m_grads);
   cudaFree(c->m_m);
@@ -3075,7 +3175,10 @@ int dm_score_topk(dm_ctx *c, const dm_plan_t *pl, int32_t k, int32_t *out_rows, 
   sink.prune_ptr = g->nonneg_weights ? &ex.prune : nullptr;
   ex.sink = &sink;
   int r = ex.run();
-  if (r == DM_OK) {
+  if (r == DM_OK && sink.on_host) {
+    *out_n = (int32_t)sink.best.n;
+    topk_enqueued(c, k, sink.best.n, sink.best.w, out_rows, out_scores);
+  } else if (r == DM_OK) {
     int64_t m = sink.have ? sink.best.n : 0;
     if (m > 0) {
       CK(cudaMemcpyAsync(out_rows, sink.best.rows, sizeof(int32_t) * m * sink.best.w, cudaMemcpyDeviceToHost, c->stream));

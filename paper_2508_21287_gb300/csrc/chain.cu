@@ -172,6 +172,9 @@ struct ChainWarp {
   unsigned long long sum;         // checksum of the lane's embeddings
   unsigned long long last_rows, last_cand;  // the lane's embeddings and candidates, where ch_count took them
   unsigned spent;                 // candidates of this warp so far (uniform)
+  float prune;                    // rows of a higher score are dropped (uniform)
+  int part;                       // of the rows in the first tile, which share of the candidates is this
+                                  // warp's: those at places = part modulo A.parts
 };
 
 // Whether one of the NV new ids (16 bits) of a candidate is among the row's ids it is compared with.
@@ -410,7 +413,8 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
     len &= in;
   }
   const bool then = CN && j + 1 == A.n_steps;
-  const unsigned seen = c == 0 ? __reduce_add_sync(FULL_MASK, len) : 0u;
+  auto mine = [&](int at) { return j > 1 || A.parts == 1 || at % A.parts == w.part; };
+  const unsigned seen = c == 0 && (j > 1 || w.part == 0) ? __reduce_add_sync(FULL_MASK, len) : 0u;
   const int nch0 = __shfl_sync(FULL_MASK, w.cnt, j + 1);
   int nch = nch0;
   const unsigned long long mul = s.mul;
@@ -426,7 +430,7 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
       const uint32_t nv[3] = {id0, h0 >> 16, h1 & 0xFFFFu};
       ok = ch_back_edges<MODE, NN>(A, s, slot + CH_ROWS, nv, sc);
     }
-    if (MODE == 0 && A.scored && sc > A.prune) ok = false;
+    if (MODE == 0 && A.scored && sc > w.prune) ok = false;
     const unsigned bal = __ballot_sync(FULL_MASK, ok);
     if (ok) {
       unsigned char *d = D + 8 * (nch + __popc(bal & lanemask_lt()));
@@ -450,7 +454,7 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
       for (int u = 0; u < 4; u++) {
         if (c > u) continue;                   // done before (uniform)
         if (u >= longest || nch >= 32) break;  // 32 rows in the next tile: that one first
-        one(id[u], 0u, true);
+        if (mine(u)) one(id[u], 0u, true);
         c = u + 1;
       }
     } else {
@@ -458,7 +462,7 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
       for (int u = 0; u < 4; u++) {
         if ((c & 3) != u) continue;
         if (c >= longest || nch >= 32) break;
-        one(x[u].x, x[u].y, same);
+        if (mine(c)) one(x[u].x, x[u].y, same);
         c++;
       }
       if ((c & 3) == 0 && c < longest) ch_load4(ids + c, x);
@@ -503,7 +507,7 @@ __device__ __forceinline__ void ch_step(const ChainArgs &A, unsigned char *W, Ch
     const unsigned tot = __reduce_add_sync(FULL_MASK, (unsigned)len);
     ch_state(L)[lane] = (uint32_t)start | ((uint32_t)len << 24);
     w.spent += tot;
-    if (lane == j) w.cand += tot;
+    if (lane == j && (j > 1 || w.part == 0)) w.cand += tot;
   } else {
     const uint32_t v = ch_state(L)[lane];
     start = (int)(v & 0xFFFFFFu);
@@ -521,6 +525,10 @@ __device__ __forceinline__ void ch_step(const ChainArgs &A, unsigned char *W, Ch
   int nch = count ? 0 : __shfl_sync(FULL_MASK, w.cnt, j + 1);
   unsigned K = 0;
   while (c < maxlen) {
+    if (j == 1 && A.parts > 1 && c % A.parts != w.part) {  // another warp's share
+      c++;
+      continue;
+    }
     bool ok = c < len;
     const uint4 x = ok ? __ldg(rec + c * units) : make_uint4(0, 0, 0, 0);
     uint4 y = make_uint4(x.z, x.w, 0, 0);
@@ -543,7 +551,7 @@ __device__ __forceinline__ void ch_step(const ChainArgs &A, unsigned char *W, Ch
     float sc = 0.f;
     if (MODE == 0) sc = __uint_as_float((uint32_t)tail) + __uint_as_float((uint32_t)add);
     if (s.n_be && ok) ok = ch_back_edges<MODE, CH_NEW>(A, s, row, nv, sc);
-    if (MODE == 0 && A.scored && sc > A.prune) ok = false;
+    if (MODE == 0 && A.scored && sc > w.prune) ok = false;
     const unsigned bal = __ballot_sync(FULL_MASK, ok);
     c++;
     if (bal == 0) continue;
@@ -596,7 +604,7 @@ __device__ __forceinline__ void ch_seed(const ChainArgs &A, unsigned char *W, Ch
       if (MODE == 0 && ok && A.scored && A.eerr) sc += ch_edge_weight(A, va, vb);
     }
   }
-  if (MODE == 0 && A.scored && sc > A.prune) ok = false;
+  if (MODE == 0 && A.scored && sc > w.prune) ok = false;
   const unsigned bal = __ballot_sync(FULL_MASK, ok);
   const int n = __shfl_sync(FULL_MASK, w.cnt, 1);
   unsigned char *D = W + (unsigned)A.st[1].in_off * 8u;
@@ -613,7 +621,7 @@ __device__ __forceinline__ void ch_seed(const ChainArgs &A, unsigned char *W, Ch
     ch_tail(D)[pos] = MODE == 1 ? p : (unsigned long long)__float_as_uint(sc);
   }
   if (lane == 1) w.cnt = n + __popc(bal);
-  if (lane == 0) {
+  if (lane == 0 && w.part == 0) {
     w.rows += __popc(bal);
     w.cand += nr;
   }
@@ -658,6 +666,49 @@ __device__ __forceinline__ bool ch_put(const ChainArgs &A, unsigned char *W, Cha
   return true;
 }
 
+// Lower the bound of a top-k run: the upper end of the bin that holds the k-th best of the rows written
+// so far by anyone. Rows above it, and partial rows above it where no weight is negative, cannot be
+// among the k best.
+__device__ __forceinline__ void ch_bound(const ChainArgs &A, ChainWarp &w) {
+  constexpr int PER = SelHist::COARSE / 32;
+  const int lane = threadIdx.x & 31;
+  unsigned c[PER], sum = 0;
+#pragma unroll
+  for (int i = 0; i < PER; i++) sum += c[i] = *(volatile unsigned *)&A.sel->coarse[lane * PER + i];
+  unsigned incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(FULL_MASK, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const unsigned k = (unsigned)A.sel_k;
+  if (__shfl_sync(FULL_MASK, incl, 31) < k) return;
+  // the first lane that reaches k, its bin, and how many of that bin are needed
+  const int at = __ffs(__ballot_sync(FULL_MASK, incl >= k)) - 1;
+  unsigned before = incl - sum;
+  int bin = lane * PER;
+  for (int i = 0; i + 1 < PER && before + c[i] < k; i++) {
+    before += c[i];
+    bin++;
+  }
+  before = __shfl_sync(FULL_MASK, before, at);
+  bin = __shfl_sync(FULL_MASK, bin, at);
+  constexpr int SUB = SelHist::FINE / SelHist::COARSE;  // 32
+  incl = *(volatile unsigned *)&A.sel->fine[bin * SUB + lane];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned v = __shfl_up_sync(FULL_MASK, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const unsigned hit = __ballot_sync(FULL_MASK, before + incl >= k);
+  if (!hit) return;  // the counts moved on between the two reads
+  const uint32_t top = ((uint32_t)(bin * SUB + __ffs(hit) - 1) << SelHist::FINE_SHIFT) | ((1u << SelHist::FINE_SHIFT) - 1);
+  // scores are not negative where this runs, so their bits order like their keys
+  const int bits = (int)(top & 0x7FFFFFFFu);
+  if (lane == 0) atomicMin(&A.sel->bound, bits);
+  w.prune = fminf(w.prune, __int_as_float(bits));
+}
+
 // All rows of the output tile to the packed result in pattern-vertex order. False when they do
 // not fit, as above.
 __device__ __forceinline__ bool ch_flush(const ChainArgs &A, unsigned char *W, ChainWarp &w, const uint16_t *ooff) {
@@ -673,7 +724,21 @@ __device__ __forceinline__ bool ch_flush(const ChainArgs &A, unsigned char *W, C
     return false;
   }
   if (A.scored)
-    for (int i = lane; i < n; i += 32) A.outs[at + i] = __uint_as_float((uint32_t)ch_tail(L)[i]);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const float sc = i < n ? __uint_as_float((uint32_t)ch_tail(L)[i]) : 0.f;
+      if (i < n) A.outs[at + i] = sc;
+      if (A.sel) {  // scores crowd in a few bins: one addition a bin and warp
+        const uint32_t key = i < n ? score_key(sc) : ~0u;
+        const unsigned f = __match_any_sync(FULL_MASK, key >> SelHist::FINE_SHIFT);
+        const unsigned c = __match_any_sync(FULL_MASK, key >> SelHist::COARSE_SHIFT);
+        if (i < n) {
+          if ((f & lanemask_lt()) == 0) atomicAdd(&A.sel->fine[key >> SelHist::FINE_SHIFT], (unsigned)__popc(f));
+          if ((c & lanemask_lt()) == 0) atomicAdd(&A.sel->coarse[key >> SelHist::COARSE_SHIFT], (unsigned)__popc(c));
+        }
+      }
+    }
+  if (A.sel) ch_bound(A, w);
   int32_t *out = A.out + at * wo;
   const unsigned char *rows = ch_rows(L);
   int r = lane / wo, q = lane - r * wo;
@@ -704,21 +769,29 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
   griddep_wait();  // the candidate tables, the counters and the input table come from the launches before
   griddep_launch_dependents();
   ChainWarp w{};
+  w.prune = A.prune;
+  float best = A.prune;  // the bound as it was asked for last
   const int64_t nw = (int64_t)gridDim.x * CH_WARPS;
   const int64_t n_in = A.in ? imin64((int64_t)*A.in_blocks, A.in_cap) - A.lo : (A.seed_n - A.lo + A.chunk - 1) / A.chunk;
   // a table of few blocks is dealt out in quarters of a block
   const int parts = A.in && n_in < 8 * nw ? 4 : 1;
-  const int64_t n_items = n_in * parts;
+  const int64_t n_items = n_in * parts * A.parts;
   // items 0 .. nw - 1 are the warps' first; the counter deals out the rest. The next item's number
   // is asked for before the present one is joined.
   long long nxt = (int64_t)blockIdx.x * CH_WARPS + wid;
   bool more = true;
   while (true) {
     __syncwarp();
+    if (MODE == 0 && A.sel) {  // used from the next turn on: nothing waits for it
+      w.prune = fminf(w.prune, best);
+      best = __int_as_float(*(volatile int *)&A.sel->bound);
+    }
     const unsigned act = __ballot_sync(FULL_MASK, w.cnt >= 32 || w.prog > 0);
     int j;
     if (act) {
       j = 31 - __clz(act);
+    } else if (A.parts > 1 && __shfl_sync(FULL_MASK, w.cnt, 1) > 0) {
+      j = 1;  // the first tile holds one share only
     } else {
       if (more) {
         const long long it = __shfl_sync(FULL_MASK, nxt, 0);
@@ -729,7 +802,8 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
           if (A.in) {
             ch_fetch(A, W, w, A.lo + it / parts, (int)(it % parts) * (4 / parts), 4 / parts);
           } else {
-            const int64_t lo = A.lo + it * A.chunk;
+            w.part = (int)(it % A.parts);
+            const int64_t lo = A.lo + it / A.parts * A.chunk;
             ch_seed<MODE>(A, W, w, lo, (int)imin64(A.chunk, A.seed_n - lo));
           }
         }

@@ -53,6 +53,14 @@ int wjoin_grid(const dmi::JoinArgs &a, int num_sms);
 bool fused_ok(const dmi::JoinArgs &a, const dmi::JoinArgs &b);
 cudaError_t launch_fused(const dmi::JoinArgs &a, const dmi::JoinArgs &b, int num_sms, cudaStream_t s, bool pdl);
 
+// Scores of a table's rows by the leading bits of their order-preserving keys (select.cu), and the bound
+// that a top-k run of the joins lowers as it goes (bits of a non-negative score).
+struct SelHist {
+  static constexpr int FINE = 8192, FINE_SHIFT = 32 - 13, COARSE = 256, COARSE_SHIFT = 32 - 8;
+  uint32_t fine[FINE], coarse[COARSE];
+  int32_t bound;
+};
+
 // Several steps of a plan, often all of them, in one launch (chain.cu).
 constexpr int CH_STEPS = 24;          // steps of a launch besides the seed, at most
 constexpr int CH_NEW = 8;             // new vertices and further keys of a step, at most
@@ -103,7 +111,10 @@ struct ChainArgs {
   const int32_t *seed_rows;
   const float *seed_score;
   int32_t seed_mw, seed_k, seed_nbe, shard, n_shards;
-  int64_t seed_n, chunk;         // chunk <= 32 rows of the first table are one work item
+  // chunk <= 32 rows of the first table are one work item, or with parts > 1 as many: every warp then
+  // takes one share of their first step's candidates
+  int64_t seed_n, chunk;
+  int32_t parts;
   int64_t lo;                    // input already joined by earlier launches: rows of the first table, or blocks
   uint8_t seed_npos[dmi::MAXM], seed_be[8][2];
   uint16_t seed_off[dmi::MAXM];
@@ -117,6 +128,8 @@ struct ChainArgs {
   float *outs;
   int32_t *out_rows;
   int64_t out_cap;               // rows, or blocks
+  SelHist *sel;                  // rows are wanted for their k best only: counted here, pruned by its bound
+  int32_t sel_k;
   uint16_t out_off[dmi::MAXW];   // output position -> byte offset in the last tile's rows
 };
 int chain_grid(const ChainArgs &a, int num_sms);  // blocks of a full launch
@@ -226,11 +239,25 @@ cudaError_t msort_rows_into(const int32_t *rows, const float *scores, int64_t n,
 cudaError_t msort_rows(const int32_t *rows, int64_t n, int32_t w, int bits, void *tmp, int32_t **perm_out,
                        unsigned long long *sum, cudaStream_t s);
 
-// The min(k, n) smallest (score key, row index) of a canonically sorted table, k <= 1024,
-// gathered into orows / osc in that order. tmp holds topk_tmp_bytes(n) bytes.
-int64_t topk_tmp_bytes(int64_t n);
-cudaError_t topk_sorted(const int32_t *rows, const float *sc, int64_t n, int32_t w, int32_t k, void *tmp,
-                        int32_t *orows, float *osc, cudaStream_t s);
+// The min(k, n) best rows of a table by (score, row), k <= SEL_K (select.cu). out: the number of rows
+// collected on the way (4 bytes, padded to 16; above SEL_CAP nothing else was written and the caller
+// takes another way), k scores, k rows. work: select_work_bytes(), zeroed once before the first call.
+constexpr int SEL_K = 1024, SEL_CAP = 16384;
+struct SelectArgs {
+  const int32_t *rows;
+  const float *sc;
+  int64_t n;                         // rows, or with n_dev the most *n_dev may say
+  const unsigned long long *n_dev;
+  int32_t w, k, sorted;              // sorted: the rows are in canonical order
+  int32_t counted;                   // the scores are in the work buffer's histogram already
+  void *work;
+  unsigned char *out;
+};
+constexpr int64_t select_out_bytes(int64_t k, int64_t w) { return 16 + 4 * k + 4 * k * w; }
+int64_t select_work_bytes();
+// (the work buffer starts with a SelHist, all zero but bound = the bits of +infinity between calls)
+constexpr int32_t SEL_NO_BOUND = 0x7F800000;
+cudaError_t topk_select(const SelectArgs &a, int num_sms, cudaStream_t s);
 
 // Images (sort.cu): sort the ids inside each row in place; then, on canonically sorted rows,
 // keep the first row of every run of equal rows (pos[n] receives the number kept; flag holds n

@@ -1,4 +1,4 @@
-// Canonical (lexicographic) order of embedding rows, and top-k by (score, row).
+// Canonical (lexicographic) order of embedding rows.
 //
 // Rows are sorted by comparison on packed keys: every row's ids are packed, bits(V) bits each
 // and most significant first, into up to MS_KW 64-bit words (floor(64 / bits) ids per word).
@@ -11,12 +11,6 @@
 // every row at its final position in one rank-scatter launch (msort_rows_into). The
 // key-packing kernel can also add the rows' checksum hashes (the same H as the join's count
 // mode) into a counter, so that delivering a table needs no separate hashing pass.
-//
-// Top-k runs on a canonically sorted table: the key of row i is (score_key(score), i), where
-// score_key maps an FP32 score to an unsigned key that orders like its value (either sign),
-// and i orders like the row.
-// Each block sorts a tile of keys and keeps its k smallest; the candidates shrink by that
-// factor per pass until one tile holds them all.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -388,203 +382,6 @@ cudaError_t unique_rows(const int32_t *rows, int64_t n, int32_t w, int32_t *flag
   int g2 = (int)((ne + 255) / 256 > 16384 ? 16384 : (ne + 255) / 256);
   k_compact_rows<<<g2, 256, 0, s>>>(rows, n, w, flag, pos, out);
   g_launches += 2;
-  return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------ top-k --------------
-constexpr int TK_BLK = 512;
-constexpr int TK_TILE = 2048;
-
-__global__ void k_topk_keys_from_scores(const float *sc, int64_t n, unsigned long long *key) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    key[i] = ((unsigned long long)score_key(__ldg(sc + i)) << 32) | (uint32_t)i;
-}
-
-// Each block sorts TK_TILE keys and writes its k smallest (k <= TK_TILE).
-__global__ void __launch_bounds__(TK_BLK) k_topk_tiles(const unsigned long long *in, int64_t n, int32_t k,
-                                                       unsigned long long *out) {
-  __shared__ unsigned long long sk[TK_TILE];
-  griddep_wait();
-  griddep_launch_dependents();
-  const int64_t base = (int64_t)blockIdx.x * TK_TILE;
-  for (int i = threadIdx.x; i < TK_TILE; i += TK_BLK) sk[i] = base + i < n ? in[base + i] : KEY_INF;
-  __syncthreads();
-  for (int kk = 2; kk <= TK_TILE; kk <<= 1)
-    for (int j = kk >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < TK_TILE / 2; t += TK_BLK) {
-        int i = 2 * t - (t & (j - 1));
-        int p = i + j;
-        bool up = (i & kk) == 0;
-        if ((sk[i] > sk[p]) == up) {
-          unsigned long long x = sk[i];
-          sk[i] = sk[p];
-          sk[p] = x;
-        }
-      }
-      __syncthreads();
-    }
-  for (int i = threadIdx.x; i < k; i += TK_BLK) out[(int64_t)blockIdx.x * k + i] = sk[i];
-}
-
-__global__ void k_topk_gather(const unsigned long long *keys, int32_t m, const int32_t *rows, const float *sc,
-                              int32_t w, int32_t *orows, float *osc) {
-  griddep_wait();
-  griddep_launch_dependents();
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)m * w;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t i = e / w;
-    int32_t c = (int32_t)(e - i * w);
-    uint32_t src = (uint32_t)(keys[i] & 0xffffffffu);
-    orows[e] = rows[(int64_t)src * w + c];
-    if (c == 0 && osc) osc[i] = sc[src];
-  }
-}
-
-// Top-k of up to TK_SMALL keys in one block: the keys sit in shared memory, an MSD radix
-// select over their 64 bits (8 bits a pass, warp-scanned histogram) finds the k-th smallest,
-// the k keys at or below it are collected and sorted by a bitonic network, and the rows are
-// gathered. One launch instead of the tile passes.
-constexpr int TK_SMALL = 16384;
-constexpr int TK_SBLK = 1024;
-
-__global__ void __launch_bounds__(TK_SBLK) k_topk_small(const float *sc, int32_t n, int32_t k, const int32_t *rows,
-                                                       int32_t w, int32_t *orows, float *osc) {
-  extern __shared__ unsigned long long K[];  // n keys
-  __shared__ unsigned long long C[1024];
-  __shared__ unsigned hist[256];
-  __shared__ unsigned long long s_prefix;
-  __shared__ int s_need, s_cnt;
-  griddep_wait();
-  griddep_launch_dependents();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < n; i += TK_SBLK) K[i] = ((unsigned long long)score_key(__ldg(sc + i)) << 32) | (uint32_t)i;
-  const int kk = k < n ? k : n;
-  if (tid == 0) {
-    s_prefix = 0;
-    s_need = kk;
-    s_cnt = 0;
-  }
-  __syncthreads();
-  unsigned long long T = KEY_INF;  // the kk-th smallest key (all keys when kk == n)
-  if (kk < n) {
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int d = tid; d < 256; d += TK_SBLK) hist[d] = 0;
-      __syncthreads();
-      const unsigned long long hi = shift == 56 ? 0ull : (~0ull << (shift + 8));
-      const unsigned long long pre = s_prefix;
-      for (int i = tid; i < n; i += TK_SBLK)
-        if ((K[i] & hi) == pre) atomicAdd(&hist[(K[i] >> shift) & 255], 1u);
-      __syncthreads();
-      if (warp == 0) {  // lane l holds bins 8l .. 8l+7
-        unsigned b[8], sum = 0;
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-          b[j] = hist[8 * lane + j];
-          sum += b[j];
-        }
-        unsigned incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          unsigned v = __shfl_up_sync(FULL_MASK, incl, o);
-          if (lane >= o) incl += v;
-        }
-        const unsigned need = (unsigned)s_need;
-        const unsigned excl = incl - sum;
-        if (excl < need && need <= incl) {  // exactly one lane: the bin holding the need-th key
-          unsigned cum = excl;
-          int d = 0;
-#pragma unroll
-          for (int j = 0; j < 8; j++) {
-            if (cum + b[j] >= need) {
-              d = j;
-              break;
-            }
-            cum += b[j];
-          }
-          s_prefix = pre | ((unsigned long long)(8 * lane + d) << shift);
-          s_need = (int)(need - cum);
-        }
-      }
-      __syncthreads();
-    }
-    T = s_prefix;
-  }
-  for (int i = tid; i < n; i += TK_SBLK)
-    if (K[i] <= T) C[atomicAdd(&s_cnt, 1)] = K[i];
-  __syncthreads();
-  int P = 1;
-  while (P < kk) P <<= 1;
-  for (int i = kk + tid; i < P; i += TK_SBLK) C[i] = KEY_INF;
-  __syncthreads();
-  for (int q = 2; q <= P; q <<= 1)
-    for (int j = q >> 1; j > 0; j >>= 1) {
-      for (int t = tid; t < P / 2; t += TK_SBLK) {
-        int i = 2 * t - (t & (j - 1));
-        int p = i + j;
-        bool up = (i & q) == 0;
-        if ((C[i] > C[p]) == up) {
-          unsigned long long x = C[i];
-          C[i] = C[p];
-          C[p] = x;
-        }
-      }
-      __syncthreads();
-    }
-  for (int64_t e = tid; e < (int64_t)kk * w; e += TK_SBLK) {
-    const int64_t i = e / w;
-    const int32_t c = (int32_t)(e - i * w);
-    const uint32_t src = (uint32_t)(C[i] & 0xffffffffu);
-    orows[e] = __ldg(rows + (int64_t)src * w + c);
-    if (c == 0 && osc) osc[i] = __ldg(sc + src);
-  }
-}
-
-int64_t topk_tmp_bytes(int64_t n) {
-  int64_t tiles = (n + TK_TILE - 1) / TK_TILE;
-  return ((n > TK_TILE ? n : TK_TILE) + tiles * TK_TILE) * 8 + 256;
-}
-
-cudaError_t topk_sorted(const int32_t *rows, const float *sc, int64_t n, int32_t w, int32_t k, void *tmp,
-                        int32_t *orows, float *osc, cudaStream_t s) {
-  if (n <= 0 || k <= 0) return cudaSuccess;
-  if (k > TK_TILE / 2) return cudaErrorInvalidValue;
-  if (n <= TK_SMALL) {
-    static std::atomic<unsigned long long> attr{0};  // per device, as for the join kernels
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (!(attr.load() & (1ull << (dev & 63)))) {
-      cudaFuncSetAttribute(k_topk_small, cudaFuncAttributeMaxDynamicSharedMemorySize, TK_SMALL * 8);
-      attr.fetch_or(1ull << (dev & 63));
-    }
-    g_launches++;
-    k_topk_small<<<1, TK_SBLK, (size_t)n * 8, s>>>(sc, (int32_t)n, k, rows, w, orows, osc);
-    return cudaGetLastError();
-  }
-  unsigned long long *a = (unsigned long long *)tmp;
-  unsigned long long *b = a + (n > TK_TILE ? n : TK_TILE);
-  int grid = (int)((n + 255) / 256);
-  if (grid > 16384) grid = 16384;
-  k_topk_keys_from_scores<<<grid, 256, 0, s>>>(sc, n, a);
-  int launches = 1;
-  unsigned long long *cur = a, *other = b;
-  int64_t m = n;
-  while (true) {  // every pass keeps k of each 2048 keys, so m at least halves
-    int64_t blocks = (m + TK_TILE - 1) / TK_TILE;
-    int32_t keep = (int32_t)(m < k ? m : k);
-    launch_pdl(k_topk_tiles, dim3((unsigned)blocks), dim3(TK_BLK), 0, s, (const unsigned long long *)cur, m, keep,
-               other);
-    launches++;
-    m = blocks * keep;
-    std::swap(cur, other);
-    if (blocks == 1) break;
-  }
-  int32_t out_n = (int32_t)(m < k ? m : k);
-  int64_t ne = (int64_t)out_n * w;
-  int g2 = (int)((ne + 255) / 256);
-  launch_pdl(k_topk_gather, dim3(g2 > 0 ? g2 : 1), dim3(256), 0, s, (const unsigned long long *)cur, out_n, rows, sc,
-             w, orows, osc);
-  launches++;
-  g_launches += launches;
   return cudaGetLastError();
 }
 

@@ -92,6 +92,35 @@ def test_every_form_equals_the_oracle(ctx, B, name):
             assert stats["rows"] == other["rows"] and stats["candidates"] == other["candidates"], (name, p.name, motifs)
 
 
+@pytest.mark.parametrize("weights", ["lognormal", "equal", "two", "negative"])
+@pytest.mark.parametrize("k", [1, 10, 1000, 1024, 1025])
+def test_best_rows(ctx, weights, k):
+    # small and large tables, first tables of fewer rows than warps, scores that thousands of rows
+    # share (the selection gives up), few distinct scores, and weights that forbid pruning
+    for g, p in ((I.heavy_hex(4, 6), I.path(18)), (I.heavy_hex(2, 2), I.path(6)), (I.random_regular3(512, 3), I.path(9)),
+                 (I.grid(9, 7), I.sub_patch(I.grid(9, 7), 8, 2))):
+        g = I.lognormal_weights(g, 11)
+        if weights == "equal":
+            g.edge_err[:] = 0.25
+        elif weights == "two":
+            g.edge_err[:] = np.where(g.edge_err > np.median(g.edge_err), 0.5, 0.25)
+        elif weights == "negative":
+            g.edge_err -= 0.006
+        gid = ctx.load(g)
+        rows, scores = ctx.plan(gid, p).topk(k)
+        ref = oracle.enumerate(g, p)
+        want = oracle.scores(g, p, ref.rows)
+        order = oracle.topk(ref.rows, want, k)
+        assert len(rows) == min(k, ref.count)
+        # sums of at most 17 terms of at most 0.5: FP32 error below 17 * 2^-24 * 8.5 ~ 9e-6
+        np.testing.assert_allclose(scores, want[order], rtol=0, atol=9e-6)
+        if weights in ("equal", "two"):  # exact in FP32: the rows are decided
+            assert np.array_equal(rows, ref.rows[order])
+        # the same again, through the form that keeps every row
+        r2, s2 = ctx.plan(gid, p, chunk_rows=4000).topk(k)
+        np.testing.assert_allclose(s2, scores, rtol=0, atol=9e-6)
+
+
 @pytest.mark.parametrize("n", [65533, 65534, 65535])
 def test_edge_of_16_bit_ids(ctx, n):
     # a path: 2 (n - k + 1) embeddings of the path of k vertices; ids up to n - 1
