@@ -64,6 +64,7 @@ struct DevGraph {
   // girth, and whether every cycle is even
   int32_t girth = 3;
   bool bipartite = false;
+  uint2 *adj4 = nullptr;  // neighbour lists of 16-bit ids, where no degree is above 4
   double edge_deg = 0;  // mean degree of the vertices that edges lead to
   std::map<int, DevTable> motifs;
   std::map<std::tuple<int, int, int, int>, Index> indices;  // (motif, key position 0, 1, sort-merge)
@@ -90,6 +91,7 @@ struct dm_ctx {
   size_t arena_bytes = 0;
   void *sel_work = nullptr, *sel_out = nullptr;  // top-k selection (select.cu)
   size_t sel_out_bytes = 0;
+  void *ord_work = nullptr;  // canonical order (order.cu)
   bool sel_dirty = false;  // its histogram holds counts that no selection has cleared
   void *tabs = nullptr;  // candidate tables of the plan that runs (chain.cu)
   int64_t tab_bytes = 0;
@@ -463,10 +465,19 @@ struct Sink {
   virtual ~Sink() {}
   // Takes ownership of a table of final rows (pattern-vertex order, unsorted).
   virtual int take(dm_ctx *c, DevTable t) = 0;
-  // Called before the stream is waited for, for a table that will be the only one if it fits: t.n is
-  // the most rows it can have, *n_dev receives how many it has. Work enqueued here is void when the
-  // table turns out not to fit; otherwise take() follows.
-  virtual int ahead(dm_ctx *, const DevTable &, const unsigned long long *) { return DM_OK; }
+  // Called before the stream is waited for, for a table that will be the only one if it fits. Work
+  // enqueued here is void when the table turns out not to fit; otherwise take() follows.
+  struct Ahead {
+    DevTable t;                       // t.n: the most rows it can have
+    const unsigned long long *n_dev;  // receives how many it has
+    unsigned char *spare;             // memory behind it until take() returns
+    int64_t spare_bytes;
+    unsigned long long *ctr;          // CTR_N zeroed counters, which come back with the joins' own
+    const unsigned long long *h_ctr;
+    const Plan *p;
+    DevGraph *g;
+  };
+  virtual int ahead(dm_ctx *, const Ahead &) { return DM_OK; }
   virtual void forget() {}  // the table did not fit, or others follow it
   // k > 0: only the k best rows are wanted, and rows whose partial score is above the k-th best of those
   // seen may be dropped; hist receives where the joins count the scores of what they write
@@ -1309,8 +1320,12 @@ struct Exec {
     unsigned char *tabs = (unsigned char *)c->tabs;
     for (int y = 0; y < C.n_tab; y++) C.tab.tab[y].out = tabs + C.tab_off[y];
     C.tab.ctr = c->d_ctr_steps;
-    C.tab.n_ctr = (int64_t)CTR_N * S;
-    const size_t half = C.launch.size() > 1 ? (c->arena_bytes / 2) / 256 * 256 : c->arena_bytes;
+    C.tab.n_ctr = (int64_t)CTR_N * (S + 1);  // and one set for the sink
+    // row mode: the sink's work behind the joins needs room that no later round of launches reads. Two
+    // halves hold the rows and that, or with tables between launches three thirds; an arena that cannot
+    // grow any more keeps halves for the tables and leaves the sink to itself.
+    const bool several = C.launch.size() > 1, spare = mode == DM_ALL && (!several || c->arena_bytes < c->budget);
+    const size_t half = c->arena_bytes / (several && spare ? 3 : 2) / 256 * 256;
     int ends = 0;  // plan steps up to the launch
     std::vector<int> grid(C.launch.size());
     for (size_t i = 0; i < C.launch.size(); i++) {
@@ -1387,15 +1402,23 @@ struct Exec {
         run_steps += A.n_steps + (A.in ? 0 : 1);
       }
       if (c->timing) CK(cudaEventRecord(c->ev1, c->stream));
-      if (first && mode == DM_ALL) {
-        DevTable t;
-        t.rows = C.launch.back().out;
-        t.score = C.launch.back().outs;
-        t.n = C.launch.back().out_cap;
-        t.w = C.launch.back().wo;
-        RET(sink->ahead(c, t, C.launch.back().ctr_last + CTR_ROWS));
+      if (first && spare) {
+        const dmk::ChainArgs &A = C.launch.back();
+        Sink::Ahead a{};
+        a.t.rows = A.out;
+        a.t.score = A.outs;
+        a.t.n = A.out_cap;
+        a.t.w = A.wo;
+        a.n_dev = A.ctr_last + CTR_ROWS;
+        a.spare = c->arena + (several ? 2 : 1) * half;
+        a.spare_bytes = (int64_t)half;
+        a.ctr = c->d_ctr_steps + (size_t)S * CTR_N;
+        a.h_ctr = c->h_ctr_steps + (size_t)S * CTR_N;
+        a.p = p;
+        a.g = g;
+        RET(sink->ahead(c, a));
       }
-      CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * S,
+      CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * (S + 1),
                          cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
       if (c->timing) {
@@ -1614,8 +1637,72 @@ struct AllSink : Sink {
     free_table(c, t);
     return r;
   }
+  // The only table, put into canonical order on the device behind the joins (order.cu): the sorted rows,
+  // their number, checksum and top-k come back with the joins' counters.
+  bool tried = false;
+  const unsigned long long *h_ahead = nullptr;
+  DevTable sorted;
+  int ahead(dm_ctx *c, const Ahead &a) override {
+    const int64_t w = a.t.w;
+    dmk::OrderArgs o{};
+    o.rows = a.t.rows;
+    o.sc = a.t.score;
+    o.n_dev = a.n_dev;
+    o.w = (int32_t)w;
+    o.adj4 = a.g->adj4;
+    // a column's code is its place among the neighbours of an earlier column's vertex, where that is short
+    const int place = std::max(2, a.g->max_deg);
+    for (int32_t col = 0; col < w; col++) {
+      o.ref[col] = dmk::ORD_NONE;
+      for (int32_t e = a.p->rp[col]; e < a.p->rp[col + 1] && a.g->adj4; e++)
+        if (a.p->ci[e] < col) o.ref[col] = (uint8_t)a.p->ci[e];
+    }
+    const int kw = dmk::order_layout(o, (unsigned)std::max(2, a.g->V), (unsigned)place);
+    o.cap = std::min<int64_t>(a.t.n, (a.spare_bytes - 2048) / (4 * w + 4 + 8 * kw + 8)) / 64 * 64;
+    if (o.cap < 64) return DM_OK;
+    if (!c->ord_work) {
+      RET(dalloc(c, &c->ord_work, (size_t)dmk::order_work_bytes()));
+      CK(cudaMemsetAsync(c->ord_work, 0, (size_t)dmk::order_work_bytes(), c->stream));
+    }
+    o.work = (dmk::OrderWork *)c->ord_work;
+    unsigned char *at = a.spare;
+    o.key = (unsigned long long *)at;
+    at += 8 * kw * o.cap;
+    o.num = (int32_t *)at;
+    at += 4 * o.cap;
+    o.idx = (int32_t *)at;
+    at += 4 * o.cap;
+    o.out = (int32_t *)at;
+    at += 4 * w * o.cap;
+    o.outs = a.t.score ? (float *)at : nullptr;
+    o.ctr = a.ctr;
+    CK(dmk::order_rows(o, kw, c->num_sms, c->stream));
+    sorted.rows = o.out;
+    sorted.score = o.outs;
+    sorted.w = (int32_t)w;
+    sorted.n = o.cap;
+    sorted.borrowed = true;
+    if (tap && final_rows && topk_small_enough(tap)) RET(topk_enqueue(c, topk_k(tap), sorted, a.n_dev, true));
+    h_ahead = a.h_ctr;
+    tried = true;
+    return DM_OK;
+  }
+  void forget() override { tried = false; }
   int take(dm_ctx *c, DevTable t) override {
     int64_t tb = t.n * (4ll * t.w + (t.score ? 4 : 0));
+    if (tried && !h_ahead[CTR_OVF] && held.empty() && !streaming && tb <= (int64_t)c->budget / 2) {
+      sorted.n = t.n;
+      count = (uint64_t)t.n;
+      checksum = h_ahead[CTR_SUM];
+      const bool fast_topk = tap && final_rows && topk_small_enough(tap);
+      if (fast_topk) {  // before the staging buffer is used for the rows
+        final_n = std::min(topk_k(tap), t.n);
+        final_done = t.n == 0 || topk_enqueued(c, topk_k(tap), t.n, t.w, final_rows, final_scores);
+      }
+      int r = deliver(c, sorted, flags, cb, user, true);
+      if (r == DM_OK && tap && !final_done) r = topk_take(c, tap, sorted);
+      return r;
+    }
     if (!streaming && held_bytes + tb <= (int64_t)c->budget / 2) {
       held.push_back(t);
       held_bytes += tb;
@@ -1782,9 +1869,9 @@ struct TopkSink : Sink {
   float *prune_ptr = nullptr;
   bool tried = false;         // the first table's selection is enqueued (ahead)
   bool on_host = false;       // ... and its result is in the staging buffer: best stays empty
-  int ahead(dm_ctx *c, const DevTable &t, const unsigned long long *n_dev) override {
-    if (input_sorted || have || k > dmk::SEL_K || !t.score) return DM_OK;
-    RET(topk_enqueue(c, k, t, n_dev, false, counted));
+  int ahead(dm_ctx *c, const Ahead &a) override {
+    if (input_sorted || have || k > dmk::SEL_K || !a.t.score) return DM_OK;
+    RET(topk_enqueue(c, k, a.t, a.n_dev, false, counted));
     counted = false;
     tried = true;
     return DM_OK;
@@ -2448,6 +2535,7 @@ void free_graph(dm_ctx *c, DevGraph *g) {
     if (kv.second.slots) dfree(c, kv.second.slots);
     if (kv.second.keys) dfree(c, kv.second.keys);
   }
+  dfree(c, g->adj4);
   cudaFree(g->row_ptr);
   cudaFree(g->col_idx);
   cudaFree(g->eerr);
@@ -2502,8 +2590,8 @@ int dm_create(dm_ctx **out, int device, uint64_t mem_budget_bytes) {
     dm_destroy(c);
     return DM_E_NOMEM;
   }
-  if (cudaMalloc(&c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * DM_MAX_STEPS) != cudaSuccess ||
-      cudaMallocHost(&c->h_ctr_steps, sizeof(unsigned long long) * CTR_N * DM_MAX_STEPS) != cudaSuccess) {
+  if (cudaMalloc(&c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * (DM_MAX_STEPS + 1)) != cudaSuccess ||
+      cudaMallocHost(&c->h_ctr_steps, sizeof(unsigned long long) * CTR_N * (DM_MAX_STEPS + 1)) != cudaSuccess) {
     dm_destroy(c);
     return DM_E_NOMEM;
   }
@@ -2554,6 +2642,7 @@ int dm_destroy(dm_ctx *c) {
   if (c->arena) cudaFree(c->arena);
   dfree(c, c->tabs);
   dfree(c, c->sel_work);
+  dfree(c, c->ord_work);
   dfree(c, c->sel_out);
   cudaFree(c->m_params);
   cudaFree(c->m_grads);
@@ -2638,6 +2727,10 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
         cudaMemcpyAsync(h_girth, d, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
       r = DM_E_CUDA;
     g->bipartite = two_colourable(h, n);
+    if (r == DM_OK && md <= 4 && n <= 65534) {
+      r = dalloc_t(c, &g->adj4, (size_t)n);
+      if (r == DM_OK && dmk::launch_adj4(g->row_ptr, g->col_idx, n, g->adj4, c->stream) != cudaSuccess) r = DM_E_CUDA;
+    }
   }
   if (r == DM_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) r = DM_E_CUDA;
   if (r == DM_OK) g->girth = *(int32_t *)c->h_ctr;

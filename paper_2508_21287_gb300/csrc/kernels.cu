@@ -126,6 +126,23 @@ cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t
   return cudaGetLastError();
 }
 
+__global__ void k_adj4(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, uint2 *adj4) {
+  const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= V) return;
+  const int32_t lo = __ldg(row_ptr + v), n = __ldg(row_ptr + v + 1) - lo;
+  uint32_t q[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) q[i] = i < n ? (uint32_t)__ldg(col_idx + lo + i) : 0xFFFFu;
+  adj4[v] = make_uint2(q[0] | (q[1] << 16), q[2] | (q[3] << 16));
+}
+
+cudaError_t launch_adj4(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, uint2 *adj4, cudaStream_t s) {
+  if (V <= 0) return cudaSuccess;
+  g_launches++;
+  k_adj4<<<(V + 127) / 128, 128, 0, s>>>(row_ptr, col_idx, V, adj4);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ scan ---------------
 static_assert(SCAN_TILE == SCAN_BLK * SCAN_ITEMS, "scan tile");
 

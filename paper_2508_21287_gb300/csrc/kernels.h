@@ -162,6 +162,8 @@ cudaError_t launch_csr_to_m2(const int32_t *row_ptr, const int32_t *col_idx, con
 // *girth = min(*girth, a lower bound of the graph's girth); the caller sets it to GIRTH_MAX before.
 constexpr int GIRTH_MAX = 32;
 cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth, cudaStream_t s);
+// adj4[v]: the neighbours of v, ascending, 16 bits each, 0xFFFF past its degree (at most 4; V <= 65 534).
+cudaError_t launch_adj4(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, uint2 *adj4, cudaStream_t s);
 cudaError_t launch_vertex_table(int32_t V, int32_t *rows, float *score, cudaStream_t s);
 cudaError_t launch_bitmap(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int64_t nnz,
                           int32_t words, unsigned long long *adj, cudaStream_t s);
@@ -238,6 +240,38 @@ cudaError_t msort_rows_into(const int32_t *rows, const float *scores, int64_t n,
 // When sum is set, the row checksums (sum of H(row), as the count-mode join) are added to it.
 cudaError_t msort_rows(const int32_t *rows, int64_t n, int32_t w, int bits, void *tmp, int32_t **perm_out,
                        unsigned long long *sum, cudaStream_t s);
+
+// Canonical order of a table of embeddings whose row count is on the device (order.cu). The counters
+// ctr[CTR_SUM] (zeroed by the caller) and ctr[CTR_OVF] receive the rows' checksum and whether the order
+// was given up (more than cap rows, or a bucket too full; nothing usable is written then).
+constexpr int ORD_KW = 4, ORD_MAX = 16384, ORD_BUCKET = 1024;  // words of a key, buckets, rows of one
+constexpr uint8_t ORD_NONE = 255;
+struct OrderWork {
+  uint32_t count[ORD_MAX];           // zero between calls
+  uint32_t start[ORD_MAX + 1];
+};
+struct OrderArgs {
+  const int32_t *rows;
+  const float *sc;                   // nullable
+  int64_t n;                         // rows, unless n_dev says it
+  const unsigned long long *n_dev;
+  int64_t cap;                       // rows key, num, idx, out and outs have room for
+  int32_t w, packed;                 // packed: columns held in the key
+  const uint2 *adj4;                 // neighbour lists of the data graph, for columns with ref
+  int32_t radix_id, radix_place;     // of a column's id, and of its place among an earlier one's neighbours
+  unsigned long long range, scale;   // the first word is below range; times scale, its fraction of 2^64
+  uint8_t ref[dmi::MAXW];            // an earlier column that is a pattern neighbour, or ORD_NONE
+  uint8_t word[dmi::MAXW];
+  OrderWork *work;
+  unsigned long long *key;           // kw x cap
+  int32_t *num, *idx;                // row -> its number in its bucket; place -> row
+  int32_t *out;
+  float *outs;
+  unsigned long long *ctr;
+};
+int64_t order_work_bytes();
+int order_layout(OrderArgs &a, unsigned radix_id, unsigned radix_place);  // returns kw
+cudaError_t order_rows(const OrderArgs &a, int kw, int num_sms, cudaStream_t s);
 
 // The min(k, n) best rows of a table by (score, row), k <= SEL_K (select.cu). out: the number of rows
 // collected on the way (4 bytes, padded to 16; above SEL_CAP nothing else was written and the caller

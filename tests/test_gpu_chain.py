@@ -92,6 +92,33 @@ def test_every_form_equals_the_oracle(ctx, B, name):
             assert stats["rows"] == other["rows"] and stats["candidates"] == other["candidates"], (name, p.name, motifs)
 
 
+def scrambled(p, seed):
+    """p with its vertices renumbered: columns far from their pattern neighbours."""
+    return I.relabel(p, np.random.RandomState(seed).permutation(p.n))
+
+
+@pytest.mark.parametrize("graph,pattern", [
+    ((9, 9), scrambled(I.path(20), 1)),     # too many rows share their leading columns: sorted another way
+    ((13, 13), scrambled(I.path(12), 2)),   # keys of several words
+    ((13, 13), I.path(13)),                 # one word
+    ((10, 10), I.sub_patch(I.heavy_hex(10, 10), 30, 4)),
+    ((25, 34), scrambled(I.path(9), 3)),
+    ((2, 2), I.path(2)),
+])
+def test_order_of_rows(ctx, B, graph, pattern):
+    g = I.lognormal_weights(I.heavy_hex(*graph), 3)
+    plan = ctx.plan(ctx.load(g), pattern)
+    rows, scores, count, checksum = plan.all()
+    ref = oracle.enumerate(g, pattern, threads=8)
+    assert (count, checksum) == (ref.count, ref.checksum) and np.array_equal(rows, ref.rows)
+    # at most 29 FP32 additions of non-negative terms: relative error below 30 * 2^-24 < 2e-6
+    np.testing.assert_allclose(scores, oracle.scores(g, pattern, ref.rows), rtol=2e-6, atol=0)
+    top_rows, top, cnt, cs = B.dm_match_topk(ctx.h, plan.h, B.DM_ALL, None, 50, pattern.n)
+    assert (cnt, cs) == (ref.count, ref.checksum)
+    order = np.lexsort((np.arange(len(scores)), scores))[:50]
+    assert np.array_equal(top_rows, rows[order]) and np.array_equal(top, scores[order])
+
+
 @pytest.mark.parametrize("weights", ["lognormal", "equal", "two", "negative"])
 @pytest.mark.parametrize("k", [1, 10, 1000, 1024, 1025])
 def test_best_rows(ctx, weights, k):
