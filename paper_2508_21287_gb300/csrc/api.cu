@@ -3530,12 +3530,48 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   }
   std::vector<float> xn;
   normalise(c, feats, n, xn);
-  const int64_t P = dmk::mlp_param_count();
+  // everything the steps read is uploaded once; losses and the timeout flag come back in the end
+  const int64_t per_epoch = (n + (int64_t)batch - 1) / batch, n_steps = per_epoch * epochs;
+  if (n_steps > (int64_t)1 << 28) return DM_E_CAPACITY;
+  float *X = nullptr, *T = nullptr, *L = nullptr;
+  int32_t *I = nullptr;
+  unsigned *E = nullptr;
+  void *work = nullptr;
+  auto release = [&](int r) {
+    dfree(c, X);
+    dfree(c, T);
+    dfree(c, L);
+    dfree(c, I);
+    dfree(c, E);
+    dfree(c, work);
+    return r;
+  };
+  const int rows = std::min(batch, n);
+  int r = dalloc_t(c, &X, (size_t)n * NFEAT);
+  if (r == DM_OK) r = dalloc_t(c, &T, n);
+  if (r == DM_OK) r = dalloc_t(c, &L, (size_t)n_steps);
+  if (r == DM_OK) r = dalloc_t(c, &I, n);
+  if (r == DM_OK) r = dalloc_t(c, &E, 1);
+  if (r == DM_OK) r = dalloc(c, &work, (size_t)dmk::mlp_train_bytes(rows));
+  if (r != DM_OK) return release(r);
+  dmk::MlpTrain A{};
+  A.params = c->m_params;
+  A.m = c->m_m;
+  A.v = c->m_v;
+  A.X = X;
+  A.target = T;
+  A.err = E;
+  dmk::mlp_train_layout(A, work, rows);
+  auto check = [&](cudaError_t e) { return e == cudaSuccess ? DM_OK : cuda_fail(c, e, "model training"); };
+  r = check(cudaMemcpyAsync(X, xn.data(), sizeof(float) * xn.size(), cudaMemcpyHostToDevice, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(T, targets, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
+  if (r == DM_OK) r = check(cudaMemsetAsync(L, 0, sizeof(float) * n_steps, c->stream));
+  if (r == DM_OK) r = check(cudaMemsetAsync(E, 0, sizeof(unsigned), c->stream));
   std::vector<int32_t> idx(n);
   for (int32_t i = 0; i < n; i++) idx[i] = i;
   uint64_t st = seed ^ 0xA5A5A5A5ull;
-  std::vector<float> bx, bt;
-  for (int32_t ep = 0; ep < epochs; ep++) {
+  int64_t step = 0;
+  for (int32_t ep = 0; ep < epochs && r == DM_OK; ep++) {
     for (int32_t i = n - 1; i > 0; i--) {  // Fisher-Yates with SplitMix64
       st += 0x9E3779B97F4A7C15ull;
       uint64_t z = st;
@@ -3544,25 +3580,30 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
       z ^= z >> 31;
       std::swap(idx[i], idx[(int32_t)(z % (uint64_t)(i + 1))]);
     }
-    double ep_loss = 0;
-    for (int32_t b0 = 0; b0 < n; b0 += batch) {
-      int32_t m = std::min(batch, n - b0);
-      bx.resize((size_t)m * NFEAT);
-      bt.resize(m);
-      for (int32_t i = 0; i < m; i++) {
-        memcpy(&bx[(size_t)i * NFEAT], &xn[(size_t)idx[b0 + i] * NFEAT], sizeof(float) * NFEAT);
-        bt[i] = targets[idx[b0 + i]];
-      }
-      float loss = 0;
-      CK(cudaMemsetAsync(c->m_grads, 0, sizeof(float) * P, c->stream));
-      RET(model_run(c, bx.data(), bt.data(), m, nullptr, c->m_grads, &loss));
+    r = check(cudaMemcpyAsync(I, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream));
+    for (int32_t b0 = 0; b0 < n && r == DM_OK; b0 += batch) {
       c->m_step++;
-      CK(dmk::mlp_adam(c->m_params, c->m_grads, c->m_m, c->m_v, P, lr, c->m_step, c->stream));
-      ep_loss += (double)loss * m;
+      r = check(dmk::mlp_train_step(A, I + b0, std::min(batch, n - b0), L + step++, lr, c->m_step, c->stream));
     }
-    if (out_loss) out_loss[ep] = (float)(ep_loss / n);
   }
-  CK(cudaStreamSynchronize(c->stream));
+  std::vector<float> losses((size_t)n_steps);
+  unsigned timed_out = 0;
+  if (r == DM_OK) r = check(cudaMemcpyAsync(losses.data(), L, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(&timed_out, E, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+  const cudaError_t se = cudaStreamSynchronize(c->stream);
+  if (r == DM_OK) r = check(se);
+  release(r);
+  if (r != DM_OK) return r;
+  if (timed_out) {
+    c->last_error = "a tensor-core wait of the cardinality model timed out";
+    return DM_E_TIMEOUT;
+  }
+  for (int32_t ep = 0; ep < epochs && out_loss; ep++) {
+    double sum = 0;
+    for (int64_t k = 0; k < per_epoch; k++)
+      sum += (double)losses[ep * per_epoch + k] * std::min<int64_t>(batch, n - k * batch);
+    out_loss[ep] = (float)(sum / n);
+  }
   c->m_trained = true;
   return DM_OK;
 }

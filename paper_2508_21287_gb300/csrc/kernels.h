@@ -1,6 +1,7 @@
 // Launchers of the library's sm_103a kernels (kernels.cu). All take the stream to run on;
 // none synchronises. Sizes are in elements unless the name says bytes.
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -356,7 +357,17 @@ int64_t mlp_work_bytes(int rows);
 unsigned *mlp_error_flag(void *work, int rows);
 cudaError_t mlp_forward_backward(const float *params, const float *X, const float *target, int rows, int n_valid,
                                  float *y, float *grads, float *loss, void *work, cudaStream_t s);
-cudaError_t mlp_adam(float *params, const float *grads, float *m, float *v, int64_t n, float lr, int step,
-                     cudaStream_t s);
+// Training (mlp.cu): one Adam step on m samples (rows idx[0 .. m) of X and target) in two launches. The
+// launches before must be this stream's kernels or copies. err is raised as mlp_error_flag is; *loss is added to.
+struct MlpTrain {
+  float *params, *m, *v;
+  const float *X, *target;   // standardised samples, n x 32, and their targets
+  __nv_bfloat16 *Xb, *H1, *H2, *dH2, *dH1;
+  float *dy;
+  unsigned *err;
+};
+int64_t mlp_train_bytes(int batch);
+void mlp_train_layout(MlpTrain &T, void *work, int batch);  // places the buffers of a batch in work
+cudaError_t mlp_train_step(const MlpTrain &T, const int32_t *idx, int m, float *loss, float lr, int step, cudaStream_t s);
 
 }  // namespace dmk

@@ -12,6 +12,7 @@
 
 #include <atomic>
 
+#include "join_device.cuh"
 #include "kernels.h"
 
 namespace dmk {
@@ -321,16 +322,408 @@ __global__ void k_colsum(const __nv_bfloat16 *dH, int rows, int cols, float *db)
   if (threadIdx.x < 32 && c < cols) db[c] += t;
 }
 
-__global__ void k_adam(float *w, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float gi = g[i];
-    float mi = b1 * m[i] + (1.f - b1) * gi;
-    float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// ------------------------------------------------------------------ training step ------
+// One training step in two launches. k_train_rows: a block per 128 samples runs them forward and back
+// to the gradients of the hidden layers, its activations in shared memory and its three products in
+// tensor memory; only what the weight gradients need (the rounded activations and their gradients) goes
+// to device memory. k_train_weights: a block per 32 columns of the weight gradients (or of a bias or
+// output-layer sum) adds over the samples and applies Adam to its own parameters.
+//
+// A step is a chain of small dependent products and nothing else, so it costs what it waits: as fifteen
+// launches with an upload, five allocations and a synchronisation of its own it took 170 us (256
+// samples), as these two launches behind one another 38 us. Products and sums run in the order of
+// mlp_forward_backward, so a step's gradients are the bits that dm_model_grad returns.
+constexpr int TR_THREADS = 512, TR_M = 128;
+
+// Offset (in elements) of (r, k) in an operand of KC columns in the canonical layout (tc_core_off).
+template <int KC>
+__device__ __forceinline__ int tr_off(int r, int k) {
+  return (((r >> 3) * (KC >> 3) + (k >> 3)) << 6) + ((r & 7) << 3) + (k & 7);
+}
+
+// K / 16 MMAs of a staged product, and the arrival of their completion at the barrier.
+template <int KA, int KB>
+__device__ __forceinline__ void tr_mma(uint32_t tmem, const uint16_t *A, const uint16_t *Bt, int N, int K, bool first,
+                                       uint32_t bar) {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  for (int kk = 0; kk < K; kk += 16) {
+    const uint64_t ad = tc_sdesc(tc_saddr(A) + (kk >> 3) * 128, 128, (KA >> 3) * 128);
+    const uint64_t bd = tc_sdesc(tc_saddr(Bt) + (kk >> 3) * 128, 128, (KB >> 3) * 128);
+    const uint32_t acc = !first || kk > 0;
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
+        "l"(ad), "l"(bd), "r"(tc_idesc(N)), "r"(acc)
+        : "memory");
   }
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// 32 columns of this thread's accumulator row.
+__device__ __forceinline__ void tr_ld32(uint32_t addr, uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
+        "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+        "=r"(v[30]), "=r"(v[31])
+      : "r"(addr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t tr_pack(float lo, float hi) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
+}
+
+struct TrainSmemA {
+  uint16_t x[TR_M * 32], w1[MLP_H * 32];              // K = 32
+  uint16_t h1[TR_M * MLP_H], w2[MLP_H * MLP_H];       // K = 128
+  uint16_t d2[TR_M * MLP_H], w2t[MLP_H * MLP_H];      // K = 128
+  uint16_t h2[TR_M * (MLP_H + 8)];                    // row-major, padded
+  float w3[MLP_H], dy[TR_M];
+  unsigned long long bar;
+  uint32_t tmem;
+};
+
+// Block-wide wait for the MMAs committed to the barrier; false (and *err raised) when it ran out.
+__device__ __forceinline__ bool tr_wait(uint32_t bar, uint32_t &phase, unsigned *err) {
+  const bool landed = tc_wait(bar, phase);
+  phase ^= 1u;
+  const bool ok = __syncthreads_and(landed);
+  if (!ok) {
+    if (threadIdx.x == 0) atomicOr(err, 1u);
+    tc_wait(bar, phase ^ 1u);  // let them finish (bounded) before the memory is freed
+  }
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  return ok;
+}
+
+__device__ __forceinline__ void tr_setup(unsigned long long *bar, uint32_t *tmem, int cols) {
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_saddr(tmem)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_saddr(bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+__device__ __forceinline__ void tr_teardown(unsigned long long *bar, uint32_t tmem, int cols) {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+  if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc_saddr(bar)) : "memory");
+}
+
+__global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, const int32_t *idx, int m, float *loss) {
+  extern __shared__ __align__(1024) unsigned char tr_smem[];
+  TrainSmemA &S = *(TrainSmemA *)tr_smem;
+  constexpr int COLS = 512;  // three accumulators of 128 columns (allocations are powers of two)
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rows = (m + 15) / 16 * 16, m0 = blockIdx.x * TR_M;
+  const float *W1 = T.params, *b1 = W1 + MLP_H * MLP_IN, *W2 = b1 + MLP_H, *b2 = W2 + MLP_H * MLP_H;
+  const float *w3 = b2 + MLP_H, *b3 = w3 + MLP_H;
+  tr_setup(&S.bar, &S.tmem, COLS);
+  const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar);
+  uint32_t phase = 0;
+  // the samples do not depend on the launch before; the parameters do
+  for (int i = tid; i < TR_M * 4; i += TR_THREADS) {  // eight inputs of a row
+    const int r = i >> 2, k = (i & 3) * 8;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (m0 + r < m) {
+      const float4 *x = (const float4 *)(T.X + (int64_t)__ldg(idx + m0 + r) * MLP_IN + k);
+      const float4 p = __ldg(x), q = __ldg(x + 1);
+      v = make_uint4(tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w));
+    }
+    *(uint4 *)(S.x + tr_off<32>(r, k)) = v;
+  }
+  griddep_wait();
+  griddep_launch_dependents();
+  for (int i = tid; i < TR_M * 4; i += TR_THREADS) {  // kept for the weights of the first layer
+    const int r = i >> 2, k = (i & 3) * 8;
+    if (m0 + r < rows) *(uint4 *)(T.Xb + (int64_t)(m0 + r) * MLP_IN + k) = *(const uint4 *)(S.x + tr_off<32>(r, k));
+  }
+  for (int i = tid; i < MLP_H * MLP_IN / 8; i += TR_THREADS) {
+    const int n = i >> 2, k = (i & 3) * 8;
+    const float4 *w = (const float4 *)(W1 + n * MLP_IN + k);
+    const float4 p = w[0], q = w[1];
+    *(uint4 *)(S.w1 + tr_off<32>(n, k)) = make_uint4(tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w));
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  if (tid == 0) tr_mma<32, 32>(tmem, S.x, S.w1, MLP_H, MLP_IN, true, bar);
+  for (int i = tid; i < MLP_H * MLP_H / 8; i += TR_THREADS) {  // meanwhile: the second layer, both ways
+    const int n = i >> 4, k = (i & 15) * 8;
+    const float *w = W2 + n * MLP_H + k;  // W2 starts 4224 floats into the parameters: 16-byte aligned
+    const float4 p = *(const float4 *)w, q = *(const float4 *)(w + 4);
+    const uint32_t h[4] = {tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w)};
+    *(uint4 *)(S.w2 + tr_off<MLP_H>(n, k)) = make_uint4(h[0], h[1], h[2], h[3]);
+#pragma unroll
+    for (int j = 0; j < 8; j++) S.w2t[tr_off<MLP_H>(k + j, n)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
+  }
+  if (tid < MLP_H) S.w3[tid] = w3[tid];
+  const int quad = warp & 3, c0 = 32 * (warp >> 2);  // a warp reads its lane quadrant (warp % 4)
+  const int r = 32 * quad + lane;                    // this thread's row: columns c0 .. c0 + 31
+  const bool live = m0 + r < rows;
+  const uint32_t mine = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+  uint32_t v[32], on1 = 0, on2 = 0;  // signs of the pre-activations: the ReLU masks
+  bool ok = tr_wait(bar, phase, T.err);
+  if (ok) {
+    tr_ld32(mine, v);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      uint32_t h[4];
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        const int c = 8 * q + j;
+        const float z = __uint_as_float(v[c]) + __ldg(b1 + c0 + c);
+        on1 |= (uint32_t)(z > 0.f) << c;
+        v[c] = __float_as_uint(z > 0.f ? z : 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) h[j] = tr_pack(__uint_as_float(v[8 * q + 2 * j]), __uint_as_float(v[8 * q + 2 * j + 1]));
+      const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
+      *(uint4 *)(S.h1 + tr_off<MLP_H>(r, c0 + 8 * q)) = x;
+      if (live) *(uint4 *)(T.H1 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) tr_mma<MLP_H, MLP_H>(tmem + 128, S.h1, S.w2, MLP_H, MLP_H, true, bar);
+    ok = tr_wait(bar, phase, T.err);
+  }
+  if (ok) {
+    tr_ld32(mine + 128, v);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      uint32_t h[4];
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        const int c = 8 * q + j;
+        const float z = __uint_as_float(v[c]) + __ldg(b2 + c0 + c);
+        on2 |= (uint32_t)(z > 0.f) << c;
+        v[c] = __float_as_uint(z > 0.f ? z : 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; j++) h[j] = tr_pack(__uint_as_float(v[8 * q + 2 * j]), __uint_as_float(v[8 * q + 2 * j + 1]));
+      const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
+      *(uint4 *)(S.h2 + r * (MLP_H + 8) + c0 + 8 * q) = x;
+      if (live) *(uint4 *)(T.H2 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+    }
+    __syncthreads();
+    for (int x = warp; x < TR_M; x += TR_THREADS / 32) {  // the output layer: a warp a row (as k_out_layer)
+      float s = 0.f;
+      for (int o = lane; o < MLP_H; o += 32)
+        s += __bfloat162float(__ushort_as_bfloat16(S.h2[x * (MLP_H + 8) + o])) * S.w3[o];
+      for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+      if (lane == 0) {
+        const float y = s + b3[0];
+        const float e = m0 + x < m ? y - __ldg(T.target + __ldg(idx + m0 + x)) : 0.f;
+        const float d = 2.f * e / (float)m;
+        S.dy[x] = d;
+        if (m0 + x < rows) T.dy[m0 + x] = d;
+        if (m0 + x < m) atomicAdd(loss, e * e / (float)m);
+      }
+    }
+    __syncthreads();
+    const float d = S.dy[r];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      uint32_t h[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int c = 8 * q + 2 * j;
+        h[j] = tr_pack((on2 >> c) & 1u ? d * S.w3[c0 + c] : 0.f, (on2 >> (c + 1)) & 1u ? d * S.w3[c0 + c + 1] : 0.f);
+      }
+      const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
+      *(uint4 *)(S.d2 + tr_off<MLP_H>(r, c0 + 8 * q)) = x;
+      if (live) *(uint4 *)(T.dH2 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) tr_mma<MLP_H, MLP_H>(tmem + 256, S.d2, S.w2t, MLP_H, MLP_H, true, bar);
+    ok = tr_wait(bar, phase, T.err);
+  }
+  if (ok) {
+    tr_ld32(mine + 256, v);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      uint32_t h[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int c = 8 * q + 2 * j;
+        h[j] = tr_pack((on1 >> c) & 1u ? __uint_as_float(v[c]) : 0.f, (on1 >> (c + 1)) & 1u ? __uint_as_float(v[c + 1]) : 0.f);
+      }
+      if (live) *(uint4 *)(T.dH1 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = make_uint4(h[0], h[1], h[2], h[3]);
+    }
+  }
+  tr_teardown(&S.bar, tmem, COLS);
+}
+
+__device__ __forceinline__ void adam_one(float *w, float gi, float *m, float *v, float lr, float b1, float b2, float eps,
+                                         float c1, float c2) {
+  const float mi = b1 * *m + (1.f - b1) * gi;
+  const float vi = b2 * *v + (1.f - b2) * gi * gi;
+  *m = mi;
+  *v = vi;
+  *w -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+constexpr int TR_KC = 256;
+struct TrainSmemB {
+  uint16_t a[MLP_H * TR_KC], b[32 * TR_KC];  // gradient rows (transposed) and inputs of up to 256 samples
+  float g[MLP_H * 33];                       // the block's gradient
+  float part[256];
+  unsigned long long bar;
+  uint32_t tmem;
+};
+
+// Blocks 0 .. 3: columns 32 b .. of gW2; 4: gW1; then 4 blocks each for b1's, b2's and w3's gradients (32
+// columns a block), the first of the last four b3's too.
+constexpr int TR_BLOCKS = 17;
+__global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain T, int m, float lr, float c1, float c2) {
+  extern __shared__ __align__(1024) unsigned char tr_smem[];
+  TrainSmemB &S = *(TrainSmemB *)tr_smem;
+  const float be1 = 0.9f, be2 = 0.999f, eps = 1e-8f;
+  const int tid = threadIdx.x, b = blockIdx.x, rows = (m + 15) / 16 * 16;
+  const int oW1 = 0, ob1 = MLP_H * MLP_IN, oW2 = ob1 + MLP_H, ob2 = oW2 + MLP_H * MLP_H, ow3 = ob2 + MLP_H, ob3 = ow3 + MLP_H;
+  auto adam = [&](int at, float g) { adam_one(T.params + at, g, T.m + at, T.v + at, lr, be1, be2, eps, c1, c2); };
+  if (b >= 5) {
+    griddep_wait();
+    griddep_launch_dependents();
+    const int what = (b - 5) >> 2, c = 32 * ((b - 5) & 3) + (tid & 31);
+    const bool sums = tid < 256;  // colsum32's eight warps; all threads take its barriers
+    float t = 0.f, u = 0.f;
+    auto add = [&](const __nv_bfloat16 *M, const float *wrow) {
+      float s = 0.f;
+      if (sums)
+        for (int r = tid >> 5; r < rows; r += 8) {
+          const float x = __bfloat162float(M[(int64_t)r * MLP_H + c]);
+          s += wrow ? wrow[r] * x : x;
+        }
+      if (sums) S.part[tid] = s;
+      __syncthreads();
+      float z = 0.f;
+      if (tid < 32)
+        for (int k = 0; k < 8; k++) z += S.part[k * 32 + tid];
+      __syncthreads();
+      return z;
+    };
+    if (what == 0) t = add(T.dH1, nullptr);
+    else if (what == 1) t = add(T.dH2, nullptr);
+    else t = add(T.H2, T.dy);
+    if (b == 13) {  // the column sum of dy, as colsum32 on a matrix of one column
+      float s = 0.f;
+      if (sums && (tid & 31) == 0)
+        for (int r = tid >> 5; r < rows; r += 8) s += T.dy[r];
+      if (sums) S.part[tid] = s;
+      __syncthreads();
+      if (tid == 0) {
+        for (int k = 0; k < 8; k++) u += S.part[k * 32];
+        adam(ob3, u);
+      }
+    }
+    if (tid < 32) adam((what == 0 ? ob1 : what == 1 ? ob2 : ow3) + c, t);
+    return;
+  }
+  constexpr int COLS = 32;
+  tr_setup(&S.bar, &S.tmem, COLS);
+  const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar);
+  griddep_wait();
+  griddep_launch_dependents();
+  // g[o][n] = sum over samples of dH[r][o] * In[r][n]
+  const __nv_bfloat16 *dH = b < 4 ? T.dH2 : T.dH1, *In = b < 4 ? T.H1 + 32 * b : (const __nv_bfloat16 *)T.Xb;
+  const int ldi = b < 4 ? MLP_H : MLP_IN;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int k0 = 0; k0 < rows && ok; k0 += TR_KC) {
+    const int kc = min(TR_KC, rows - k0);  // a multiple of 16
+    for (int i = tid; i < kc * (MLP_H >> 3); i += TR_THREADS) {  // neighbouring threads: neighbouring samples
+      const int o = (i / kc) << 3, k = i % kc;
+      const uint4 x = *(const uint4 *)(dH + (int64_t)(k0 + k) * MLP_H + o);
+      const uint32_t h[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 8; j++) S.a[tr_off<TR_KC>(o + j, k)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
+    }
+    for (int i = tid; i < kc * 4; i += TR_THREADS) {
+      const int n = (i / kc) << 3, k = i % kc;
+      const uint4 x = *(const uint4 *)(In + (int64_t)(k0 + k) * ldi + n);
+      const uint32_t h[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 8; j++) S.b[tr_off<TR_KC>(n + j, k)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) tr_mma<TR_KC, TR_KC>(tmem, S.a, S.b, 32, kc, k0 == 0, bar);
+    ok = tr_wait(bar, phase, T.err);
+  }
+  if (ok) {
+    if (tid < 128) {
+      uint32_t v[32];
+      const int row = tid;  // warps 0 .. 3 read their lane quadrants
+      tr_ld32(tmem + ((uint32_t)(32 * (tid >> 5)) << 16), v);
+#pragma unroll
+      for (int j = 0; j < 32; j++) S.g[row * 33 + j] = __uint_as_float(v[j]);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    for (int i = tid; i < MLP_H * 32; i += TR_THREADS) {
+      const int o = i >> 5, n = i & 31;
+      adam(b < 4 ? oW2 + o * MLP_H + 32 * b + n : oW1 + o * MLP_IN + n, S.g[o * 33 + n]);
+    }
+  }
+  tr_teardown(&S.bar, tmem, COLS);
+}
+
+int64_t mlp_train_bytes(int batch) {
+  const int64_t r = (batch + 15) / 16 * 16;
+  return r * MLP_IN * 2 + 4 * r * MLP_H * 2 + r * 4 + 6 * 256;
+}
+
+void mlp_train_layout(MlpTrain &T, void *work, int batch) {
+  const int64_t r = (batch + 15) / 16 * 16;
+  unsigned char *p = (unsigned char *)work;
+  auto take = [&](int64_t bytes) {
+    void *q = p;
+    p += (bytes + 255) / 256 * 256;
+    return (__nv_bfloat16 *)q;
+  };
+  T.Xb = take(r * MLP_IN * 2);
+  T.H1 = take(r * MLP_H * 2);
+  T.H2 = take(r * MLP_H * 2);
+  T.dH2 = take(r * MLP_H * 2);
+  T.dH1 = take(r * MLP_H * 2);
+  T.dy = (float *)take(r * 4);
+}
+
+cudaError_t mlp_train_step(const MlpTrain &T, const int32_t *idx, int m, float *loss, float lr, int step, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr_set{0};  // one bit per device ordinal below 64
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+  if (!bit || !(attr_set.load() & bit)) {
+    cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmemA));
+    cudaFuncSetAttribute(k_train_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmemB));
+    attr_set.fetch_or(bit);
+  }
+  const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
+  cudaError_t e = launch_pdl(k_train_rows, dim3((m + TR_M - 1) / TR_M), dim3(TR_THREADS), sizeof(TrainSmemA), s, T, idx, m,
+                             loss);
+  if (e == cudaSuccess)
+    e = launch_pdl(k_train_weights, dim3(TR_BLOCKS), dim3(TR_THREADS), sizeof(TrainSmemB), s, T, m, lr, c1, c2);
+  g_launches += 2;
+  return e;
 }
 
 static int blocks_for(int64_t n, int per = 256) {
@@ -426,15 +819,6 @@ cudaError_t mlp_forward_backward(const float *params, const float *X, const floa
     if (e != cudaSuccess) return e;
   }
   g_launches += launches;
-  return cudaGetLastError();
-}
-
-cudaError_t mlp_adam(float *params, const float *grads, float *m, float *v, int64_t n, float lr, int step,
-                     cudaStream_t s) {
-  const float b1 = 0.9f, b2 = 0.999f;
-  float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  g_launches++;
-  k_adam<<<blocks_for(n), 256, 0, s>>>(params, grads, m, v, n, lr, b1, b2, 1e-8f, c1, c2);
   return cudaGetLastError();
 }
 
