@@ -2031,6 +2031,8 @@ struct BatchState {
   dmk::BatchParams prm{};
   int grid = 0;
   void *d_args = nullptr, *d_plans = nullptr, *d_items = nullptr, *d_work = nullptr, *scratch = nullptr;
+  void *d_wide = nullptr, *d_sig = nullptr, *d_sigs = nullptr;  // wide plans: items, id bitmaps, each step's own
+  int launches = 0;                   // kernel launches of one replay of the graph
   unsigned long long *h_out = nullptr;
   int32_t n_plans = 0;
   cudaGraph_t graph = nullptr;
@@ -2050,13 +2052,16 @@ void batch_release(dm_ctx *c, BatchState *b) {
   cudaFree(b->d_items);
   cudaFree(b->d_work);
   cudaFree(b->d_left0);
+  cudaFree(b->d_wide);
+  cudaFree(b->d_sig);
+  cudaFree(b->d_sigs);
   cudaFree(b->scratch);
   if (b->h_out) cudaFreeHost(b->h_out);
   delete b;
 }
 
 int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n, int TR, int64_t root_chunk,
-                double heavy_rows, int threads, int ctas_per_sm, BatchState **out);
+                double heavy_rows, int threads, int ctas_per_sm, BatchState **out, bool bitmaps = true);
 
 DevGraph *get_graph(dm_ctx *c, dm_graph g) {
   if (!c || g < 0 || g >= (int)c->graphs.size()) return nullptr;
@@ -2064,7 +2069,7 @@ DevGraph *get_graph(dm_ctx *c, dm_graph g) {
 }
 
 int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n, int TR, int64_t root_chunk,
-                double heavy_rows, int threads, int ctas_per_sm, BatchState **out) {
+                double heavy_rows, int threads, int ctas_per_sm, BatchState **out, bool bitmaps) {
   std::unique_ptr<BatchState> b(new BatchState());
   b->key.assign(plans, plans + n);
   b->hash_lf = c->hash_lf;
@@ -2079,7 +2084,13 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
   std::vector<uint64_t> items_per(n, 0);
   std::vector<JoinArgs> args;
   std::vector<dmk::BatchPlan> bplans(n);
-  std::vector<std::pair<double, dmk::BatchItem>> items;
+  std::vector<std::pair<double, dmk::BatchItem>> items, wide_items;
+  // motif tables of the wide plans -> first word of their id bitmaps
+  std::map<const int32_t *, int64_t> sig_at;
+  std::vector<dmi::IndexView> sig_tabs;
+  const int sig_units = (g->V + 255) / 256;
+  int64_t sig_words = 0;
+  bitmaps = bitmaps && walk && sig_units <= dmk::BATCH_SIG_UNITS;
   std::vector<int64_t> cap(MAXSTEPS, 0), maxw(MAXSTEPS, 0);
   int ws_max = 1, max_steps = 1;
   bool wide = false;  // some step maps more than 4 new vertices
@@ -2099,8 +2110,8 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
     const int S = (int)ex.st.size();
     bplans[i].n_steps = S;
     bplans[i].args_off = (int32_t)args.size();
-    max_steps = std::max(max_steps, S);
     double cost = 0;
+    for (int j = 0; j < S; j++) cost += ex.p->steps[j].est_rows;
     for (int j = 0; j < S; j++) {
       JoinArgs a = ex.st[j].base;
       a.scored = 0;
@@ -2118,31 +2129,58 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
         if (identity) a.rs_out = (a.wo + 3) / 4 * 4;
       }
       args.push_back(a);
-      ws_max = std::max(ws_max, join_row_stride(a.w));
-      wide |= j > 0 && a.n_new > 4;
-      maxw[j] = std::max<int64_t>(maxw[j], a.rs_out ? a.rs_out : a.wo);
+    }
+    const JoinArgs *pa = args.data() + bplans[i].args_off;
+    bool direct = walk && S > 1 && !pa[0].n_be && !pa[0].induced && pa[0].n_shards <= 1 && pa[0].n_new == pa[0].ix.mw &&
+                  pa[0].wo == pa[0].n_new;
+    for (int q = 0; q < pa[0].wo; q++) direct = direct && pa[0].src_col[q] == q && pa[0].new_mpos[q] == q;
+    bplans[i].seed_direct = direct;
+    // a wide plan: two motif tables met in one step whose only test is the injectivity of more than
+    // 4 new vertices. The bitmaps of all wide plans take at most an eighth of the scratch budget.
+    bool wide_plan = bitmaps && direct && S == 2 && pa[1].n_new > 4 && !pa[1].n_chk && !pa[1].n_be && !pa[1].induced &&
+                     !pa[1].ix.keys && pa[1].ix.nkeys >= 1 && pa[1].w == pa[0].ix.mw;
+    if (wide_plan) {
+      int64_t more = 0;
+      for (int j = 0; j < 2; j++)
+        if (!sig_at.count(pa[j].ix.rows)) more += 8ll * sig_units * pa[j].ix.n;
+      wide_plan = (sig_words + more) * 4 <= (int64_t)(c->budget / 8);
+    }
+    for (int j = 0; wide_plan && j < 2; j++) {
+      if (sig_at.count(pa[j].ix.rows)) continue;
+      sig_at[pa[j].ix.rows] = sig_words;
+      sig_tabs.push_back(pa[j].ix);
+      sig_words += 8ll * sig_units * pa[j].ix.n;
+    }
+    if (!wide_plan) max_steps = std::max(max_steps, S);
+    for (int j = 0; !wide_plan && j < S; j++) {
+      ws_max = std::max(ws_max, join_row_stride(pa[j].w));
+      wide |= j > 0 && pa[j].n_new > 4;
+      maxw[j] = std::max<int64_t>(maxw[j], pa[j].rs_out ? pa[j].rs_out : pa[j].wo);
       if (j > 0) cap[j] = std::max<int64_t>(cap[j], (int64_t)TR * ex.st[j].max_group);
-      cost += ex.p->steps[j].est_rows;
     }
     // root chunks: the tuned size, larger for plans whose first table is so long that the
     // tuned size would cut it into many more items than the GPU has CTAs (per-item overhead)
     int64_t n0 = ex.st[0].seed_table->n;
     const int64_t chunk = std::max<int64_t>(root_chunk, (n0 + 4ll * c->num_sms - 1) / (4ll * c->num_sms));
-    cap[0] = std::max<int64_t>(cap[0], chunk);
+    if (!wide_plan) cap[0] = std::max<int64_t>(cap[0], chunk);
     for (int64_t lo = 0; lo < n0; lo += chunk) {
       dmk::BatchItem it{};
       it.plan = i;
       it.lo = lo;
       it.hi = std::min(n0, lo + chunk);
-      items.push_back({cost / std::max<double>(1.0, (double)(n0 + chunk - 1) / chunk), it});
+      (wide_plan ? wide_items : items).push_back({cost / std::max<double>(1.0, (double)(n0 + chunk - 1) / chunk), it});
       items_per[i]++;
     }
   }
   // expensive chunks first: the tail of the persistent loop is made of cheap ones
-  std::stable_sort(items.begin(), items.end(), [](const std::pair<double, dmk::BatchItem> &x,
-                                                  const std::pair<double, dmk::BatchItem> &y) { return x.first > y.first; });
-  std::vector<dmk::BatchItem> hitems(items.size());
-  for (size_t i = 0; i < items.size(); i++) hitems[i] = items[i].second;
+  auto sorted = [](std::vector<std::pair<double, dmk::BatchItem>> &v) {
+    std::stable_sort(v.begin(), v.end(), [](const std::pair<double, dmk::BatchItem> &x,
+                                            const std::pair<double, dmk::BatchItem> &y) { return x.first > y.first; });
+    std::vector<dmk::BatchItem> h(v.size());
+    for (size_t i = 0; i < v.size(); i++) h[i] = v[i].second;
+    return h;
+  };
+  const std::vector<dmk::BatchItem> hitems = sorted(items), hwide = sorted(wide_items);
   dmk::BatchParams &P = b->prm;
   int64_t off = 0;
   for (int j = 0; j < MAXSTEPS; j++) {
@@ -2182,28 +2220,49 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
   RET(up(&b->d_args, args.data(), sizeof(JoinArgs) * args.size()));
   RET(up(&b->d_plans, bplans.data(), sizeof(dmk::BatchPlan) * bplans.size()));
   RET(up(&b->d_items, hitems.data(), sizeof(dmk::BatchItem) * hitems.size()));
-  // work counter, overflow flag, (count, checksum) per plan, items left per plan, done times,
-  // start time
-  if (cudaMalloc(&b->d_work, sizeof(unsigned long long) * (3 + 4 * (size_t)n)) != cudaSuccess) {
+  if (sig_words) {
+    if (cudaMalloc(&b->d_sig, sizeof(uint32_t) * (size_t)sig_words) != cudaSuccess) {
+      cudaGetLastError();
+      batch_release(c, b.release());
+      return batch_build(c, g, plans, n, TR, root_chunk, heavy_rows, threads, ctas_per_sm, out, false);
+    }
+    uint32_t *sig = (uint32_t *)b->d_sig;
+    for (const dmi::IndexView &ix : sig_tabs)
+      CK(dmk::launch_row_bits(ix.rows, ix.mw, ix.n, sig_units, sig + sig_at[ix.rows], c->stream));
+    std::vector<const uint32_t *> sigs(args.size(), nullptr);
+    for (size_t k = 0; k < args.size(); k++)
+      if (sig_at.count(args[k].ix.rows)) sigs[k] = sig + sig_at[args[k].ix.rows];
+    RET(up(&b->d_sigs, sigs.data(), sizeof(const uint32_t *) * sigs.size()));
+    RET(up(&b->d_wide, hwide.data(), sizeof(dmk::BatchItem) * hwide.size()));
+  }
+  // work counters, overflow flag, (count, checksum) per plan, items left per plan, start time, done
+  // times; the items left and the start time are set before each run
+  if (cudaMalloc(&b->d_work, sizeof(unsigned long long) * (4 + 4 * (size_t)n)) != cudaSuccess) {
     cudaGetLastError();
     return DM_E_NOMEM;
   }
-  RET(up(&b->d_left0, items_per.data(), sizeof(uint64_t) * n));
+  items_per.push_back(~0ull);
+  RET(up(&b->d_left0, items_per.data(), sizeof(uint64_t) * (n + 1)));
   if (cudaMalloc(&b->scratch, std::max<size_t>(16, (size_t)b->grid * slices * P.cta_bytes)) != cudaSuccess) {
     cudaGetLastError();
     return DM_E_NOMEM;
   }
-  if (cudaMallocHost(&b->h_out, sizeof(unsigned long long) * (3 + 4 * (size_t)n)) != cudaSuccess) return DM_E_NOMEM;
+  if (cudaMallocHost(&b->h_out, sizeof(unsigned long long) * (4 + 4 * (size_t)n)) != cudaSuccess) return DM_E_NOMEM;
   unsigned long long *work = (unsigned long long *)b->d_work;
   P.args = (const JoinArgs *)b->d_args;
   P.plans = (const dmk::BatchPlan *)b->d_plans;
   P.items = (const dmk::BatchItem *)b->d_items;
   P.next_item = work;
-  P.ovf = work + 1;
-  P.out = work + 2;
-  P.plan_left = work + 2 + 2 * n;
-  P.plan_done = work + 2 + 3 * n;
-  P.start_ns = work + 2 + 4 * n;
+  P.next_wide = work + 1;
+  P.ovf = work + 2;
+  P.out = work + 3;
+  P.plan_left = work + 3 + 2 * n;
+  P.start_ns = work + 3 + 3 * n;
+  P.plan_done = work + 4 + 3 * n;
+  P.wide = (const dmk::BatchItem *)b->d_wide;
+  P.n_wide = (int64_t)hwide.size();
+  P.sigs = (const uint32_t *const *)b->d_sigs;
+  P.sig_units = sig_units;
   P.scratch = (unsigned char *)b->scratch;
   *out = b.release();
   return DM_OK;
@@ -2213,39 +2272,60 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
 // back. The sequence is captured once into a CUDA graph and replayed afterwards.
 int batch_run(dm_ctx *c, DevGraph *g, BatchState *b) {
   const size_t n = (size_t)b->n_plans;
-  size_t wbytes = sizeof(unsigned long long) * (3 + 4 * n);
+  size_t wbytes = sizeof(unsigned long long) * (4 + 4 * n);
   auto t0 = std::chrono::steady_clock::now();
   c->batch_latency.assign(n, 0.0);
   if (!b->light.empty()) {
     if (!b->exec) {
-      cudaStream_t cs;
+      cudaStream_t cs, ws = nullptr;
+      cudaEvent_t fork = nullptr, join = nullptr;
       CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-      cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+      cudaError_t e = cudaSuccess;
+      if (b->prm.n_wide) {  // the wide plans' kernel on a branch of its own
+        e = cudaStreamCreateWithFlags(&ws, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+      }
+      const long long before = dmk::launch_count();
+      if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long) * (2 + 2 * n), cs);
-        cudaMemcpyAsync((unsigned long long *)b->d_work + 2 + 2 * n, b->d_left0, sizeof(unsigned long long) * n,
+        cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long) * (3 + 2 * n), cs);
+        cudaMemcpyAsync((unsigned long long *)b->d_work + 3 + 2 * n, b->d_left0, sizeof(unsigned long long) * (n + 1),
                         cudaMemcpyDeviceToDevice, cs);
-        if (b->threads == 32) dmk::launch_batch_walk(b->prm, b->grid, cs);
-        else dmk::launch_batch(b->prm, b->grid, b->threads, cs);
+        if (ws) {
+          cudaEventRecord(fork, cs);
+          cudaStreamWaitEvent(ws, fork, 0);
+        }
+        if (b->threads != 32) dmk::launch_batch(b->prm, b->grid, b->threads, cs);
+        else if (b->prm.n_items) dmk::launch_batch_walk(b->prm, b->grid, cs);
+        if (ws) {
+          dmk::launch_batch_wide(b->prm, c->num_sms, ws);
+          cudaEventRecord(join, ws);
+          cudaStreamWaitEvent(cs, join, 0);
+        }
         cudaMemcpyAsync(b->h_out, b->d_work, wbytes, cudaMemcpyDeviceToHost, cs);
         e = cudaStreamEndCapture(cs, &b->graph);
       }
       if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+      b->launches = (int)(dmk::launch_count() - before);
+      if (fork) cudaEventDestroy(fork);
+      if (join) cudaEventDestroy(join);
+      if (ws) cudaStreamDestroy(ws);
       cudaStreamDestroy(cs);
       if (e != cudaSuccess) return cuda_fail(c, e, "batch graph capture");
     } else {
-      dmk::g_launches++;  // the replayed graph holds one launch of the batch kernel
+      dmk::g_launches += b->launches;
     }
     CK(cudaGraphLaunch(b->exec, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    if (b->h_out[1]) {
+    if (b->h_out[2]) {
       c->last_error = "batch level buffer overflow";
       return DM_E_CAPACITY;
     }
     // GPU global-timer offset of each plan's last item from the start of the launch
-    unsigned long long st = b->h_out[2 + 4 * n];
+    unsigned long long st = b->h_out[3 + 3 * n];
     for (int32_t i : b->light) {
-      unsigned long long d = b->h_out[2 + 3 * n + i];
+      unsigned long long d = b->h_out[4 + 3 * n + i];
       c->batch_latency[i] = d > st ? (double)(d - st) * 1e-6 : 0.0;
     }
   }
@@ -2260,8 +2340,8 @@ int batch_run(dm_ctx *c, DevGraph *g, BatchState *b) {
     dm_stats saved = c->stats;
     RET(ex.run());
     c->stats = saved;
-    b->h_out[2 + 2 * i] = ex.count;
-    b->h_out[3 + 2 * i] = ex.checksum;
+    b->h_out[3 + 2 * i] = ex.count;
+    b->h_out[4 + 2 * i] = ex.checksum;
     c->batch_latency[i] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   }
   return DM_OK;
@@ -3185,8 +3265,8 @@ int dm_match_batch(dm_ctx *c, const dm_plan_t *const *plans, int32_t n_plans, in
   }
   RET(batch_run(c, g, b));
   for (int32_t i = 0; i < n_plans; i++) {
-    if (out_counts) out_counts[i] = b->h_out[2 + 2 * i];
-    if (out_checksums) out_checksums[i] = b->h_out[3 + 2 * i];
+    if (out_counts) out_counts[i] = b->h_out[3 + 2 * i];
+    if (out_checksums) out_checksums[i] = b->h_out[4 + 2 * i];
   }
   finish_stats(c, t0);
   return DM_OK;

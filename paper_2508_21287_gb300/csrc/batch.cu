@@ -8,8 +8,8 @@
 // ever waits for another; load balance comes from small root chunks taken in order of the
 // plans' estimated cost. Join, filter, score and compaction are the same device code as the
 // per-step kernel (join_device.cuh). The kernel exists for two block shapes (128 and 256
-// threads); a third shape, one walk per warp, is k_batchw (below). The autotuner picks
-// the shape and how many CTAs run per SM.
+// threads); a third shape, one walk per warp, is k_batchw (below), with k_batch_wide beside it for
+// the plans that meet two large tables. The autotuner picks the shape and how many CTAs run per SM.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -443,19 +443,26 @@ __global__ void __launch_bounds__(BW_BLK, 14) k_batchw(const __grid_constant__ B
   unsigned char *wbase = smem + (size_t)wid * walk_warp_bytes(P.tile_words, P.max_steps);
   const WarpSmem W = walk_warp(wbase, P.tile_words);
   const WalkSmem K = walk_smem(wbase, P.tile_words, P.max_steps);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *P.start_ns = globaltimer_ns();
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicMin(P.start_ns, globaltimer_ns());
   unsigned char *mine = P.scratch + ((int64_t)blockIdx.x * BW_WARPS + wid) * P.cta_bytes;
+  long long next = 0;
+  if (lane == 0) next = (long long)atomicAdd(P.next_item, 1ull);
   while (true) {
-    long long it = 0;
-    if (lane == 0) it = (long long)atomicAdd(P.next_item, 1ull);
-    it = __shfl_sync(FULL_MASK, it, 0);
+    const long long it = __shfl_sync(FULL_MASK, next, 0);
     if (it >= P.n_items) break;
+    if (lane == 0) next = (long long)atomicAdd(P.next_item, 1ull);  // arrives while this item is walked
     const BatchItem item = P.items[it];
     const BatchPlan plan = P.plans[item.plan];
     const int S = plan.n_steps;
     const JoinArgs *args = P.args + plan.args_off;
     unsigned long long ar = 0, as = 0;
-    {  // first step: the item's motif rows are the candidates, 32 at a time
+    if (plan.seed_direct) {  // every motif row is a row of level 0 as it stands: read in place
+      if (lane == 0) {
+        K.n_lvl[0] = (int32_t)(item.hi - item.lo);
+        K.cur[0] = 0;
+      }
+      __syncwarp();
+    } else {  // first step: the item's motif rows are the candidates, 32 at a time
       const JoinArgs &a0 = args[0];
       int32_t *out = (int32_t *)(mine + P.lvl_off[0]);
       int64_t n_out = 0;
@@ -481,8 +488,10 @@ __global__ void __launch_bounds__(BW_BLK, 14) k_batchw(const __grid_constant__ B
       }
       const int j = top + 1;
       const int nr = min(walk_tile_rows(P.tile_words, args[j].w), have - cur);
-      const int rs_in = walk_level_stride(args[top]);
-      const int32_t *src = (const int32_t *)(mine + P.lvl_off[top]) + (int64_t)cur * rs_in;
+      const bool direct = top == 0 && plan.seed_direct;
+      const int rs_in = direct ? args[0].ix.mw : walk_level_stride(args[top]);
+      const int32_t *src = (direct ? args[0].ix.rows + item.lo * rs_in : (const int32_t *)(mine + P.lvl_off[top])) +
+                           (int64_t)cur * rs_in;
       const JoinArgs &a = args[j];
       int64_t n_out = 0;
       if (j == S - 1)
@@ -535,6 +544,227 @@ cudaError_t launch_batch_walk(const BatchParams &p, int grid, cudaStream_t s) {
   cudaFuncSetAttribute(k_batchw, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   g_launches++;
   k_batchw<<<grid, BW_BLK, walk_smem_bytes(p.tile_words, p.max_steps), s>>>(p);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------
+// Plans of two steps that meet two large motif tables (half paths of up to 24 vertices joined at
+// their ends) on graphs of up to 256 * BATCH_SIG_UNITS vertices. Nearly all of a mixed batch's
+// candidates are theirs, three to ten for each row of the first table, and a candidate is decided by
+// injectivity alone: up to 24 x 24 compares. Every row of either table has a bitmap of its ids
+// (k_row_bits), so the test is one AND over 8 x SU words; the tile's bitmaps lie in shared memory
+// (without the ids the two rows share by their keys), the candidates' are read in whole 32-byte
+// sectors. Rows are never copied: survivors are listed as (row, motif row), and eight lanes at a
+// time read both halves of one for its checksum terms -- its two rows lie on a line or two each,
+// where a lane for each survivor would gather over 32.
+// 512 mixed patterns on the heavy-hex 12 x 6 lattice (72 M candidates, 43 M of them here, 14 M first
+// rows): 4.2 ms in walks that read each new vertex and scanned the row for it (3.6 G warp
+// instructions, 14 of 32 lanes active); 3.0 ms with bitmaps set tile by tile within k_batchw; 1.95 ms
+// with the first table read in place instead of written and read back; 1.73 ms with the rows' own
+// bitmaps; 1.42 ms in a kernel of its own (64 registers and no spills, where the walk's many
+// instances kept it at 72 and 28 warps an SM). Bound by latency: 0.49 G warp instructions at 2.0 an
+// SM and clock, the L1 pipe 60 % busy. Reading the next tile's keys ahead, two survivors' passes at
+// once and 80 registers at 24 warps were all within 1 % of this.
+constexpr int WD_WARPS = 4, WD_BLK = 32 * WD_WARPS, WD_STAGE = 64, WD_COLS = (MAXM + 7) / 8;
+
+template <int SU>
+struct WideWarp {
+  uint32_t bits[WT][8 * SU + 4];  // 16 bytes of padding: neighbouring rows on different banks
+  int32_t st_r[WD_STAGE], st_m[WD_STAGE];
+  uint8_t pos[2][8 * WD_COLS];    // 1 + output position of each column, of each new vertex (0: none)
+};
+
+// 32 bytes of a bitmap, read-only path.
+__device__ __forceinline__ void load_bits(const uint32_t *p, uint4 &x, uint4 &y) {
+  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+      : "l"(p));
+}
+
+template <int SU>
+__global__ void __launch_bounds__(WD_BLK, 8) k_batch_wide(const __grid_constant__ BatchParams P) {
+  __shared__ __align__(16) WideWarp<SU> sm[WD_WARPS];
+  constexpr int SW = 8 * SU;
+  const int lane = threadIdx.x & 31, l8 = lane & 7;
+  WideWarp<SU> &W = sm[threadIdx.x >> 5];
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicMin(P.start_ns, globaltimer_ns());
+  long long next = 0;
+  if (lane == 0) next = (long long)atomicAdd(P.next_wide, 1ull);
+  while (true) {
+    const long long it = __shfl_sync(FULL_MASK, next, 0);
+    if (it >= P.n_wide) break;
+    if (lane == 0) next = (long long)atomicAdd(P.next_wide, 1ull);  // arrives while this item is walked
+    const BatchItem item = P.wide[it];
+    const int off = P.plans[item.plan].args_off;
+    const JoinArgs &a = P.args[off + 1];
+    const int w = a.w, wo = a.wo, n_new = a.n_new, mw = a.ix.mw, n = (int)(item.hi - item.lo);
+    const int key0 = a.key_col[0], key1 = a.key_col[1];
+    const bool two = a.ix.nkeys == 2;
+    const int32_t *src = P.args[off].ix.rows + item.lo * w, *mrows = a.ix.rows;
+    const uint32_t *ssig = P.sigs[off] + item.lo * SW, *sig = P.sigs[off + 1];
+    for (int q = lane; q < 16 * WD_COLS; q += 32) W.pos[0][q] = 0;
+    __syncwarp();
+    for (int q = lane; q < wo; q += 32) {
+      const int col = a.src_col[q];
+      (col < w ? W.pos[0][col] : W.pos[1][col - w]) = (uint8_t)(q + 1);
+    }
+    __syncwarp();
+    int mpos[WD_COLS], pos[WD_COLS];  // this lane's columns l8 + 8 k of both halves
+#pragma unroll
+    for (int k = 0; k < WD_COLS; k++) {
+      const int c = l8 + 8 * k;
+      mpos[k] = c < n_new ? a.new_mpos[c] : 0;
+      pos[k] = W.pos[0][c] | W.pos[1][c] << 8;
+    }
+    unsigned long long ar = 0, as = 0;
+    int nst = 0;
+    for (int t = 0; t < n; t += WT) {
+      const int nr = min(WT, n - t);
+      int start = 0, len = 0, k0 = 0, k1 = 0;
+      if (lane < nr) {
+        const int32_t *row = src + (t + lane) * w;
+        k0 = __ldg(row + key0);
+        if (two) k1 = __ldg(row + key1);
+      }
+      const uint4 *s4 = (const uint4 *)(ssig + t * SW);
+      uint4 x[2 * SU];
+#pragma unroll
+      for (int k = 0; k < 2 * SU; k++)
+        if (lane + 32 * k < nr * 2 * SU) x[k] = __ldg(s4 + lane + 32 * k);
+#pragma unroll
+      for (int k = 0; k < 2 * SU; k++) {
+        const int e = lane + 32 * k;
+        if (e < nr * 2 * SU) *(uint4 *)&W.bits[e / (2 * SU)][4 * (e % (2 * SU))] = x[k];
+      }
+      if (lane < nr) ix_lookup(a.ix, k0, k1, start, len);
+      __syncwarp();
+      if (lane < nr) {
+        W.bits[lane][k0 >> 5] &= ~(1u << (k0 & 31));
+        if (two) W.bits[lane][k1 >> 5] &= ~(1u << (k1 & 31));
+      }
+      int incl = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL_MASK, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int C = __shfl_sync(FULL_MASK, incl, 31);
+      const int g_off = incl - len;
+      __syncwarp();
+      const bool last = t + WT >= n;  // one round more if survivors are left over
+      for (int cb = 0; cb < C || (last && nst > 0); cb += 32) {
+        int r, m;
+        round_rows(start, g_off, cb, C, r, m);
+        const uint32_t *sg = sig + (int64_t)m * SW;
+        uint32_t hit = 0;
+#pragma unroll
+        for (int u = 0; u < SU; u++) {
+          uint4 y, z;
+          load_bits(sg + 8 * u, y, z);
+          const uint4 p = *(const uint4 *)&W.bits[r][8 * u], q = *(const uint4 *)&W.bits[r][8 * u + 4];
+          hit |= (y.x & p.x) | (y.y & p.y) | (y.z & p.z) | (y.w & p.w) | (z.x & q.x) | (z.y & q.y) | (z.z & q.z) |
+                 (z.w & q.w);
+        }
+        const bool ok = cb + lane < C && hit == 0;
+        const unsigned bal = __ballot_sync(FULL_MASK, ok);
+        if (ok) {
+          const int at = nst + __popc(bal & lanemask_lt());
+          W.st_r[at] = t + r;
+          W.st_m[at] = m;
+        }
+        nst += __popc(bal);
+        if (nst < 32 && !(last && cb + 32 >= C && nst > 0)) continue;
+        const int m32 = min(nst, 32);
+        __syncwarp();
+        unsigned long long mine = 0;
+#pragma unroll 1
+        for (int p = 0; p < 8; p++) {
+          const int s = 4 * p + (lane >> 3);
+          unsigned long long h = 0;
+          if (s < m32) {
+            const int32_t *rrow = src + W.st_r[s] * w + l8, *trow = mrows + (int64_t)W.st_m[s] * mw;
+            int32_t u[WD_COLS], v[WD_COLS];
+#pragma unroll
+            for (int k = 0; k < WD_COLS; k++) {
+              u[k] = pos[k] & 255 ? __ldg(rrow + 8 * k) : 0;
+              v[k] = pos[k] >> 8 ? __ldg(trow + mpos[k]) : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < WD_COLS; k++) {
+              if (pos[k] & 255) h += pos_term(pos[k] & 255, u[k]);
+              if (pos[k] >> 8) h += pos_term(pos[k] >> 8, v[k]);
+            }
+          }
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) h += __shfl_xor_sync(FULL_MASK, h, o);
+          if (l8 == p) mine = h;
+        }
+        if (4 * l8 + (lane >> 3) < m32) {
+          as += dmix64(mine + (unsigned long long)(uint32_t)wo);
+          ar++;
+        }
+        nst -= m32;
+        const int kr = W.st_r[32 + lane], km = W.st_m[32 + lane];  // the rest, if any, to the front
+        __syncwarp();
+        if (lane < nst) {
+          W.st_r[lane] = kr;
+          W.st_m[lane] = km;
+        }
+        __syncwarp();
+      }
+      __syncwarp();  // the next tile overwrites the bitmaps
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      ar += __shfl_down_sync(FULL_MASK, ar, o);
+      as += __shfl_down_sync(FULL_MASK, as, o);
+    }
+    if (lane == 0) {
+      if (ar) {
+        atomicAdd(P.out + 2 * item.plan, ar);
+        atomicAdd(P.out + 2 * item.plan + 1, as);
+      }
+      __threadfence();
+      if (atomicAdd(P.plan_left + item.plan, ~0ull) == 1ull) P.plan_done[item.plan] = globaltimer_ns();
+    }
+    __syncwarp();
+  }
+}
+
+// The id bitmaps of a motif table: su units of 256 bits a row, bit v set for each id v of the row.
+constexpr int RB_ROWS = 64;
+__global__ void __launch_bounds__(256) k_row_bits(const int32_t *rows, int mw, int64_t n, int su, uint32_t *out) {
+  __shared__ uint32_t b[RB_ROWS * 8 * BATCH_SIG_UNITS];
+  const int64_t r0 = (int64_t)blockIdx.x * RB_ROWS;
+  const int nr = (int)imin64(RB_ROWS, n - r0), nb = nr * su * 8;
+  for (int i = threadIdx.x; i < nb; i += 256) b[i] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < nr * mw; e += 256) {
+    const uint32_t v = (uint32_t)__ldg(rows + r0 * mw + e);
+    atomicOr(b + e / mw * su * 8 + (v >> 5), 1u << (v & 31));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nb; i += 256) out[r0 * su * 8 + i] = b[i];
+}
+
+cudaError_t launch_row_bits(const int32_t *rows, int mw, int64_t n, int su, uint32_t *out, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  g_launches++;
+  k_row_bits<<<(unsigned)((n + RB_ROWS - 1) / RB_ROWS), 256, 0, s>>>(rows, mw, n, su, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_wide(const BatchParams &p, int num_sms, cudaStream_t s) {
+  static_assert(BATCH_SIG_UNITS == 4, "one instance for each width");
+  BatchKernel k = p.sig_units == 1   ? k_batch_wide<1>
+                  : p.sig_units == 2 ? k_batch_wide<2>
+                  : p.sig_units == 3 ? k_batch_wide<3>
+                                     : k_batch_wide<4>;
+  int per_sm = 1;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, WD_BLK, 0);
+  const int64_t full = (int64_t)num_sms * (per_sm < 1 ? 1 : per_sm), need = (p.n_wide + WD_WARPS - 1) / WD_WARPS;
+  g_launches++;
+  k<<<(unsigned)imin64(full, need), WD_BLK, 0, s>>>(p);
   return cudaGetLastError();
 }
 

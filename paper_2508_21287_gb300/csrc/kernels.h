@@ -305,6 +305,8 @@ cudaError_t unique_rows(const int32_t *rows, int64_t n, int32_t w, int32_t *flag
 struct BatchPlan {
   int32_t n_steps;
   int32_t args_off;  // index of the plan's first step in BatchParams::args
+  int32_t seed_direct;  // warp walks: the first step keeps every motif row as it stands (no check, columns
+                        // in table order) and is not the last; the second reads the table
 };
 struct BatchItem {
   int32_t plan;
@@ -332,6 +334,14 @@ struct BatchParams {
   unsigned long long *start_ns;   // GPU global-timer time at the start of the launch
   int max_steps;                  // warp walks: the most steps of a plan (per-warp level state)
   int tile_words;                 // warp walks: words of each walk's shared tile (a multiple of 4)
+  // warp walks: items of plans that k_batch_wide runs (two steps, the second deciding many new vertices
+  // by injectivity alone), and per entry of args the id bitmaps (sig_units x 256 bits a row) of the
+  // motif rows such a plan reads, or null
+  const BatchItem *wide;
+  int64_t n_wide;
+  unsigned long long *next_wide;  // work counter (zeroed before the launch)
+  const uint32_t *const *sigs;
+  int sig_units;
 };
 // threads: 128 or 256 per CTA. batch_grid: SMs x resident CTAs per SM (at most max_per_sm when
 // it is > 0).
@@ -345,6 +355,11 @@ cudaError_t launch_batch(const BatchParams &p, int grid, int threads, cudaStream
 // when it is > 0); BW_WALK_WARPS warps a CTA. BW_WALK_TILE_STRIDE: the row stride (words) that a
 // walk's tile holds 32 rows of.
 constexpr int BW_WALK_WARPS = 2, BW_WALK_TILE_STRIDE = 28;
+// The wide plans of a batch of warp walks, on graphs of up to 256 * BATCH_SIG_UNITS vertices; and the
+// id bitmaps of a motif table (su units of 256 bits a row).
+constexpr int BATCH_SIG_UNITS = 4;
+cudaError_t launch_batch_wide(const BatchParams &p, int num_sms, cudaStream_t s);
+cudaError_t launch_row_bits(const int32_t *rows, int mw, int64_t n, int su, uint32_t *out, cudaStream_t s);
 size_t walk_smem_bytes(int tile_words, int max_steps);
 int walk_grid(int tile_words, int max_steps, int num_sms, int max_per_sm);
 cudaError_t launch_batch_walk(const BatchParams &p, int grid, cudaStream_t s);
