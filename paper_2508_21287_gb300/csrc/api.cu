@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <map>
 #include <set>
@@ -493,13 +494,45 @@ struct StepRT {
 };
 
 // Launches of several steps (chain.cu): shared memory of an SM, warps it holds at most, the most bytes
-// of candidate tables; and what cuts a plan into launches: the cost of a launch (its start, the first
-// loads of every step, the uneven end), of a row at full occupancy (a 24-vertex path on 16 082 vertices:
-// 149 M rows in 2.2 ms), and of a byte of a table between launches.
+// of candidate tables; and what cuts a plan into launches: the cost of a launch (its start behind the
+// one before, the uneven end), of a row at full occupancy (a 24-vertex path on 16 082 vertices: 149 M
+// rows in 2.2 ms; twice that, for the plans whose rows are spread unevenly over the seeds), and of a
+// byte of a table between launches. 27-vertex patch on heavy-hex 16x15: 380 us with 15 us a launch
+// and 0.015 ns a row (one launch of 11 steps), 173 so (three); 38-vertex patch on 6x11 166 and 105.
 constexpr int CHAIN_SM_BYTES = 224 * 1024;
 constexpr int CHAIN_WARPS = 16;
-constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20;
-constexpr double CHAIN_LAUNCH_NS = 15000, CHAIN_ROW_NS = 0.015, CHAIN_BYTE_NS = 0.0002;
+constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20, CHAIN_TAB_MIN = 4ll << 20;
+constexpr double CHAIN_LAUNCH_NS = 4000, CHAIN_ROW_NS = 0.03, CHAIN_BYTE_NS = 0.0002;
+// Rows of work that an item of a launch's input stands for at the least: each further item is a turn
+// at one counter that all warps share. A 7-vertex tree on 2640 vertices (31 656 first rows, 0.25 M
+// embeddings) took 53 us in eight items a warp, 47 without the rounding to whole rows, 36.5 at 32 rows an
+// item, 34.4 at 256; a 6-vertex path on 5000 vertices 43.6, 39.8, 34.6, 34.6; larger counts do not notice.
+constexpr double CHAIN_ITEM_ROWS = 256;
+
+// A set of pattern vertices or columns.
+struct VSet {
+  uint64_t w[MAXW / 64] = {};
+  void add(int i) { w[i >> 6] |= 1ull << (i & 63); }
+  bool has(int i) const { return w[i >> 6] >> (i & 63) & 1; }
+  bool any() const { return (w[0] | w[1]) != 0; }
+  VSet &operator|=(const VSet &o) {
+    w[0] |= o.w[0];
+    w[1] |= o.w[1];
+    return *this;
+  }
+  VSet without(const VSet &o) const {
+    VSet r = *this;
+    r.w[0] &= ~o.w[0];
+    r.w[1] &= ~o.w[1];
+    return r;
+  }
+  template <class F>
+  void each(F f) const {  // in ascending order
+    for (int k = 0; k < 2; k++)
+      for (uint64_t x = w[k]; x; x &= x - 1) f(64 * k + __builtin_ctzll(x));
+  }
+};
+static_assert(MAXW == 128, "two words");
 
 struct Exec {
   dm_ctx *c;
@@ -941,33 +974,32 @@ struct Exec {
     std::vector<int64_t> ids, extra;     // per step: 1 + place of its tables (0: none)
     int64_t tab_bytes = 0;
     bool needs_arena = false;
+    double work = 0;                     // estimated rows of all steps
   };
 
-  // Estimated rows after each step, for the cut into launches only. A new vertex next to a mapped one
+  // Estimated rows after each step, for the cut into launches and into items. A new vertex next to a mapped one
   // with k mapped neighbours finds about D - k places, D the mean degree met along an edge; an edge that
   // closes a cycle is there for about one row in eight (lattices: 1/7 to 1/9 of the rows of a 12-cycle).
-  std::vector<double> chain_rows() const {
-    const int np = p->n_p;
-    std::vector<std::vector<int>> adj(np);
-    std::vector<char> in(np, 0);
+  std::vector<double> chain_rows(const std::vector<const MotifDef *> &motifs) const {
+    int deg[MAXW] = {};
+    char in[MAXW] = {}, used[MAXM * (MAXM - 1) / 2];
     std::vector<double> rows;
     double r = (double)st[0].seed_table->n;
     for (size_t j = 0; j < p->steps.size(); j++) {
       const StepSpec &s = p->steps[j];
-      MotifDef md;
-      motif_def(s.motif, &md);
+      const MotifDef &md = *motifs[j];
       auto join = [&](int a, int b) {
-        adj[a].push_back(b);
-        adj[b].push_back(a);
+        deg[a]++;
+        deg[b]++;
       };
-      std::vector<char> used(md.edges.size(), 0);
+      memset(used, 0, md.edges.size());
       for (bool more = true; more && j;) {  // edges of the motif that reach a new vertex
         more = false;
         for (size_t e = 0; e < md.edges.size(); e++) {
           int a = s.slice[md.edges[e].first], b = s.slice[md.edges[e].second];
           if (used[e] || in[a] == in[b]) continue;
           if (in[b]) std::swap(a, b);
-          r *= std::max(0.3, g->edge_deg - (double)adj[a].size());
+          r *= std::max(0.3, g->edge_deg - (double)deg[a]);
           join(a, b);
           in[b] = 1;
           used[e] = 1;
@@ -1016,56 +1048,64 @@ struct Exec {
 
     // the columns each new vertex is compared with, from the pattern edges enforced up to its step,
     // and the columns each step reads
-    std::vector<std::vector<int>> adj(np);
-    auto enforce = [&](const StepSpec &s) {
-      MotifDef md;
-      motif_def(s.motif, &md);
+    VSet adj[MAXW];
+    std::map<int, MotifDef> defs;
+    std::vector<const MotifDef *> motifs(S);
+    for (int j = 0; j < S; j++) {
+      const auto at = defs.try_emplace(p->steps[j].motif);
+      if (at.second) motif_def(p->steps[j].motif, &at.first->second);
+      motifs[j] = &at.first->second;
+    }
+    auto enforce = [&](int j) {
+      const StepSpec &s = p->steps[j];
       auto add = [&](int a, int b) {
-        adj[a].push_back(b);
-        adj[b].push_back(a);
+        adj[a].add(b);
+        adj[b].add(a);
       };
-      for (auto &e : md.edges) add(s.slice[e.first], s.slice[e.second]);
+      for (auto &e : motifs[j]->edges) add(s.slice[e.first], s.slice[e.second]);
       for (int i = 0; i < s.n_be; i++) add(s.be_vtx[i][0], s.be_vtx[i][1]);
     };
-    enforce(s0);
-    std::vector<std::vector<std::vector<int>>> ck(S);
-    std::vector<std::vector<int>> ex(S);  // one key, one new vertex: mapped pattern neighbours of the key
-    std::vector<std::vector<char>> need(S + 1, std::vector<char>(MAXW, 0));  // by steps >= j
+    enforce(0);
+    std::vector<std::array<VSet, dmk::CH_NEW>> ck(S);
+    std::vector<VSet> ex(S);        // one key, one new vertex: mapped pattern neighbours of the key
+    std::vector<VSet> need(S + 1);  // by steps >= j
     for (int j = 1; j < S; j++) {
       const StepSpec &s = p->steps[j];
-      if (s.n_keys == 1 && s.n_new == 1)
-        for (int v : adj[p->col_vertex[s.key_col[0]]])
-          for (int col = 0; col < s.w_in && ex[j].size() < 2; col++)
-            if (p->col_vertex[col] == v && std::find(ex[j].begin(), ex[j].end(), col) == ex[j].end()) ex[j].push_back(col);
-      enforce(s);
-      ck[j].resize(s.n_new);
+      if (s.n_keys == 1 && s.n_new == 1) {
+        const VSet &by = adj[p->col_vertex[s.key_col[0]]];
+        for (int col = 0, n = 0; col < s.w_in && n < 2; col++)
+          if (by.has(p->col_vertex[col])) {
+            ex[j].add(col);
+            n++;
+          }
+      }
+      enforce(j);
+      VSet slice;
+      for (int m = 0; m < s.k; m++) slice.add(s.slice[m]);
       for (int i = 0; i < s.n_new; i++) {
-        std::vector<int> dist(np, -1), q{(int)s.slice[s.new_mpos[i]]};
-        dist[q[0]] = 0;
-        for (size_t h = 0; h < q.size(); h++)
-          for (int v : adj[q[h]])
-            if (dist[v] < 0) {
-              dist[v] = dist[q[h]] + 1;
-              q.push_back(v);
-            }
+        VSet untested = slice, seen, level;  // vertices by their distance d along the edges
+        level.add(s.slice[s.new_mpos[i]]);
+        for (int d = 0; level.any(); d++) {
+          seen |= level;
+          if (d == 1 || (d > 2 && (d < g->girth || (g->bipartite && (d & 1))))) untested |= level;
+          VSet next;
+          level.each([&](int v) { next |= adj[v]; });
+          level = next.without(seen);
+        }
         for (int col = 0; col < s.w_in; col++) {
-          const int v = p->col_vertex[col], d = dist[v];
-          bool in_slice = false;
-          for (int m = 0; m < s.k; m++) in_slice |= s.slice[m] == v;
-          if (in_slice || d == 1 || (d > 2 && (d < g->girth || (g->bipartite && (d & 1))))) continue;
-          ck[j][i].push_back(col);
-          need[j][col] = 1;
+          if (untested.has(p->col_vertex[col])) continue;
+          ck[j][i].add(col);
+          need[j].add(col);
         }
       }
-      for (int i = 0; i < s.n_keys; i++) need[j][s.key_col[i]] = 1;
+      for (int i = 0; i < s.n_keys; i++) need[j].add(s.key_col[i]);
       for (int i = 0; i < s.n_be; i++)
         for (int h = 0; h < 2; h++)
-          if (s.be_col[i][h] < s.w_in) need[j][s.be_col[i][h]] = 1;
+          if (s.be_col[i][h] < s.w_in) need[j].add(s.be_col[i][h]);
     }
     if (!count_mode)  // every column is handed over in the end
-      for (int col = 0; col < np; col++) need[S][col] = 1;
-    for (int j = S - 1; j >= 1; j--)
-      for (int col = 0; col < np; col++) need[j][col] |= need[j + 1][col];
+      for (int col = 0; col < np; col++) need[S].add(col);
+    for (int j = S - 1; j >= 1; j--) need[j] |= need[j + 1];
 
     // a place in the row for every column: the first free one of its colour class
     std::vector<int> cls(np, -1);
@@ -1073,48 +1113,50 @@ struct Exec {
     if (two) {
       std::vector<int> q{(int)s0.slice[0]};
       cls[q[0]] = 0;
-      for (size_t h = 0; h < q.size(); h++)
-        for (int v : adj[q[h]]) {
+      for (size_t h = 0; h < q.size(); h++) {
+        const int u = q[h];
+        adj[u].each([&](int v) {
           if (cls[v] < 0) {
-            cls[v] = 1 - cls[q[h]];
+            cls[v] = 1 - cls[u];
             q.push_back(v);
-          } else if (cls[v] == cls[q[h]]) {
+          } else if (cls[v] == cls[u]) {
             two = false;  // an odd cycle: no embedding, but the plan runs as any other
           }
-        }
+        });
+      }
     }
     std::vector<int> place(MAXW, -1), nc(S + 1, 0);
-    std::vector<int> held;  // columns that hold a place in the tile of step j
+    std::vector<int> held, keep;  // columns that hold a place in the tile of step j
     auto place_new = [&](int j, int first, int n) {  // columns first .. first + n - 1 enter tile j
-      std::vector<char> used(4 * dmk::CH_CHUNKS, 0);
-      std::vector<int> keep;
+      char used[4 * dmk::CH_CHUNKS] = {};
+      keep.clear();
       for (int col : held)
-        if (need[j][col]) {
+        if (need[j].has(col)) {
           keep.push_back(col);
           used[place[col]] = 1;
         }
       for (int col = first; col < first + n; col++) {
-        if (!need[j][col]) continue;
+        if (!need[j].has(col)) continue;
         int h = 0;
-        while (h < (int)used.size() && (used[h] || (two && ((h >> 2) & 1) != cls[p->col_vertex[col]]))) h++;
-        if (h == (int)used.size()) return false;
+        while (h < (int)sizeof(used) && (used[h] || (two && ((h >> 2) & 1) != cls[p->col_vertex[col]]))) h++;
+        if (h == (int)sizeof(used)) return false;
         place[col] = h;
         used[h] = 1;
         keep.push_back(col);
       }
-      held = keep;
+      held.swap(keep);
       for (int col : held) nc[j] = std::max(nc[j], (place[col] >> 2) + 1);
       if (two) nc[j] = (nc[j] + 1) / 2 * 2;
       return true;
     };
     // place[] of a column is final when it enters, so a step's offsets can be taken afterwards; a
     // column's place is free for the new vertices of the step that reads it last
-    std::vector<std::vector<int>> at(S + 1);  // tile j: place of each column, -1 if not held
+    std::vector<std::array<int8_t, MAXW>> at(S + 1);  // tile j: place of each column, -1 if not held
     for (int j = 1; j <= S; j++) {
       const StepSpec &s = p->steps[j - 1];
       if (!place_new(j, s.w_in, s.n_new)) return false;
-      at[j].assign(MAXW, -1);
-      for (int col : held) at[j][col] = place[col];
+      at[j].fill(-1);
+      for (int col : held) at[j][col] = (int8_t)place[col];
     }
     auto off = [](int h) { return (uint16_t)((h >> 2) * 512 + (h & 3) * 2); };
 
@@ -1126,7 +1168,9 @@ struct Exec {
       for (int j = a; j <= b; j++) t += dmk::chain_tile_bytes(nc[j]);
       return t;
     };
-    const std::vector<double> rows = chain_rows();
+    const std::vector<double> rows = chain_rows(motifs);
+    C.work = 0;
+    for (const double r : rows) C.work += r;
     std::vector<double> cost(S + 1, 1e300);  // steps 1 .. j done, tile j + 1 written
     std::vector<int> from(S + 1, -1);
     cost[0] = 0;
@@ -1205,19 +1249,19 @@ struct Exec {
         for (int x = 0; x < t.n_chk; x++) t.chk_off[x] = off(at[j][s.key_col[a.ix.nkeys + x]]);
         // one key and 1 or 3 new vertices (M2, M4): room for the longest group at every key, and of
         // three new vertices two of one colour class first
-        std::vector<int> ord(s.n_new);
+        int ord[dmk::CH_NEW], rank[dmk::CH_NEW];  // rank: new vertex -> its place in the record
         for (int x = 0; x < s.n_new; x++) ord[x] = x;
         auto cl = [&](int x) { return two ? cls[s.slice[s.new_mpos[x]]] : 0; };
         if (a.ix.nkeys == 1 && t.n_chk == 0 && !(counted && s.n_be) &&
             (s.n_new == 3 || (s.n_new == 1 && st[j].max_group <= 4))) {
           t.group = (int32_t)st[j].max_group;
-          for (int col : ex[j])
+          ex[j].each([&](int col) {
             if (s.k == 2 && t.n_ex + 1 < t.group) t.ex_off[t.n_ex++] = off(at[j][col]);
+          });
           if (s.n_new == 3 && cl(0) != cl(1)) std::swap(ord[cl(0) == cl(2) ? 1 : 0], ord[2]);
           t.q = (uint8_t)cl(ord[0]);
           t.same = s.n_new == 3 && cl(ord[2]) == cl(ord[0]);
         }
-        std::vector<int> rank(s.n_new);  // new vertex -> its place in the record
         for (int x = 0; x < s.n_new; x++) rank[ord[x]] = x;
         t.n_be = (uint8_t)s.n_be;
         for (int x = 0; x < s.n_be; x++)
@@ -1227,7 +1271,7 @@ struct Exec {
           }
         for (int x = 0; x < s.n_new; x++) {
           const int v = ord[x];
-          for (int col : ck[j][v]) t.cm[x] |= (uint8_t)(1u << (at[j][col] >> 2));
+          ck[j][v].each([&](int col) { t.cm[x] |= (uint8_t)(1u << (at[j][col] >> 2)); });
           const int h = counted ? -1 : at[j + 1][s.w_in + v];
           t.new_off[x] = h >= 0 ? off(h) : dmk::CH_DEAD;
         }
@@ -1302,6 +1346,7 @@ struct Exec {
 
   int ensure_tables(int64_t bytes) {
     if (c->tab_bytes >= bytes) return DM_OK;
+    bytes = std::max(bytes, CHAIN_TAB_MIN);  // so that the next plan finds room as well
     dfree(c, c->tabs);  // in stream order: behind what still reads it
     c->tabs = nullptr;
     c->tab_bytes = 0;
@@ -1363,8 +1408,9 @@ struct Exec {
       }
     }
     dmk::ChainArgs &F = C.launch[0];
-    // a few items a warp, so that dealing them out evens the warps' loads; where there are not even as
-    // many rows as warps, several warps share a row's first candidates
+    // up to eight items a warp, so that dealing them out evens the warps' loads, fewer where a warp has
+    // little to do (CHAIN_ITEM_ROWS); where there are not even as many rows as warps, several warps
+    // share a row's first candidates
     const int64_t warps0 = (int64_t)grid[0] * dmk::CH_CTA_WARPS;
     F.parts = F.n_steps < 2 || 2 * n0 > warps0 ? 1 : (int32_t)std::min<int64_t>(4, warps0 / n0);
     for (auto &A : C.launch) {
@@ -1382,7 +1428,9 @@ struct Exec {
           A.sel_k = (int32_t)k;
         }
     }
-    F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, n0 / (8ll * grid[0] * dmk::CH_CTA_WARPS)));
+    const int64_t deal =
+        std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)(C.work / (CHAIN_ITEM_ROWS * (double)warps0))));
+    F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, (n0 + deal * warps0 - 1) / (deal * warps0)));
     F.seed_n = n0;
     float ms = 0.f;
     int64_t run_steps = 0;
@@ -1398,6 +1446,9 @@ struct Exec {
           if (blocks[i] == 0) continue;  // the first table is used up
         }
         if (!first) CK(cudaMemsetAsync(A.ctr_last + CTR_ITEM, 0, sizeof(unsigned long long), c->stream));
+        A.h_out = first && mode == DM_COUNT && i + 1 == C.launch.size() ? c->h_ctr_steps : nullptr;
+        A.n_out = CTR_N * (S + 1);
+        A.done = c->d_ctr_steps + (size_t)S * CTR_N;  // a count has no sink that would use this set
         CK(dmk::launch_chain(A, blocks[i], c->stream));
         run_steps += A.n_steps + (A.in ? 0 : 1);
       }
@@ -1418,8 +1469,9 @@ struct Exec {
         a.g = g;
         RET(sink->ahead(c, a));
       }
-      CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * (S + 1),
-                         cudaMemcpyDeviceToHost, c->stream));
+      if (!C.launch.back().h_out)
+        CK(cudaMemcpyAsync(c->h_ctr_steps, c->d_ctr_steps, sizeof(unsigned long long) * CTR_N * (S + 1),
+                           cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
       if (c->timing) {
         float t = 0.f;

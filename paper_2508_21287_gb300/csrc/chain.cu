@@ -627,12 +627,13 @@ __device__ __forceinline__ void ch_seed(const ChainArgs &A, unsigned char *W, Ch
   }
 }
 
-// Rows [8 part, 8 part + 8 span) of block b of the input table into the first tile.
+// The rows of block b of the input table whose number is part modulo parts (a power of two) into the
+// first tile.
 __device__ __forceinline__ void ch_fetch(const ChainArgs &A, unsigned char *W, ChainWarp &w, int64_t b, int part,
-                                         int span) {
+                                         int parts) {
   const int lane = threadIdx.x & 31, nc = A.st[1].nc_in;
-  const int nr = min(max(__ldg(A.in_rows + b) - 8 * part, 0), 8 * span), n = __shfl_sync(FULL_MASK, w.cnt, 1);
-  const uint2 *src = (const uint2 *)(A.in + b * (nc + 1) * 256) + 8 * part + lane;
+  const int nr = (__ldg(A.in_rows + b) - part + parts - 1) >> (__ffs(parts) - 1), n = __shfl_sync(FULL_MASK, w.cnt, 1);
+  const uint2 *src = (const uint2 *)(A.in + b * (nc + 1) * 256) + part + parts * lane;
   unsigned char *D = W + (unsigned)A.st[1].in_off * 8u;
   if (lane < nr) {
     unsigned char *d = ch_rows(D) + 8 * (n + lane);
@@ -773,8 +774,11 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
   float best = A.prune;  // the bound as it was asked for last
   const int64_t nw = (int64_t)gridDim.x * CH_WARPS;
   const int64_t n_in = A.in ? imin64((int64_t)*A.in_blocks, A.in_cap) - A.lo : (A.seed_n - A.lo + A.chunk - 1) / A.chunk;
-  // a table of few blocks is dealt out in quarters of a block
-  const int parts = A.in && n_in < 8 * nw ? 4 : 1;
+  // a table of few blocks is dealt out in shares of a block: every warp of the launch before leaves a
+  // partly filled one, so a share is every second or fourth row. 23-vertex path on heavy-hex 9x11: 169 us
+  // in quarters of 8 rows, 111 in twos, 104 in fours; 27-vertex patch on 17x19: 225, 210, 226, by this
+  // line 209
+  const int parts = !A.in || n_in >= 8 * nw ? 1 : n_in < 4 * nw ? 4 : 2;
   const int64_t n_items = n_in * parts * A.parts;
   // items 0 .. nw - 1 are the warps' first; the counter deals out the rest. The next item's number
   // is asked for before the present one is joined.
@@ -797,10 +801,10 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
         const long long it = __shfl_sync(FULL_MASK, nxt, 0);
         more = it < n_items;
         if (more) {
-          if (w.spent > A.limit && parts == 1) nxt = n_items;  // leave the rest to another launch
+          if (n_items <= nw || (w.spent > A.limit && parts == 1)) nxt = n_items;  // one each; or the rest is left to another launch
           else if (lane == 0) nxt = nw + (long long)atomicAdd(A.ctr_last + CTR_ITEM, 1ull);
           if (A.in) {
-            ch_fetch(A, W, w, A.lo + it / parts, (int)(it % parts) * (4 / parts), 4 / parts);
+            ch_fetch(A, W, w, A.lo + it / parts, (int)(it % parts), parts);
           } else {
             w.part = (int)(it % A.parts);
             const int64_t lo = A.lo + it / A.parts * A.chunk;
@@ -854,6 +858,18 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
   for (int i = threadIdx.x; i < 2 * (A.n_steps + 1); i += CH_BLK)
     if (red[i]) atomicAdd(ctr + (int64_t)(i >> 1) * CTR_N + ((i & 1) ? CTR_CAND : CTR_ROWS), red[i]);
   if (MODE == 1 && A.out_kind == 0 && threadIdx.x == 0) atomicAdd(A.ctr_last + CTR_SUM, red[64]);
+  if (MODE == 1 && A.h_out) {  // the last block hands the totals over: a copy behind the launch costs 4 us
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(A.done, 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (last) {
+      __threadfence();
+      const unsigned long long *c0 = A.done - (A.n_out - CTR_N);
+      for (int i = threadIdx.x; i < A.n_out; i += CH_BLK) A.h_out[i] = __ldcg(c0 + i);
+    }
+  }
 }
 
 typedef void (*ChainKernel)(ChainArgs);

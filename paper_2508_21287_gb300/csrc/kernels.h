@@ -125,6 +125,9 @@ struct ChainArgs {
   int64_t in_cap;
   unsigned limit;                // candidates after which a warp takes no further items
   unsigned long long *ctr_last;  // CTR_N counters of the launch's last step, behind those of its others
+  unsigned long long *h_out;     // where set (pinned host memory), the last block writes the n_out
+  unsigned long long *done;      // counters there whose last CTR_N begin at done (one of them, zero
+  int32_t n_out;                 // before the launch, tells which block is the last)
   int32_t *out;                  // packed rows in pattern-vertex order, or blocks
   float *outs;
   int32_t *out_rows;

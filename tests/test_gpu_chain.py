@@ -160,3 +160,15 @@ def test_edge_of_16_bit_ids(ctx, n):
         first = np.arange(n - k + 1)[:, None] + np.arange(k)
         want = np.concatenate([first, first[:, ::-1]])
         assert np.array_equal(rows, want[np.lexsort(want.T[::-1])])
+
+
+@pytest.mark.parametrize("m,n,length", [(4, 4, 30), (5, 6, 27), (9, 11, 23), (15, 16, 21), (27, 28, 20)])
+def test_tables_between_launches(B, ctx, m, n, length):
+    """Deep plans, cut into launches: the table between them in shares of four, of two, and whole blocks,
+    and first tables of fewer rows than warps and of several a warp."""
+    g, p = I.heavy_hex(m, n), I.path(length)
+    gid = ctx.load(g, False)
+    plan = ctx.plan(gid, p)
+    ref = oracle.enumerate(g, p, threads=8, rows=False)
+    for _ in range(2):
+        assert plan.count() == (ref.count, ref.checksum)
