@@ -974,7 +974,8 @@ struct Exec {
     std::vector<int64_t> ids, extra;     // per step: 1 + place of its tables (0: none)
     int64_t tab_bytes = 0;
     bool needs_arena = false;
-    double work = 0;                     // estimated rows of all steps
+    double work = 0, most = 0;           // estimated rows of all steps, of the step with the most
+    bool spare = true;                   // row mode: leave the sink room behind the tables, where that is wise
   };
 
   // Estimated rows after each step, for the cut into launches and into items. A new vertex next to a mapped one
@@ -1170,7 +1171,11 @@ struct Exec {
     };
     const std::vector<double> rows = chain_rows(motifs);
     C.work = 0;
-    for (const double r : rows) C.work += r;
+    C.most = 0;
+    for (const double r : rows) {
+      C.work += r;
+      C.most = std::max(C.most, r);
+    }
     std::vector<double> cost(S + 1, 1e300);  // steps 1 .. j done, tile j + 1 written
     std::vector<int> from(S + 1, -1);
     cost[0] = 0;
@@ -1368,8 +1373,12 @@ struct Exec {
     C.tab.n_ctr = (int64_t)CTR_N * (S + 1);  // and one set for the sink
     // row mode: the sink's work behind the joins needs room that no later round of launches reads. Two
     // halves hold the rows and that, or with tables between launches three thirds; an arena that cannot
-    // grow any more keeps halves for the tables and leaves the sink to itself.
-    const bool several = C.launch.size() > 1, spare = mode == DM_ALL && (!several || c->arena_bytes < c->budget);
+    // grow any more keeps halves for the tables and leaves the sink to itself, unless a third is far more
+    // than the estimated rows take (run() comes back without the spare third should that be wrong).
+    const bool several = C.launch.size() > 1;
+    const bool roomy = C.spare && 8.0 * C.most * (4.0 * p->n_p + 8) < (double)c->arena_bytes / 3;
+    const bool spare = mode == DM_ALL && (!several || c->arena_bytes < c->budget || roomy);
+    C.spare = several && spare;
     const size_t half = c->arena_bytes / (several && spare ? 3 : 2) / 256 * 256;
     int ends = 0;  // plan steps up to the launch
     std::vector<int> grid(C.launch.size());
@@ -1569,7 +1578,11 @@ struct Exec {
         RET(chain ? run_chain(C, &fits) : run_fast(&fits));
         if (fits) return DM_OK;
         c->stats = saved;
-        if (want >= (size_t)c->budget) break;
+        if (want >= (size_t)c->budget) {
+          if (!chain || !C.spare) break;
+          C.spare = false;
+          continue;
+        }
         want *= 4;
       }
       if (c->arena_bytes > ((size_t)4 << 30)) {  // streaming needs the budget the arena holds
