@@ -2489,10 +2489,14 @@ int model_run(dm_ctx *c, const float *x_host, const float *t_host, int32_t n, fl
   return DM_OK;
 }
 
-void normalise(const dm_ctx *c, const float *x, int32_t n, std::vector<float> &out) {
-  out.resize((size_t)n * NFEAT);
+void normalise(const dm_ctx *c, const float *x, int32_t n, float *out) {
   for (int32_t i = 0; i < n; i++)
     for (int k = 0; k < NFEAT; k++) out[(size_t)i * NFEAT + k] = (x[(size_t)i * NFEAT + k] - c->m_mean[k]) / c->m_std[k];
+}
+
+void normalise(const dm_ctx *c, const float *x, int32_t n, std::vector<float> &out) {
+  out.resize((size_t)n * NFEAT);
+  normalise(c, x, n, out.data());
 }
 
 // Predicted cost of a plan: bytes of every intermediate table it writes (rows from the chain
@@ -3587,28 +3591,8 @@ int dm_model_init(dm_ctx *c, uint64_t seed) {
   if (!c) return DM_E_INVAL;
   cudaSetDevice(c->device);
   RET(model_alloc(c));
-  const int64_t P = dmk::mlp_param_count();
-  std::vector<float> w(P, 0.f);
-  uint64_t st = seed;
-  auto next = [&]() {  // SplitMix64
-    st += 0x9E3779B97F4A7C15ull;
-    uint64_t z = st;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-  };
-  auto unif = [&]() { return ((double)(next() >> 11) + 0.5) * (1.0 / 9007199254740992.0) * 2.0 - 1.0; };
-  const int H = 128, IN = NFEAT;
-  double a1 = sqrt(6.0 / IN), a2 = sqrt(6.0 / H), a3 = sqrt(3.0 / H);  // He-uniform
-  size_t o = 0;
-  for (int i = 0; i < H * IN; i++) w[o++] = (float)(a1 * unif());
-  o += H;
-  for (int i = 0; i < H * H; i++) w[o++] = (float)(a2 * unif());
-  o += H;
-  for (int i = 0; i < H; i++) w[o++] = (float)(a3 * unif());
-  CK(cudaMemcpy(c->m_params, w.data(), sizeof(float) * P, cudaMemcpyHostToDevice));
-  CK(cudaMemset(c->m_m, 0, sizeof(float) * P));
-  CK(cudaMemset(c->m_v, 0, sizeof(float) * P));
+  CK(dmk::mlp_init(c->m_params, c->m_m, c->m_v, seed, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
   c->m_step = 0;
   c->m_trained = false;
   for (int k = 0; k < NFEAT; k++) {
@@ -3661,23 +3645,31 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   cudaSetDevice(c->device);
   if (!c->m_params) RET(dm_model_init(c, seed));
   if (!c->m_trained) {  // standardise each input feature over the training set
-    for (int k = 0; k < NFEAT; k++) {
-      double s = 0, s2 = 0;
-      for (int32_t i = 0; i < n; i++) {
-        double v = feats[(size_t)i * NFEAT + k];
-        s += v;
-        s2 += v * v;
+    double s[NFEAT] = {}, s2[NFEAT] = {};
+    for (int32_t i = 0; i < n; i++)
+      for (int k = 0; k < NFEAT; k++) {
+        const double v = feats[(size_t)i * NFEAT + k];
+        s[k] += v;
+        s2[k] += v * v;
       }
-      double mu = s / n, var = s2 / n - mu * mu;
+    for (int k = 0; k < NFEAT; k++) {
+      const double mu = s[k] / n, var = s2[k] / n - mu * mu;
       c->m_mean[k] = (float)mu;
       c->m_std[k] = var > 1e-12 ? (float)sqrt(var) : 1.f;
     }
   }
-  std::vector<float> xn;
-  normalise(c, feats, n, xn);
-  // everything the steps read is uploaded once; losses and the timeout flag come back in the end
+  // everything the steps read is uploaded once; losses and the timeout flag come back in the end. Staged
+  // in the context's pinned buffer where it fits (a copy from other memory is made twice, and waited for)
   const int64_t per_epoch = (n + (int64_t)batch - 1) / batch, n_steps = per_epoch * epochs;
   if (n_steps > (int64_t)1 << 28) return DM_E_CAPACITY;
+  const size_t stage = sizeof(float) * ((size_t)n * (NFEAT + 1) + (size_t)n_steps + 1 + (size_t)n * epochs);
+  const bool pinned = stage <= c->h_stage_bytes;
+  std::vector<float> unpinned(pinned ? 0 : (stage + 3) / sizeof(float));
+  float *hX = pinned ? (float *)c->h_stage : unpinned.data(), *hT = hX + (size_t)n * NFEAT, *hL = hT + n;
+  unsigned *hE = (unsigned *)(hL + n_steps);
+  int32_t *hI = (int32_t *)(hE + 1);
+  normalise(c, feats, n, hX);
+  memcpy(hT, targets, sizeof(float) * n);
   float *X = nullptr, *T = nullptr, *L = nullptr;
   int32_t *I = nullptr;
   unsigned *E = nullptr;
@@ -3708,10 +3700,11 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   A.err = E;
   dmk::mlp_train_layout(A, work, rows);
   auto check = [&](cudaError_t e) { return e == cudaSuccess ? DM_OK : cuda_fail(c, e, "model training"); };
-  r = check(cudaMemcpyAsync(X, xn.data(), sizeof(float) * xn.size(), cudaMemcpyHostToDevice, c->stream));
-  if (r == DM_OK) r = check(cudaMemcpyAsync(T, targets, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
+  r = check(cudaMemcpyAsync(X, hX, sizeof(float) * (size_t)n * NFEAT, cudaMemcpyHostToDevice, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(T, hT, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
   if (r == DM_OK) r = check(cudaMemsetAsync(L, 0, sizeof(float) * n_steps, c->stream));
   if (r == DM_OK) r = check(cudaMemsetAsync(E, 0, sizeof(unsigned), c->stream));
+  if (r == DM_OK) r = check(dmk::mlp_train_begin(A, c->stream));
   std::vector<int32_t> idx(n);
   for (int32_t i = 0; i < n; i++) idx[i] = i;
   uint64_t st = seed ^ 0xA5A5A5A5ull;
@@ -3725,28 +3718,28 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
       z ^= z >> 31;
       std::swap(idx[i], idx[(int32_t)(z % (uint64_t)(i + 1))]);
     }
-    r = check(cudaMemcpyAsync(I, idx.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream));
+    int32_t *hi = hI + (size_t)ep * n;
+    memcpy(hi, idx.data(), sizeof(int32_t) * n);
+    r = check(cudaMemcpyAsync(I, hi, sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream));
     for (int32_t b0 = 0; b0 < n && r == DM_OK; b0 += batch) {
       c->m_step++;
       r = check(dmk::mlp_train_step(A, I + b0, std::min(batch, n - b0), L + step++, lr, c->m_step, c->stream));
     }
   }
-  std::vector<float> losses((size_t)n_steps);
-  unsigned timed_out = 0;
-  if (r == DM_OK) r = check(cudaMemcpyAsync(losses.data(), L, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, c->stream));
-  if (r == DM_OK) r = check(cudaMemcpyAsync(&timed_out, E, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(hL, L, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(hE, E, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
   const cudaError_t se = cudaStreamSynchronize(c->stream);
   if (r == DM_OK) r = check(se);
   release(r);
   if (r != DM_OK) return r;
-  if (timed_out) {
+  if (*hE) {
     c->last_error = "a tensor-core wait of the cardinality model timed out";
     return DM_E_TIMEOUT;
   }
   for (int32_t ep = 0; ep < epochs && out_loss; ep++) {
     double sum = 0;
     for (int64_t k = 0; k < per_epoch; k++)
-      sum += (double)losses[ep * per_epoch + k] * std::min<int64_t>(batch, n - k * batch);
+      sum += (double)hL[ep * per_epoch + k] * std::min<int64_t>(batch, n - k * batch);
     out_loss[ep] = (float)(sum / n);
   }
   c->m_trained = true;

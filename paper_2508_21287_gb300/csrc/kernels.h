@@ -380,12 +380,17 @@ cudaError_t mlp_forward_backward(const float *params, const float *X, const floa
 struct MlpTrain {
   float *params, *m, *v;
   const float *X, *target;   // standardised samples, n x 32, and their targets
-  __nv_bfloat16 *Xb, *H1, *H2, *dH2, *dH1;
+  __nv_bfloat16 *Xb, *H1, *H2, *dH2, *dH1;  // kept for the weight gradients: column blocks of 8 x R samples
   float *dy;
+  uint16_t *W1b, *W2b;       // the rounded weights, in the products' layout
+  int64_t R;
   unsigned *err;
 };
+// Fresh parameters from a seed, and zero moments.
+cudaError_t mlp_init(float *params, float *m, float *v, uint64_t seed, cudaStream_t s);
 int64_t mlp_train_bytes(int batch);
 void mlp_train_layout(MlpTrain &T, void *work, int batch);  // places the buffers of a batch in work
+cudaError_t mlp_train_begin(const MlpTrain &T, cudaStream_t s);  // before the first step: W1b, W2b from params
 cudaError_t mlp_train_step(const MlpTrain &T, const int32_t *idx, int m, float *loss, float lr, int step, cudaStream_t s);
 
 }  // namespace dmk

@@ -329,9 +329,18 @@ __global__ void k_colsum(const __nv_bfloat16 *dH, int rows, int cols, float *db)
 // to device memory. k_train_weights: a block per 32 columns of the weight gradients (or of a bias or
 // output-layer sum) adds over the samples and applies Adam to its own parameters.
 //
-// A step is a chain of small dependent products and nothing else, so it costs what it waits: as fifteen
-// launches with an upload, five allocations and a synchronisation of its own it took 170 us (256
-// samples), as these two launches behind one another 38 us. Products and sums run in the order of
+// A step is a chain of small dependent products and nothing else, so it costs what it waits. What is kept
+// between the launches is kept as the next product reads it, so that a launch begins with bulk copies and
+// no thread converts or transposes: the rounded weights in the canonical layout (written by the threads
+// that apply Adam), and activations and gradients as sample-major 8 x 8 core matrices, whose 16-byte rows
+// are what a thread of k_train_rows holds and which the weight gradients' products read as MN-major
+// operands. The second layer's weights serve both directions from one copy: K-major forward, MN-major back.
+//
+// 256 samples: 170 us a step as fifteen launches with an upload, five allocations and a synchronisation of
+// its own; 38 us as these two launches with every thread converting and transposing what it loads (a
+// transposed copy of W2 alone cost 8000 clocks of bank conflicts); 18 us so. A call of 2048 samples, two
+// epochs: 2.55 ms, 0.85, 0.44. What is left is waiting: two launches behind one another, a bulk copy and
+// three dependent products in the first, one in the second. Products and sums run in the order of
 // mlp_forward_backward, so a step's gradients are the bits that dm_model_grad returns.
 constexpr int TR_THREADS = 512, TR_M = 128;
 
@@ -342,21 +351,37 @@ __device__ __forceinline__ int tr_off(int r, int k) {
 }
 
 // K / 16 MMAs of a staged product, and the arrival of their completion at the barrier.
-template <int KA, int KB>
-__device__ __forceinline__ void tr_mma(uint32_t tmem, const uint16_t *A, const uint16_t *Bt, int N, int K, bool first,
-                                       uint32_t bar) {
+// An operand is its address, the bytes between core matrices along K and along M / N, and whether the
+// 16-byte rows of a core matrix run along M / N (bits 15 and 16 of the instruction descriptor).
+struct TrOp {
+  const uint16_t *p;
+  uint32_t k, mn;
+  bool mn_major;
+};
+__device__ __forceinline__ void tr_mma(uint32_t tmem, const TrOp &A, const TrOp &B, int N, int K, bool first, uint32_t bar) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t idesc = tc_idesc(N) | ((uint32_t)A.mn_major << 15) | ((uint32_t)B.mn_major << 16);
   for (int kk = 0; kk < K; kk += 16) {
-    const uint64_t ad = tc_sdesc(tc_saddr(A) + (kk >> 3) * 128, 128, (KA >> 3) * 128);
-    const uint64_t bd = tc_sdesc(tc_saddr(Bt) + (kk >> 3) * 128, 128, (KB >> 3) * 128);
+    const uint64_t ad = tc_sdesc(tc_saddr(A.p) + (kk >> 3) * A.k, A.k, A.mn);
+    const uint64_t bd = tc_sdesc(tc_saddr(B.p) + (kk >> 3) * B.k, B.k, B.mn);
     const uint32_t acc = !first || kk > 0;
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-        "l"(ad), "l"(bd), "r"(tc_idesc(N)), "r"(acc)
+        "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
         : "memory");
   }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tr_expect(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Bulk copy into shared memory (16-byte aligned, a multiple of 16 bytes), counted at the barrier.
+__device__ __forceinline__ void tr_bulk(void *dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(tc_saddr(dst)),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
 }
 
 // 32 columns of this thread's accumulator row.
@@ -380,12 +405,12 @@ __device__ __forceinline__ uint32_t tr_pack(float lo, float hi) {
 }
 
 struct TrainSmemA {
-  uint16_t x[TR_M * 32], w1[MLP_H * 32];              // K = 32
-  uint16_t h1[TR_M * MLP_H], w2[MLP_H * MLP_H];       // K = 128
-  uint16_t d2[TR_M * MLP_H], w2t[MLP_H * MLP_H];      // K = 128
-  uint16_t h2[TR_M * (MLP_H + 8)];                    // row-major, padded
-  float w3[MLP_H], dy[TR_M];
-  unsigned long long bar;
+  uint16_t x[TR_M * 32], w1[MLP_H * 32];        // K = 32
+  uint16_t h1[TR_M * MLP_H], w2[MLP_H * MLP_H]; // K = 128
+  uint16_t d2[TR_M * MLP_H];
+  uint16_t h2[TR_M * (MLP_H + 8)];              // row-major, padded
+  float b1[MLP_H], b2[MLP_H], w3[MLP_H], dy[TR_M];
+  unsigned long long bar, load[2];              // products; the first and the second layer's weights
   uint32_t tmem;
 };
 
@@ -402,14 +427,15 @@ __device__ __forceinline__ bool tr_wait(uint32_t bar, uint32_t &phase, unsigned 
   return ok;
 }
 
-__device__ __forceinline__ void tr_setup(unsigned long long *bar, uint32_t *tmem, int cols) {
+__device__ __forceinline__ void tr_setup(unsigned long long *bar, int n_bar, uint32_t *tmem, int cols) {
   if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_saddr(tmem)), "r"(cols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_saddr(bar)) : "memory");
+    for (int i = 0; i < n_bar; i++)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tc_saddr(bar + i)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -417,61 +443,80 @@ __device__ __forceinline__ void tr_setup(unsigned long long *bar, uint32_t *tmem
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__device__ __forceinline__ void tr_teardown(unsigned long long *bar, uint32_t tmem, int cols) {
+__device__ __forceinline__ void tr_teardown(unsigned long long *bar, int n_bar, uint32_t tmem, int cols) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (threadIdx.x < 32)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
-  if (threadIdx.x == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc_saddr(bar)) : "memory");
+  if (threadIdx.x == 0)
+    for (int i = 0; i < n_bar; i++) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(tc_saddr(bar + i)) : "memory");
+}
+
+// Wait of the thread that issues the products for a bulk copy; false (and *err raised) when it ran out,
+// after a second bounded wait: the copy must not outlive the block.
+__device__ __forceinline__ bool tr_landed(uint32_t bar, uint32_t phase, unsigned *err) {
+  if (tc_wait(bar, phase)) return true;
+  atomicOr(err, 1u);
+  tc_wait(bar, phase);
+  return false;
+}
+
+// Place (in elements) of column block c8 (eight columns) of sample r in a kept matrix of R samples.
+__device__ __forceinline__ int64_t tr_at(int64_t R, int r, int c8) { return ((int64_t)c8 * R + r) * 8; }
+
+// The rounded weights of both layers from the parameters, before the first step.
+__global__ void __launch_bounds__(256) k_train_begin(const MlpTrain T) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const float *W1 = T.params, *W2 = T.params + MLP_H * MLP_IN + MLP_H;
+  auto bits = [](float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); };
+  if (i < MLP_H * MLP_IN) T.W1b[tr_off<MLP_IN>(i / MLP_IN, i % MLP_IN)] = bits(W1[i]);
+  if (i < MLP_H * MLP_H) T.W2b[tr_off<MLP_H>(i / MLP_H, i % MLP_H)] = bits(W2[i]);
 }
 
 __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, const int32_t *idx, int m, float *loss) {
   extern __shared__ __align__(1024) unsigned char tr_smem[];
   TrainSmemA &S = *(TrainSmemA *)tr_smem;
   constexpr int COLS = 512;  // three accumulators of 128 columns (allocations are powers of two)
+  constexpr int OUT = TR_M / (TR_THREADS / 32);  // rows of the output layer a warp
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rows = (m + 15) / 16 * 16, m0 = blockIdx.x * TR_M;
-  const float *W1 = T.params, *b1 = W1 + MLP_H * MLP_IN, *W2 = b1 + MLP_H, *b2 = W2 + MLP_H * MLP_H;
+  const float *b1 = T.params + MLP_H * MLP_IN, *b2 = b1 + MLP_H + MLP_H * MLP_H;
   const float *w3 = b2 + MLP_H, *b3 = w3 + MLP_H;
-  tr_setup(&S.bar, &S.tmem, COLS);
+  tr_setup(&S.bar, 3, &S.tmem, COLS);
   const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar);
   uint32_t phase = 0;
   // the samples do not depend on the launch before; the parameters do
-  for (int i = tid; i < TR_M * 4; i += TR_THREADS) {  // eight inputs of a row
-    const int r = i >> 2, k = (i & 3) * 8;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (m0 + r < m) {
-      const float4 *x = (const float4 *)(T.X + (int64_t)__ldg(idx + m0 + r) * MLP_IN + k);
-      const float4 p = __ldg(x), q = __ldg(x + 1);
-      v = make_uint4(tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w));
-    }
-    *(uint4 *)(S.x + tr_off<32>(r, k)) = v;
+  static_assert(TR_M * 4 == TR_THREADS, "eight inputs of a row a thread");
+  uint4 xin = make_uint4(0, 0, 0, 0);
+  const int xr = tid >> 2, xk = tid & 3;
+  if (m0 + xr < m) {
+    const float4 *x = (const float4 *)(T.X + (int64_t)__ldg(idx + m0 + xr) * MLP_IN + 8 * xk);
+    const float4 p = __ldg(x), q = __ldg(x + 1);
+    xin = make_uint4(tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w));
   }
+  *(uint4 *)(S.x + tr_off<32>(xr, 8 * xk)) = xin;
+  const int ox = warp + (TR_THREADS / 32) * lane;  // the row of the output layer whose target this lane keeps
+  const float target = lane < OUT && m0 + ox < m ? __ldg(T.target + __ldg(idx + m0 + ox)) : 0.f;
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   griddep_wait();
   griddep_launch_dependents();
-  for (int i = tid; i < TR_M * 4; i += TR_THREADS) {  // kept for the weights of the first layer
-    const int r = i >> 2, k = (i & 3) * 8;
-    if (m0 + r < rows) *(uint4 *)(T.Xb + (int64_t)(m0 + r) * MLP_IN + k) = *(const uint4 *)(S.x + tr_off<32>(r, k));
+  if (tid == 0) {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    tr_expect(tc_saddr(&S.load[0]), sizeof(S.w1));
+    tr_bulk(S.w1, T.W1b, sizeof(S.w1), tc_saddr(&S.load[0]));
+    tr_expect(tc_saddr(&S.load[1]), sizeof(S.w2));
+    tr_bulk(S.w2, T.W2b, sizeof(S.w2), tc_saddr(&S.load[1]));
   }
-  for (int i = tid; i < MLP_H * MLP_IN / 8; i += TR_THREADS) {
-    const int n = i >> 2, k = (i & 3) * 8;
-    const float4 *w = (const float4 *)(W1 + n * MLP_IN + k);
-    const float4 p = w[0], q = w[1];
-    *(uint4 *)(S.w1 + tr_off<32>(n, k)) = make_uint4(tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w));
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (tid < MLP_H) S.b1[tid] = b1[tid];
+  else if (tid < 2 * MLP_H) S.b2[tid - MLP_H] = b2[tid - MLP_H];
+  else if (tid < 3 * MLP_H) S.w3[tid - 2 * MLP_H] = w3[tid - 2 * MLP_H];
+  const float bias3 = b3[0];
+  if (m0 + xr < rows) *(uint4 *)(T.Xb + tr_at(T.R, m0 + xr, xk)) = xin;  // kept for the weights of the first layer
   __syncthreads();
-  if (tid == 0) tr_mma<32, 32>(tmem, S.x, S.w1, MLP_H, MLP_IN, true, bar);
-  for (int i = tid; i < MLP_H * MLP_H / 8; i += TR_THREADS) {  // meanwhile: the second layer, both ways
-    const int n = i >> 4, k = (i & 15) * 8;
-    const float *w = W2 + n * MLP_H + k;  // W2 starts 4224 floats into the parameters: 16-byte aligned
-    const float4 p = *(const float4 *)w, q = *(const float4 *)(w + 4);
-    const uint32_t h[4] = {tr_pack(p.x, p.y), tr_pack(p.z, p.w), tr_pack(q.x, q.y), tr_pack(q.z, q.w)};
-    *(uint4 *)(S.w2 + tr_off<MLP_H>(n, k)) = make_uint4(h[0], h[1], h[2], h[3]);
-#pragma unroll
-    for (int j = 0; j < 8; j++) S.w2t[tr_off<MLP_H>(k + j, n)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
-  }
-  if (tid < MLP_H) S.w3[tid] = w3[tid];
+  const TrOp X{S.x, 128, 512, false}, L1{S.w1, 128, 512, false};
+  const TrOp H1{S.h1, 128, 2048, false}, L2{S.w2, 128, 2048, false};  // h2 x h1, K = h1 ...
+  const TrOp D2{S.d2, 128, 2048, false}, L2t{S.w2, 2048, 128, true};  // ... and backwards h1 x h2, K = h2
+  if (tid == 0 && tr_landed(tc_saddr(&S.load[0]), 0, T.err)) tr_mma(tmem, X, L1, MLP_H, MLP_IN, true, bar);
   const int quad = warp & 3, c0 = 32 * (warp >> 2);  // a warp reads its lane quadrant (warp % 4)
   const int r = 32 * quad + lane;                    // this thread's row: columns c0 .. c0 + 31
   const bool live = m0 + r < rows;
@@ -486,7 +531,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
 #pragma unroll
       for (int j = 0; j < 8; j++) {
         const int c = 8 * q + j;
-        const float z = __uint_as_float(v[c]) + __ldg(b1 + c0 + c);
+        const float z = __uint_as_float(v[c]) + S.b1[c0 + c];
         on1 |= (uint32_t)(z > 0.f) << c;
         v[c] = __float_as_uint(z > 0.f ? z : 0.f);
       }
@@ -494,12 +539,12 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
       for (int j = 0; j < 4; j++) h[j] = tr_pack(__uint_as_float(v[8 * q + 2 * j]), __uint_as_float(v[8 * q + 2 * j + 1]));
       const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
       *(uint4 *)(S.h1 + tr_off<MLP_H>(r, c0 + 8 * q)) = x;
-      if (live) *(uint4 *)(T.H1 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+      if (live) *(uint4 *)(T.H1 + tr_at(T.R, m0 + r, (c0 >> 3) + q)) = x;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) tr_mma<MLP_H, MLP_H>(tmem + 128, S.h1, S.w2, MLP_H, MLP_H, true, bar);
+    if (tid == 0 && tr_landed(tc_saddr(&S.load[1]), 0, T.err)) tr_mma(tmem + 128, H1, L2, MLP_H, MLP_H, true, bar);
     ok = tr_wait(bar, phase, T.err);
   }
   if (ok) {
@@ -510,7 +555,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
 #pragma unroll
       for (int j = 0; j < 8; j++) {
         const int c = 8 * q + j;
-        const float z = __uint_as_float(v[c]) + __ldg(b2 + c0 + c);
+        const float z = __uint_as_float(v[c]) + S.b2[c0 + c];
         on2 |= (uint32_t)(z > 0.f) << c;
         v[c] = __float_as_uint(z > 0.f ? z : 0.f);
       }
@@ -518,22 +563,33 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
       for (int j = 0; j < 4; j++) h[j] = tr_pack(__uint_as_float(v[8 * q + 2 * j]), __uint_as_float(v[8 * q + 2 * j + 1]));
       const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
       *(uint4 *)(S.h2 + r * (MLP_H + 8) + c0 + 8 * q) = x;
-      if (live) *(uint4 *)(T.H2 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+      if (live) *(uint4 *)(T.H2 + tr_at(T.R, m0 + r, (c0 >> 3) + q)) = x;
     }
     __syncthreads();
-    for (int x = warp; x < TR_M; x += TR_THREADS / 32) {  // the output layer: a warp a row (as k_out_layer)
-      float s = 0.f;
-      for (int o = lane; o < MLP_H; o += 32)
-        s += __bfloat162float(__ushort_as_bfloat16(S.h2[x * (MLP_H + 8) + o])) * S.w3[o];
-      for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-      if (lane == 0) {
-        const float y = s + b3[0];
-        const float e = m0 + x < m ? y - __ldg(T.target + __ldg(idx + m0 + x)) : 0.f;
-        const float d = 2.f * e / (float)m;
-        S.dy[x] = d;
-        if (m0 + x < rows) T.dy[m0 + x] = d;
-        if (m0 + x < m) atomicAdd(loss, e * e / (float)m);
-      }
+    float o[OUT];  // the output layer: a warp a row (as k_out_layer), its rows side by side
+#pragma unroll
+    for (int i = 0; i < OUT; i++) {
+      const uint16_t *h = S.h2 + (warp + (TR_THREADS / 32) * i) * (MLP_H + 8) + lane;
+      o[i] = 0.f;
+#pragma unroll
+      for (int k = 0; k < MLP_H; k += 32) o[i] += __bfloat162float(__ushort_as_bfloat16(h[k])) * S.w3[lane + k];
+    }
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int i = 0; i < OUT; i++) o[i] += __shfl_down_sync(0xffffffffu, o[i], off);
+    float y = 0.f;
+#pragma unroll
+    for (int i = 0; i < OUT; i++) {
+      const float t = __shfl_sync(0xffffffffu, o[i], 0);
+      if (lane == i) y = t;
+    }
+    if (lane < OUT) {
+      y += bias3;
+      const float e = m0 + ox < m ? y - target : 0.f;
+      const float d = 2.f * e / (float)m;
+      S.dy[ox] = d;
+      if (m0 + ox < rows) T.dy[m0 + ox] = d;
+      if (m0 + ox < m) atomicAdd(loss, e * e / (float)m);
     }
     __syncthreads();
     const float d = S.dy[r];
@@ -547,12 +603,12 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
       }
       const uint4 x = make_uint4(h[0], h[1], h[2], h[3]);
       *(uint4 *)(S.d2 + tr_off<MLP_H>(r, c0 + 8 * q)) = x;
-      if (live) *(uint4 *)(T.dH2 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = x;
+      if (live) *(uint4 *)(T.dH2 + tr_at(T.R, m0 + r, (c0 >> 3) + q)) = x;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) tr_mma<MLP_H, MLP_H>(tmem + 256, S.d2, S.w2t, MLP_H, MLP_H, true, bar);
+    if (tid == 0) tr_mma(tmem + 256, D2, L2t, MLP_H, MLP_H, true, bar);
     ok = tr_wait(bar, phase, T.err);
   }
   if (ok) {
@@ -565,27 +621,28 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
         const int c = 8 * q + 2 * j;
         h[j] = tr_pack((on1 >> c) & 1u ? __uint_as_float(v[c]) : 0.f, (on1 >> (c + 1)) & 1u ? __uint_as_float(v[c + 1]) : 0.f);
       }
-      if (live) *(uint4 *)(T.dH1 + (int64_t)(m0 + r) * MLP_H + c0 + 8 * q) = make_uint4(h[0], h[1], h[2], h[3]);
+      if (live) *(uint4 *)(T.dH1 + tr_at(T.R, m0 + r, (c0 >> 3) + q)) = make_uint4(h[0], h[1], h[2], h[3]);
     }
   }
-  tr_teardown(&S.bar, tmem, COLS);
+  else if (tid == 0) tr_landed(tc_saddr(&S.load[1]), 0, T.err);  // given up: its copy has still to land
+  tr_teardown(&S.bar, 3, tmem, COLS);
 }
 
-__device__ __forceinline__ void adam_one(float *w, float gi, float *m, float *v, float lr, float b1, float b2, float eps,
-                                         float c1, float c2) {
-  const float mi = b1 * *m + (1.f - b1) * gi;
-  const float vi = b2 * *v + (1.f - b2) * gi * gi;
+__device__ __forceinline__ float adam_one(float w, float gi, float *m, float *v, float m0, float v0, float lr, float b1,
+                                          float b2, float eps, float c1, float c2) {
+  const float mi = b1 * m0 + (1.f - b1) * gi;
+  const float vi = b2 * v0 + (1.f - b2) * gi * gi;
   *m = mi;
   *v = vi;
-  *w -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  return w - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
 constexpr int TR_KC = 256;
 struct TrainSmemB {
-  uint16_t a[MLP_H * TR_KC], b[32 * TR_KC];  // gradient rows (transposed) and inputs of up to 256 samples
+  uint16_t a[MLP_H * TR_KC], b[32 * TR_KC];  // gradients and inputs of up to 256 samples, as they are kept
   float g[MLP_H * 33];                       // the block's gradient
   float part[256];
-  unsigned long long bar;
+  unsigned long long bar, load;
   uint32_t tmem;
 };
 
@@ -598,7 +655,9 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
   const float be1 = 0.9f, be2 = 0.999f, eps = 1e-8f;
   const int tid = threadIdx.x, b = blockIdx.x, rows = (m + 15) / 16 * 16;
   const int oW1 = 0, ob1 = MLP_H * MLP_IN, oW2 = ob1 + MLP_H, ob2 = oW2 + MLP_H * MLP_H, ow3 = ob2 + MLP_H, ob3 = ow3 + MLP_H;
-  auto adam = [&](int at, float g) { adam_one(T.params + at, g, T.m + at, T.v + at, lr, be1, be2, eps, c1, c2); };
+  auto adam = [&](int at, float g) {
+    T.params[at] = adam_one(T.params[at], g, T.m + at, T.v + at, T.m[at], T.v[at], lr, be1, be2, eps, c1, c2);
+  };
   if (b >= 5) {
     griddep_wait();
     griddep_launch_dependents();
@@ -607,9 +666,11 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
     float t = 0.f, u = 0.f;
     auto add = [&](const __nv_bfloat16 *M, const float *wrow) {
       float s = 0.f;
+      const __nv_bfloat16 *col = M + tr_at(T.R, 0, c >> 3) + (c & 7);
       if (sums)
+#pragma unroll 8
         for (int r = tid >> 5; r < rows; r += 8) {
-          const float x = __bfloat162float(M[(int64_t)r * MLP_H + c]);
+          const float x = __bfloat162float(col[8 * r]);
           s += wrow ? wrow[r] * x : x;
         }
       if (sums) S.part[tid] = s;
@@ -638,34 +699,43 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
     return;
   }
   constexpr int COLS = 32;
-  tr_setup(&S.bar, &S.tmem, COLS);
-  const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar);
+  tr_setup(&S.bar, 2, &S.tmem, COLS);
+  const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar), load = tc_saddr(&S.load);
   griddep_wait();
   griddep_launch_dependents();
   // g[o][n] = sum over samples of dH[r][o] * In[r][n]
-  const __nv_bfloat16 *dH = b < 4 ? T.dH2 : T.dH1, *In = b < 4 ? T.H1 + 32 * b : (const __nv_bfloat16 *)T.Xb;
-  const int ldi = b < 4 ? MLP_H : MLP_IN;
-  uint32_t phase = 0;
+  const __nv_bfloat16 *dH = b < 4 ? T.dH2 : T.dH1, *In = b < 4 ? T.H1 + tr_at(T.R, 0, 4 * b) : T.Xb;
+  const TrOp A{S.a, 128, TR_KC * 16, true}, B{S.b, 128, TR_KC * 16, true};
+  constexpr int OWN = MLP_H * 32 / TR_THREADS;
+  float w[OWN], am[OWN], av[OWN];  // the block's parameters, read while the copies and products run
+  auto own = [&](int j) {
+    const int i = tid + j * TR_THREADS, o = i >> 5, n = i & 31;
+    return b < 4 ? oW2 + o * MLP_H + 32 * b + n : oW1 + o * MLP_IN + n;
+  };
+  uint32_t phase = 0, phase_l = 0;
   bool ok = true;
   for (int k0 = 0; k0 < rows && ok; k0 += TR_KC) {
     const int kc = min(TR_KC, rows - k0);  // a multiple of 16
-    for (int i = tid; i < kc * (MLP_H >> 3); i += TR_THREADS) {  // neighbouring threads: neighbouring samples
-      const int o = (i / kc) << 3, k = i % kc;
-      const uint4 x = *(const uint4 *)(dH + (int64_t)(k0 + k) * MLP_H + o);
-      const uint32_t h[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-      for (int j = 0; j < 8; j++) S.a[tr_off<TR_KC>(o + j, k)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
+    if (tid < 32) {
+      if (tid == 0) {
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        tr_expect(load, (uint32_t)kc * 16 * (MLP_H / 8 + 4));
+      }
+      __syncwarp();
+      if (tid < MLP_H / 8) tr_bulk(S.a + tid * TR_KC * 8, dH + tr_at(T.R, k0, tid), (uint32_t)kc * 16, load);
+      else if (tid < MLP_H / 8 + 4)
+        tr_bulk(S.b + (tid - MLP_H / 8) * TR_KC * 8, In + tr_at(T.R, k0, tid - MLP_H / 8), (uint32_t)kc * 16, load);
     }
-    for (int i = tid; i < kc * 4; i += TR_THREADS) {
-      const int n = (i / kc) << 3, k = i % kc;
-      const uint4 x = *(const uint4 *)(In + (int64_t)(k0 + k) * ldi + n);
-      const uint32_t h[4] = {x.x, x.y, x.z, x.w};
+    if (k0 == 0)
 #pragma unroll
-      for (int j = 0; j < 8; j++) S.b[tr_off<TR_KC>(n + j, k)] = (uint16_t)(h[j >> 1] >> (16 * (j & 1)));
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) tr_mma<TR_KC, TR_KC>(tmem, S.a, S.b, 32, kc, k0 == 0, bar);
+      for (int j = 0; j < OWN; j++) {
+        const int at = own(j);
+        w[j] = T.params[at];
+        am[j] = T.m[at];
+        av[j] = T.v[at];
+      }
+    if (tid == 0 && tr_landed(load, phase_l, T.err)) tr_mma(tmem, A, B, 32, kc, k0 == 0, bar);
+    phase_l ^= 1u;
     ok = tr_wait(bar, phase, T.err);
   }
   if (ok) {
@@ -678,17 +748,55 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    for (int i = tid; i < MLP_H * 32; i += TR_THREADS) {
-      const int o = i >> 5, n = i & 31;
-      adam(b < 4 ? oW2 + o * MLP_H + 32 * b + n : oW1 + o * MLP_IN + n, S.g[o * 33 + n]);
+#pragma unroll
+    for (int j = 0; j < OWN; j++) {
+      const int i = tid + j * TR_THREADS, o = i >> 5, n = i & 31, at = own(j);
+      const float x = adam_one(w[j], S.g[o * 33 + n], T.m + at, T.v + at, am[j], av[j], lr, be1, be2, eps, c1, c2);
+      T.params[at] = x;
+      const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(x));  // for the next step's products
+      if (b < 4) T.W2b[tr_off<MLP_H>(o, 32 * b + n)] = h;
+      else T.W1b[tr_off<MLP_IN>(o, n)] = h;
     }
   }
-  tr_teardown(&S.bar, tmem, COLS);
+  tr_teardown(&S.bar, 2, tmem, COLS);
+}
+
+// He-uniform weights from SplitMix64 (draw d from the state seed + (d + 1) * step: W1, W2, w3 in that
+// order, biases zero), and zero moments.
+__global__ void __launch_bounds__(256) k_mlp_init(float *params, float *m, float *v, unsigned long long seed, double a1,
+                                                  double a2, double a3) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int ob1 = MLP_H * MLP_IN, oW2 = ob1 + MLP_H, ob2 = oW2 + MLP_H * MLP_H, ow3 = ob2 + MLP_H, n = ow3 + MLP_H + 1;
+  if (i >= n) return;
+  int d = -1;  // which draw
+  double a = 0.0;
+  if (i < ob1) d = i, a = a1;
+  else if (i >= oW2 && i < ob2) d = i - MLP_H, a = a2;
+  else if (i >= ow3 && i < ow3 + MLP_H) d = i - 2 * MLP_H, a = a3;
+  float x = 0.f;
+  if (d >= 0) {
+    unsigned long long z = seed + (unsigned long long)(d + 1) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z ^= z >> 31;
+    const double u = __dmul_rn(__dadd_rn((double)(z >> 11), 0.5), 2.0 / 9007199254740992.0);
+    x = __double2float_rn(__dmul_rn(a, __dadd_rn(u, -1.0)));
+  }
+  params[i] = x;
+  m[i] = 0.f;
+  v[i] = 0.f;
+}
+
+cudaError_t mlp_init(float *params, float *m, float *v, uint64_t seed, cudaStream_t s) {
+  g_launches++;
+  k_mlp_init<<<(unsigned)((mlp_param_count() + 255) / 256), 256, 0, s>>>(params, m, v, seed, sqrt(6.0 / MLP_IN),
+                                                                       sqrt(6.0 / MLP_H), sqrt(3.0 / MLP_H));
+  return cudaGetLastError();
 }
 
 int64_t mlp_train_bytes(int batch) {
   const int64_t r = (batch + 15) / 16 * 16;
-  return r * MLP_IN * 2 + 4 * r * MLP_H * 2 + r * 4 + 6 * 256;
+  return r * MLP_IN * 2 + 4 * r * MLP_H * 2 + r * 4 + (MLP_IN + MLP_H) * MLP_H * 2 + 8 * 256;
 }
 
 void mlp_train_layout(MlpTrain &T, void *work, int batch) {
@@ -705,6 +813,15 @@ void mlp_train_layout(MlpTrain &T, void *work, int batch) {
   T.dH2 = take(r * MLP_H * 2);
   T.dH1 = take(r * MLP_H * 2);
   T.dy = (float *)take(r * 4);
+  T.W1b = (uint16_t *)take(MLP_H * MLP_IN * 2);
+  T.W2b = (uint16_t *)take(MLP_H * MLP_H * 2);
+  T.R = r;
+}
+
+cudaError_t mlp_train_begin(const MlpTrain &T, cudaStream_t s) {
+  g_launches++;
+  k_train_begin<<<MLP_H * MLP_H / 256, 256, 0, s>>>(T);
+  return cudaGetLastError();
 }
 
 cudaError_t mlp_train_step(const MlpTrain &T, const int32_t *idx, int m, float *loss, float lr, int step, cudaStream_t s) {
