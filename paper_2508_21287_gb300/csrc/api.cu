@@ -93,6 +93,8 @@ struct dm_ctx {
   void *sel_work = nullptr, *sel_out = nullptr;  // top-k selection (select.cu)
   size_t sel_out_bytes = 0;
   void *ord_work = nullptr;  // canonical order (order.cu)
+  void *train_buf = nullptr;  // tables of a training call (dm_model_train)
+  size_t train_bytes = 0;
   bool sel_dirty = false;  // its histogram holds counts that no selection has cleared
   void *tabs = nullptr;  // candidate tables of the plan that runs (chain.cu)
   int64_t tab_bytes = 0;
@@ -2792,6 +2794,7 @@ int dm_destroy(dm_ctx *c) {
   dfree(c, c->tabs);
   dfree(c, c->sel_work);
   dfree(c, c->ord_work);
+  dfree(c, c->train_buf);
   dfree(c, c->sel_out);
   cudaFree(c->m_params);
   cudaFree(c->m_grads);
@@ -3639,6 +3642,8 @@ int dm_model_grad(dm_ctx *c, const float *feats, const float *targets, int32_t n
   return DM_OK;
 }
 
+constexpr size_t TRAIN_KEEP = 64ull << 20;  // bytes of training tables that a context keeps between calls
+
 int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t n, int32_t epochs, int32_t batch,
                    float lr, uint64_t seed, float *out_loss) {
   if (!c || !feats || !targets || n < 1 || epochs < 1 || batch < 16) return DM_E_INVAL;
@@ -3670,27 +3675,38 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   int32_t *hI = (int32_t *)(hE + 1);
   normalise(c, feats, n, hX);
   memcpy(hT, targets, sizeof(float) * n);
-  float *X = nullptr, *T = nullptr, *L = nullptr;
-  int32_t *I = nullptr;
-  unsigned *E = nullptr;
-  void *work = nullptr;
+  // one buffer for the call's tables, kept for the next call up to TRAIN_KEEP
+  const int rows = std::min(batch, n);
+  size_t used = 0;
+  auto place = [&](size_t bytes) {
+    const size_t at = used;
+    used += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t atX = place(sizeof(float) * (size_t)n * NFEAT), atT = place(sizeof(float) * (size_t)n),
+               atL = place(sizeof(float) * (size_t)n_steps), atI = place(sizeof(int32_t) * (size_t)n),
+               atE = place(sizeof(unsigned)), atW = place((size_t)dmk::mlp_train_bytes(rows));
+  if (c->train_bytes < used) {
+    dfree(c, c->train_buf);
+    c->train_buf = nullptr;
+    c->train_bytes = 0;
+    RET(dalloc(c, &c->train_buf, used));
+    c->train_bytes = used;
+  }
+  unsigned char *buf = (unsigned char *)c->train_buf;
+  float *X = (float *)(buf + atX), *T = (float *)(buf + atT), *L = (float *)(buf + atL);
+  int32_t *I = (int32_t *)(buf + atI);
+  unsigned *E = (unsigned *)(buf + atE);
+  void *work = buf + atW;
   auto release = [&](int r) {
-    dfree(c, X);
-    dfree(c, T);
-    dfree(c, L);
-    dfree(c, I);
-    dfree(c, E);
-    dfree(c, work);
+    if (c->train_bytes > TRAIN_KEEP) {
+      dfree(c, c->train_buf);
+      c->train_buf = nullptr;
+      c->train_bytes = 0;
+    }
     return r;
   };
-  const int rows = std::min(batch, n);
-  int r = dalloc_t(c, &X, (size_t)n * NFEAT);
-  if (r == DM_OK) r = dalloc_t(c, &T, n);
-  if (r == DM_OK) r = dalloc_t(c, &L, (size_t)n_steps);
-  if (r == DM_OK) r = dalloc_t(c, &I, n);
-  if (r == DM_OK) r = dalloc_t(c, &E, 1);
-  if (r == DM_OK) r = dalloc(c, &work, (size_t)dmk::mlp_train_bytes(rows));
-  if (r != DM_OK) return release(r);
+  int r = DM_OK;
   dmk::MlpTrain A{};
   A.params = c->m_params;
   A.m = c->m_m;
