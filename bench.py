@@ -47,15 +47,13 @@ BATCH = 32
 WORKLOAD_C2 = ("C2 layout queries: heavy-hex 4x6 (V=159, E=182), 32 queries/step of 10-30 vertices, all "
                "embeddings + FP32 scores + top-100")
 
-# Mean DRAM bytes (read + write) per k_joinw launch over the join launches of one step of the
-# workload, from one ncu pass (metrics dram__bytes_read.sum and dram__bytes_write.sum, with
+# Mean DRAM bytes (read + write) per join step (k_chain runs several in a launch, k_joinw one) over
+# one step of the workload, from one ncu pass (metrics dram__bytes_read.sum and dram__bytes_write.sum, with
 # --clock-control none) over `bench.py --steps 1 --warmup 0 --no-extras --no-cpu --no-e2e`,
-# keyed by workload and by the digest of the join kernel's sources at capture time: after any
+# keyed by workload and by the digest of the join kernels' sources at capture time: after any
 # change to those sources the number no longer describes the kernel and the line reports null.
-JOIN_SOURCES = ("join_warp.cu", "join_warp.cuh", "join_device.cuh", "dm_internal.h")
+JOIN_SOURCES = ("chain.cu", "join_warp.cu", "join_warp.cuh", "join_device.cuh", "dm_internal.h")
 JOIN_TRAFFIC_BYTES_PER_LAUNCH: dict[tuple[str, str], float] = {
-    # C3 heavy-hex 53x59, the default workload: 283 join launches of one step
-    ("c3:heavyhex:53,59:0:32", "77d42d2fa826a22f"): 252958173.0,
 }
 
 
@@ -454,7 +452,7 @@ def measure_queries(args, kind: str, with_e2e: bool, with_cpu: bool, fuse: bool 
             if rec is not None:
                 st = B.dm_get_stats(ctx.h)
                 record(rec, st)
-                with lock:  # counters of every join launch come back to the host: 8 x u64 each
+                with lock:  # counters of every join step come back to the host: 8 x u64 each
                     rec["d2h"] += 64 * st["join_launches"]
             emb += cnt
         return emb
@@ -534,12 +532,14 @@ def measure_queries(args, kind: str, with_e2e: bool, with_cpu: bool, fuse: bool 
     achieved = racc["join_bytes"] / (racc["join_ms"] / 1e3) / 1e9 if racc["join_ms"] > 0 else 0.0
     digest = join_kernel_digest()
     traffic = JOIN_TRAFFIC_BYTES_PER_LAUNCH.get((workload_key(args, kind), digest))
-    roofline = {"bound": "hbm", "kernel": "k_joinw", "achieved": achieved, "peak": peak, "unit": "GB/s",
+    roofline = {"bound": "hbm", "kernel": "k_chain", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_source": "measured (burst copy)" if "hbm_gbs" in peaks else "fallback",
                 "traffic": traffic, "kernel_digest": digest,
                 "algorithmic_bytes_per_launch": racc["join_bytes"] / max(1, racc["join_launches"]),
                 "avg_launch_us": 1e3 * racc["join_ms"] / max(1, racc["join_launches"]),
                 "launches": racc["join_launches"],
+                "note": "per join step; rows between the steps stay in shared memory, so the bytes are the motif "
+                        "tables' and those of tables between launches: bound by instructions, not by memory",
                 "timed": ("in the timed steps (CUDA events on the library's stream)" if n_ctx == 1 else
                           "separate pass, one context, queries in sequence")}
 
@@ -583,10 +583,9 @@ def run_ours(args):
                             "gpu_launches": fz["gpu_launches"],
                             "roofline": {k: fz["roofline"][k] for k in ("achieved", "frac", "avg_launch_us", "launches",
                                                                         "algorithmic_bytes_per_launch")},
-                            "note": "the same queries with each plan's last two joins in one kernel "
-                                    "(dm_set_fusion): the table between them stays in shared memory, "
-                                    "so fewer bytes move and the fraction of the HBM peak falls while "
-                                    "embeddings/s rise"}
+                            "note": "the same queries with dm_set_fusion: the last two joins in one kernel for plans "
+                                    "that run a launch a step (those that run several steps a launch keep every "
+                                    "table between them in shared memory with or without it)"}
         line["c2"] = summary_c2(measure_queries(args_for(args, "c2"), "c2", with_e2e=True, with_cpu=False))
         line["c4"] = summary_c4(run_c4(args_for(args, "c4"), emit=False))
         line["c5"] = summary_c5(run_c5(args_for(args, "c5"), emit=False))
