@@ -172,3 +172,19 @@ def test_tables_between_launches(B, ctx, m, n, length):
     ref = oracle.enumerate(g, p, threads=8, rows=False)
     for _ in range(2):
         assert plan.count() == (ref.count, ref.checksum)
+
+
+@pytest.mark.parametrize("budget", [2 << 30, 400 << 20, 40 << 20])
+def test_rows_of_several_launches_at_the_budget(B, budget):
+    """Rows of a plan cut into launches with the arena at its budget: room for the order behind the joins,
+    room for the tables only, and too little for one table (streamed)."""
+    g, p = I.lognormal_weights(I.heavy_hex(9, 11), 5), I.path(20)
+    ref = oracle.enumerate(g, p, threads=8)
+    with B.Context(0, budget) as c:
+        plan = c.plan(c.load(g), p)
+        for _ in range(2):
+            rows, scores, cnt, cs = plan.all()
+            assert (cnt, cs) == (ref.count, ref.checksum)
+            if budget < 400 << 20:  # chunks are sorted one by one
+                rows = rows[np.lexsort(rows.T[::-1])]
+            assert np.array_equal(rows, ref.rows)
