@@ -481,6 +481,7 @@ struct Sink {
     DevGraph *g;
   };
   virtual int ahead(dm_ctx *, const Ahead &) { return DM_OK; }
+  virtual bool counts() const { return true; }  // ahead() uses those counters
   virtual void forget() {}  // the table did not fit, or others follow it
   // k > 0: only the k best rows are wanted, and rows whose partial score is above the k-th best of those
   // seen may be dropped; hist receives where the joins count the scores of what they write
@@ -1457,9 +1458,10 @@ struct Exec {
           if (blocks[i] == 0) continue;  // the first table is used up
         }
         if (!first) CK(cudaMemsetAsync(A.ctr_last + CTR_ITEM, 0, sizeof(unsigned long long), c->stream));
-        A.h_out = first && mode == DM_COUNT && i + 1 == C.launch.size() ? c->h_ctr_steps : nullptr;
+        const bool own = mode == DM_COUNT || (sink && !sink->counts());  // no sink's counters to wait for
+        A.h_out = first && own && i + 1 == C.launch.size() ? c->h_ctr_steps : nullptr;
         A.n_out = CTR_N * (S + 1);
-        A.done = c->d_ctr_steps + (size_t)S * CTR_N;  // a count has no sink that would use this set
+        A.done = c->d_ctr_steps + (size_t)S * CTR_N;  // nothing else uses this set then
         CK(dmk::launch_chain(A, blocks[i], c->stream));
         run_steps += A.n_steps + (A.in ? 0 : 1);
       }
@@ -1667,6 +1669,8 @@ int64_t topk_k(const TopkSink *t);
 int topk_enqueue(dm_ctx *c, int64_t k, const DevTable &t, const unsigned long long *n_dev, bool sorted,
                  bool counted = false);
 bool topk_enqueued(dm_ctx *c, int64_t k, int64_t n, int32_t w, int32_t *rows, float *scores);
+
+constexpr size_t TOPK_DIRECT = 64 << 10;
 
 struct AllSink : Sink {
   TopkSink *tap = nullptr;  // also feeds every final chunk to a top-k accumulator
@@ -1885,9 +1889,12 @@ int topk_enqueue(dm_ctx *c, int64_t k, const DevTable &t, const unsigned long lo
   a.counted = counted;
   a.work = c->sel_work;
   a.out = (unsigned char *)c->sel_out;
+  // few rows are written to the host's buffer as well, by the kernel itself: a copy behind it costs more
+  const bool direct = bytes <= TOPK_DIRECT;
+  a.h_out = direct ? (unsigned char *)c->h_stage : nullptr;
   CK(dmk::topk_select(a, c->num_sms, c->stream));
   c->sel_dirty = false;  // it leaves the histogram zeroed
-  CK(cudaMemcpyAsync(c->h_stage, c->sel_out, bytes, cudaMemcpyDeviceToHost, c->stream));
+  if (!direct) CK(cudaMemcpyAsync(c->h_stage, c->sel_out, bytes, cudaMemcpyDeviceToHost, c->stream));
   return DM_OK;
 }
 
@@ -1943,6 +1950,7 @@ struct TopkSink : Sink {
     tried = true;
     return DM_OK;
   }
+  bool counts() const override { return false; }
   void forget() override { tried = false; }
   bool counted = false;       // the joins count the scores and lower the bound (best_only)
   int64_t best_only(dm_ctx *c, dmk::SelHist **hist) override {

@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(CH_BLK, 4) k_chain(const __grid_constant__ Cha
   for (int i = threadIdx.x; i < 2 * (A.n_steps + 1); i += CH_BLK)
     if (red[i]) atomicAdd(ctr + (int64_t)(i >> 1) * CTR_N + ((i & 1) ? CTR_CAND : CTR_ROWS), red[i]);
   if (MODE == 1 && A.out_kind == 0 && threadIdx.x == 0) atomicAdd(A.ctr_last + CTR_SUM, red[64]);
-  if (MODE == 1 && A.h_out) {  // the last block hands the totals over: a copy behind the launch costs 4 us
+  if (A.h_out) {  // the last block hands the totals over: a copy behind the launch costs 4 us
     __shared__ bool last;
     __threadfence();
     __syncthreads();

@@ -289,7 +289,7 @@ struct SelectArgs {
   int32_t w, k, sorted;              // sorted: the rows are in canonical order
   int32_t counted;                   // the scores are in the work buffer's histogram already
   void *work;
-  unsigned char *out;
+  unsigned char *out, *h_out;        // the result; where set, pinned host memory that receives it as well
 };
 constexpr int64_t select_out_bytes(int64_t k, int64_t w) { return 16 + 4 * k + 4 * k * w; }
 int64_t select_work_bytes();

@@ -16,7 +16,9 @@
 // it is launch latency, 3 + 8 + 5 us. It replaces a radix select with a read-back of the histogram to
 // the host after each of four passes, a canonical sort of the selected rows and four radix passes over
 // them (30 launches, 7 synchronisations). Wall clock of whole calls: best 100 of the 26 258 layouts of a
-// 22-qubit circuit 640 us -> 113 us, best 10 of 3.1 M 593 us -> 143 us (254 us without the pruning).
+// 22-qubit circuit 640 us -> 113 us, best 10 of 3.1 M 593 us -> 143 us (254 us without the pruning). Results
+of up to 64 KB are written to the host's pinned buffer by k_sel_rank itself, and the joins' counters by
+their last block: two copies fewer behind the kernels, 90 us -> 84 and 119 -> 113 on the same calls later.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -141,7 +143,10 @@ __global__ void __launch_bounds__(SEL_BLK) k_sel_rank(const SelectArgs a) {
   griddep_launch_dependents();
   const int lane = threadIdx.x & 31;
   const uint32_t m = W->m;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ((uint32_t *)a.out)[0] = m;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ((uint32_t *)a.out)[0] = m;
+    if (a.h_out) ((uint32_t *)a.h_out)[0] = m;
+  }
   for (int i = blockIdx.x * SEL_BLK + threadIdx.x; i < SEL_BINS; i += gridDim.x * SEL_BLK) {
     W->h.fine[i] = 0;
     if (i < SelHist::COARSE) W->h.coarse[i] = 0;
@@ -150,6 +155,8 @@ __global__ void __launch_bounds__(SEL_BLK) k_sel_rank(const SelectArgs a) {
   if (m > SEL_CAP) return;
   float *osc = (float *)(a.out + 16);
   int32_t *orows = (int32_t *)(osc + a.k);
+  float *hsc = (float *)(a.h_out + 16);
+  int32_t *hrows = (int32_t *)(hsc + a.k);
   for (uint32_t i = (blockIdx.x * SEL_BLK + threadIdx.x) >> 5; i < m; i += (gridDim.x * SEL_BLK) >> 5) {
     const uint32_t key = W->key[i];
     const int32_t row = W->idx[i];
@@ -160,8 +167,15 @@ __global__ void __launch_bounds__(SEL_BLK) k_sel_rank(const SelectArgs a) {
     }
     rank = __reduce_add_sync(FULL_MASK, rank);
     if (rank >= (unsigned)a.k) continue;
-    if (lane == 0) osc[rank] = __ldg(a.sc + row);
-    for (int c = lane; c < a.w; c += 32) orows[(int64_t)rank * a.w + c] = __ldg(a.rows + (int64_t)row * a.w + c);
+    const float sc = __ldg(a.sc + row);
+    if (lane == 0) osc[rank] = sc;
+    if (lane == 0 && a.h_out) hsc[rank] = sc;
+    for (int c = lane; c < a.w; c += 32) {
+      const int64_t at = (int64_t)rank * a.w + c;
+      const int32_t v = __ldg(a.rows + (int64_t)row * a.w + c);
+      orows[at] = v;
+      if (a.h_out) hrows[at] = v;
+    }
   }
 }
 
