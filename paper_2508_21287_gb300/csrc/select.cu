@@ -17,8 +17,8 @@
 // the host after each of four passes, a canonical sort of the selected rows and four radix passes over
 // them (30 launches, 7 synchronisations). Wall clock of whole calls: best 100 of the 26 258 layouts of a
 // 22-qubit circuit 640 us -> 113 us, best 10 of 3.1 M 593 us -> 143 us (254 us without the pruning). Results
-of up to 64 KB are written to the host's pinned buffer by k_sel_rank itself, and the joins' counters by
-their last block: two copies fewer behind the kernels, 90 us -> 84 and 119 -> 113 on the same calls later.
+// of up to 64 KB are written to the host's pinned buffer by k_sel_rank itself, and the joins' counters by
+// their last block: two copies fewer behind the kernels, 90 us -> 84 and 119 -> 113 on the same calls later.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
