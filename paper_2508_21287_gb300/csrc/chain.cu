@@ -36,9 +36,9 @@
 // an SM, whose tiles take all shared memory; about 130 warp instructions for 32 candidates and 2 a
 // cycle and SM, where the launch-per-step kernel (k_joinw) needs about 450 and moves every table
 // through device memory. Counts, wall clock, that kernel against this one: 24-vertex path on heavy-hex
-// 53x59 5.21 ms -> 2.23 ms (54 M embeddings, 256 M candidates), 37-vertex patch there 1.60 -> 0.89 ms,
-// 10-vertex path on the 60x60 grid 1.81 -> 0.68 ms, 13-vertex path on a random 3-regular graph of 4096
-// vertices 0.58 -> 0.32 ms. Steps on the way (24-vertex path): columns of half-words copied one by one
+// 53x59 5.21 ms -> 2.36 ms (53 M embeddings, 251 M candidates), 37-vertex patch there 1.60 -> 0.86 ms,
+// 10-vertex path on the 60x60 grid 1.81 -> 0.67 ms, 13-vertex path on a random 3-regular graph of 4096
+// vertices 0.58 -> 0.30 ms. Steps on the way (24-vertex path): columns of half-words copied one by one
 // 9.0 ms, chunks of four 5.0, candidates in groups of one size 2.9, chunks by colour class and the last
 // step counted on the spot 2.5, the key's own neighbours left out 2.2. Unrolling every step for every
 // number of chunks in one kernel cost more in instruction-cache misses than it saved (3.0).
