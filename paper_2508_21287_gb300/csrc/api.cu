@@ -1424,7 +1424,7 @@ struct Exec {
     // little to do (CHAIN_ITEM_ROWS); where there are not even as many rows as warps, several warps
     // share a row's first candidates
     const int64_t warps0 = (int64_t)grid[0] * dmk::CH_CTA_WARPS;
-    F.parts = F.n_steps < 2 || 2 * n0 > warps0 ? 1 : (int32_t)std::min<int64_t>(4, warps0 / n0);
+    F.parts = F.n_steps < 2 || 2 * n0 > warps0 ? 1 : 4 * n0 > warps0 ? 2 : 4;
     for (auto &A : C.launch) {
       A.sel = nullptr;
       A.sel_k = 0;

@@ -36,8 +36,8 @@
 // an SM, whose tiles take all shared memory; about 130 warp instructions for 32 candidates and 2 a
 // cycle and SM, where the launch-per-step kernel (k_joinw) needs about 450 and moves every table
 // through device memory. Counts, wall clock, that kernel against this one: 24-vertex path on heavy-hex
-// 53x59 5.21 ms -> 2.36 ms (53 M embeddings, 251 M candidates), 37-vertex patch there 1.60 -> 0.86 ms,
-// 10-vertex path on the 60x60 grid 1.81 -> 0.67 ms, 13-vertex path on a random 3-regular graph of 4096
+// 53x59 5.21 ms -> 2.28 ms (53 M embeddings, 251 M candidates), 37-vertex patch there 1.60 -> 0.86 ms,
+// 10-vertex path on the 60x60 grid 1.81 -> 0.66 ms, 13-vertex path on a random 3-regular graph of 4096
 // vertices 0.58 -> 0.30 ms. Steps on the way (24-vertex path): columns of half-words copied one by one
 // 9.0 ms, chunks of four 5.0, candidates in groups of one size 2.9, chunks by colour class and the last
 // step counted on the spot 2.5, the key's own neighbours left out 2.2. Unrolling every step for every
@@ -413,7 +413,9 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
     len &= in;
   }
   const bool then = CN && j + 1 == A.n_steps;
-  auto mine = [&](int at) { return j > 1 || A.parts == 1 || at % A.parts == w.part; };
+  // the places that are this warp's, modulo 4 (taking a remainder for each candidate instead: 24-vertex path 2.36 ms
+  // against 2.28)
+  const unsigned own = j > 1 || A.parts == 1 ? 0xFu : (A.parts == 2 ? 0x5u : 0x1u) << w.part;
   const unsigned seen = c == 0 && (j > 1 || w.part == 0) ? __reduce_add_sync(FULL_MASK, len) : 0u;
   const int nch0 = __shfl_sync(FULL_MASK, w.cnt, j + 1);
   int nch = nch0;
@@ -454,7 +456,7 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
       for (int u = 0; u < 4; u++) {
         if (c > u) continue;                   // done before (uniform)
         if (u >= longest || nch >= 32) break;  // 32 rows in the next tile: that one first
-        if (mine(u)) one(id[u], 0u, true);
+        if (own >> u & 1u) one(id[u], 0u, true);
         c = u + 1;
       }
     } else {
@@ -462,7 +464,7 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
       for (int u = 0; u < 4; u++) {
         if ((c & 3) != u) continue;
         if (c >= longest || nch >= 32) break;
-        if (mine(c)) one(x[u].x, x[u].y, same);
+        if (own >> u & 1u) one(x[u].x, x[u].y, same);
         c++;
       }
       if ((c & 3) == 0 && c < longest) ch_load4(ids + c, x);
