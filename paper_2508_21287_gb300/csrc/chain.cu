@@ -413,8 +413,8 @@ __device__ __forceinline__ void ch_step_dense(const ChainArgs &A, unsigned char 
     len &= in;
   }
   const bool then = CN && j + 1 == A.n_steps;
-  // the places that are this warp's, modulo 4 (taking a remainder for each candidate instead: 24-vertex path 2.36 ms
-  // against 2.28)
+  // the places that are this warp's, modulo 4 (with a remainder for each candidate instead, a 24-vertex
+  // path took 2.36 ms against 2.28)
   const unsigned own = j > 1 || A.parts == 1 ? 0xFu : (A.parts == 2 ? 0x5u : 0x1u) << w.part;
   const unsigned seen = c == 0 && (j > 1 || w.part == 0) ? __reduce_add_sync(FULL_MASK, len) : 0u;
   const int nch0 = __shfl_sync(FULL_MASK, w.cnt, j + 1);
