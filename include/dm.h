@@ -278,6 +278,12 @@ int dm_set_tuning(dm_ctx *ctx, int autotune, double hash_load_factor, double hea
  * Results are identical in every case. No counterpart in the paper (its joins are library calls). */
 int dm_set_fusion(dm_ctx *ctx, int on);
 
+/* Work of a launch that runs several join steps (no counterpart in the paper): a warp takes no further
+ * rows of the plan's first table after this many candidates (0 = the default, 2^20: about 2.5e9 a
+ * launch), and what is left is joined by further rounds of launches. Results are identical for every
+ * value. DM_E_INVAL if negative. */
+int dm_set_launch_limit(dm_ctx *ctx, int32_t candidates);
+
 /* Block shape of dm_match_batch when autotuning is off (no counterpart in the paper):
  * threads_per_cta 128 or 256 (every CTA walks its work items through the plan's steps in
  * tiles of the tuned row count), or 32 (every warp walks its own work items in 32-row tiles,

@@ -119,6 +119,7 @@ _SIGS = {
                                        _i32p, _i32p, ctypes.POINTER(ctypes.c_double)]),
     "dm_set_batch_shape": (ctypes.c_int, [_vp, _i32, _i32]),
     "dm_set_fusion": (ctypes.c_int, [_vp, ctypes.c_int]),
+    "dm_set_launch_limit": (ctypes.c_int, [_vp, _i32]),
     "dm_batch_latency": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double), _i32]),
     "dm_set_tuning": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_double, ctypes.c_double]),
     "dm_model_init": (ctypes.c_int, [_vp, _u64]),
@@ -484,6 +485,10 @@ def dm_set_batch_shape(ctx, threads_per_cta: int = 256, ctas_per_sm: int = 0) ->
 
 def dm_set_fusion(ctx, on: bool = True) -> None:
     _check(_lib.dm_set_fusion(ctx, int(bool(on))), "dm_set_fusion", ctx)
+
+
+def dm_set_launch_limit(ctx, candidates: int = 0) -> None:
+    _check(_lib.dm_set_launch_limit(ctx, int(candidates)), "dm_set_launch_limit", ctx)
 
 
 def dm_batch_latency(ctx, n: int) -> np.ndarray:

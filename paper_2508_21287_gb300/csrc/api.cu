@@ -112,6 +112,7 @@ struct dm_ctx {
   double hash_lf = 0.5;               // load factor of two-key hash indices
   double heavy_rows = 1e300;          // plans predicted to hold more rows run step by step
   int batch_threads = 256, batch_ctas = 0;  // block shape of dm_match_batch without autotuning
+  uint32_t launch_limit = 1u << 20;  // a warp's candidates (dm_set_launch_limit): about 2.5e9 a launch, tens of ms
   bool fuse_last = false;  // counted plans: the last two joins in one launch when they qualify
   std::vector<double> batch_latency;  // per plan, ms from the start of the last dm_match_batch
 };
@@ -1229,7 +1230,6 @@ struct Exec {
       A.eerr = g->eerr;
       A.qerr = a0.qerr;
       A.scored = a0.scored;
-      A.limit = 1u << 20;  // a warp's candidates: about 2.5e9 a launch, tens of milliseconds
       int o = 0;
       std::vector<int> tile(last + 2, 0);
       for (int j = first + 1; j <= (end ? last_tile : last + 1); j++) {
@@ -1363,9 +1363,11 @@ struct Exec {
     return DM_OK;
   }
 
-  // Run the launches of a laid-out plan. A launch is bounded in work: what it leaves of its input
-  // is taken up by another round of launches. *fits is false when a table or the rows overflow the
-  // arena (nothing is delivered then).
+  // Run the launches of a laid-out plan. The first launch is bounded in work: what it leaves of the first
+  // table is taken up by another round of launches. The others join all of their input, so that a table
+  // between launches is read to its end by the next launch and holds nothing from one round to the next:
+  // it can share its memory with the one after the next, and each round starts it from its first block.
+  // *fits is false when a table or the rows overflow the arena (nothing is delivered then).
   int run_chain(Chain &C, bool *fits) {
     const int S = (int)st.size();
     *fits = false;
@@ -1399,26 +1401,31 @@ struct Exec {
       ends += A.n_steps;
       A.ctr_last = c->d_ctr_steps + (size_t)ends * CTR_N;
       A.prune = prune;
-      unsigned char *buf = C.needs_arena ? c->arena + (i & 1) * half : nullptr;
+      A.limit = i ? ~0u : c->launch_limit;
       if (A.out_kind == 1) {
+        unsigned char *buf = c->arena + (i & 1) * half;
         const int64_t rb = 4ll * A.wo + (A.scored ? 4 : 0);
         A.out_cap = std::max<int64_t>(1, ((int64_t)half - 512) / rb);
         A.out = (int32_t *)buf;
         A.outs = A.scored ? (float *)(buf + ((size_t)A.out_cap * A.wo * 4 + 255) / 256 * 256) : nullptr;
-      } else if (A.out_kind == 2) {
+      }
+      if (i) A.in_blocks = c->d_ctr_steps + (size_t)before * CTR_N + CTR_BLOCKS;
+    }
+    // tables between launches, the even ones at t0 and the odd ones at t1, `bytes` each
+    auto place_tables = [&](unsigned char *t0, unsigned char *t1, size_t bytes) {
+      for (size_t i = 0; i + 1 < C.launch.size(); i++) {
+        dmk::ChainArgs &A = C.launch[i], &N = C.launch[i + 1];
+        unsigned char *buf = i & 1 ? t1 : t0;
         const int64_t bb = (A.st[A.n_steps].nc_out + 1) * 256;
-        A.out_cap = std::max<int64_t>(1, ((int64_t)half - 512) / (bb + 4));
+        A.out_cap = std::max<int64_t>(1, ((int64_t)bytes - 512) / (bb + 4));
         A.out = (int32_t *)buf;
         A.out_rows = (int32_t *)(buf + A.out_cap * bb);
+        N.in = (const unsigned char *)A.out;
+        N.in_rows = A.out_rows;
+        N.in_cap = A.out_cap;
       }
-      if (i) {
-        const dmk::ChainArgs &P = C.launch[i - 1];
-        A.in = (const unsigned char *)P.out;
-        A.in_rows = P.out_rows;
-        A.in_blocks = c->d_ctr_steps + (size_t)before * CTR_N + CTR_BLOCKS;
-        A.in_cap = P.out_cap;
-      }
-    }
+    };
+    if (several) place_tables(c->arena, c->arena + half, half);
     dmk::ChainArgs &F = C.launch[0];
     // up to eight items a warp, so that dealing them out evens the warps' loads, fewer where a warp has
     // little to do (CHAIN_ITEM_ROWS); where there are not even as many rows as warps, several warps
@@ -1445,24 +1452,26 @@ struct Exec {
     F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, (n0 + deal * warps0 - 1) / (deal * warps0)));
     F.seed_n = n0;
     float ms = 0.f;
-    int64_t run_steps = 0;
+    int64_t run_steps = 0, warps = 0;  // warps of the first launch
     for (bool more = true, first = true; more; first = false) {
       if (c->timing) CK(cudaEventRecord(c->ev0, c->stream));
       if (first) CK(dmk::launch_chain_tables(C.tab, c->stream));
-      std::vector<int> blocks(grid);
+      static_assert(CTR_BLOCKS == CTR_ITEM + 1, "set back together");
+      for (size_t i = 0; !first && i < C.launch.size(); i++)  // items dealt out, blocks of the table written
+        CK(cudaMemsetAsync(C.launch[i].ctr_last + CTR_ITEM, 0, 2 * sizeof(unsigned long long), c->stream));
       for (size_t i = 0; i < C.launch.size(); i++) {
         dmk::ChainArgs &A = C.launch[i];
+        int blocks = grid[i];
         if (!A.in) {
           const int64_t items = (n0 - A.lo + A.chunk - 1) / A.chunk * A.parts;
-          blocks[i] = (int)std::min<int64_t>(grid[i], (items + dmk::CH_CTA_WARPS - 1) / dmk::CH_CTA_WARPS);
-          if (blocks[i] == 0) continue;  // the first table is used up
+          blocks = (int)std::min<int64_t>(blocks, (items + dmk::CH_CTA_WARPS - 1) / dmk::CH_CTA_WARPS);
+          warps = (int64_t)blocks * dmk::CH_CTA_WARPS;
         }
-        if (!first) CK(cudaMemsetAsync(A.ctr_last + CTR_ITEM, 0, sizeof(unsigned long long), c->stream));
         const bool own = mode == DM_COUNT || (sink && !sink->counts());  // no sink's counters to wait for
         A.h_out = first && own && i + 1 == C.launch.size() ? c->h_ctr_steps : nullptr;
         A.n_out = CTR_N * (S + 1);
         A.done = c->d_ctr_steps + (size_t)S * CTR_N;  // nothing else uses this set then
-        CK(dmk::launch_chain(A, blocks[i], c->stream));
+        CK(dmk::launch_chain(A, blocks, c->stream));
         run_steps += A.n_steps + (A.in ? 0 : 1);
       }
       if (c->timing) CK(cudaEventRecord(c->ev1, c->stream));
@@ -1496,18 +1505,19 @@ struct Exec {
           if (sink) sink->forget();
           return DM_OK;
         }
-      more = false;
-      for (size_t i = 0; i < C.launch.size(); i++) {  // every warp's first item and those the counter gave out are done
-        dmk::ChainArgs &A = C.launch[i];
-        const unsigned long long *h = c->h_ctr_steps + (A.ctr_last - c->d_ctr_steps);
-        const int64_t n_in = A.in ? (int64_t)c->h_ctr_steps[A.in_blocks - c->d_ctr_steps] : n0;
-        // (a table of few blocks is always joined to its end)
-        const int64_t warps = (int64_t)blocks[i] * dmk::CH_CTA_WARPS;
-        const int64_t done = A.in && n_in - A.lo < 8 * warps ? n_in : warps + (blocks[i] ? (int64_t)h[CTR_ITEM] : 0);
-        A.lo = std::min<int64_t>(n_in, A.lo + (A.in ? done : done / A.parts * A.chunk));
-        more |= A.lo < n_in;
-      }
+      // every warp's first item and those the counter gave out are done
+      const int64_t done = warps + (int64_t)c->h_ctr_steps[(F.ctr_last - c->d_ctr_steps) + CTR_ITEM];
+      F.lo = std::min<int64_t>(n0, F.lo + done / F.parts * F.chunk);
+      more = F.lo < n0;
       if (more && sink) sink->forget();
+      // rows that are there stay while further rounds add to them: three launches or more then keep their
+      // tables out of the rows' region, in the other one and the spare third, or in the halves of the other
+      if (more && first && mode == DM_ALL && C.launch.size() > 2) {
+        unsigned char *other = c->arena + (C.launch.size() & 1 ? half : 0);
+        const size_t part = half / 512 * 256;
+        if (spare) place_tables(other, c->arena + 2 * half, half);
+        else place_tables(other, other + part, part);
+      }
       for (auto &A : C.launch) A.sel = nullptr;  // what was counted went with the first round's selection
     }
     *fits = true;
@@ -3382,6 +3392,12 @@ int dm_set_batch_shape(dm_ctx *c, int32_t threads_per_cta, int32_t ctas_per_sm) 
     batch_release(c, c->batch);
     c->batch = nullptr;
   }
+  return DM_OK;
+}
+
+int dm_set_launch_limit(dm_ctx *c, int32_t candidates) {
+  if (!c || candidates < 0) return DM_E_INVAL;
+  c->launch_limit = candidates ? (uint32_t)candidates : 1u << 20;
   return DM_OK;
 }
 

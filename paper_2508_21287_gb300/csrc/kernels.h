@@ -123,7 +123,7 @@ struct ChainArgs {
   const int32_t *in_rows;
   const unsigned long long *in_blocks;
   int64_t in_cap;
-  unsigned limit;                // candidates after which a warp takes no further items
+  unsigned limit;                // candidates after which a warp takes no further items (first launch only)
   unsigned long long *ctr_last;  // CTR_N counters of the launch's last step, behind those of its others
   unsigned long long *h_out;     // where set (pinned host memory), the last block writes the n_out
   unsigned long long *done;      // counters there whose last CTR_N begin at done (one of them, zero
