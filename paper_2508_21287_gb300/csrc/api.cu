@@ -1451,6 +1451,7 @@ struct Exec {
         std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)(C.work / (CHAIN_ITEM_ROWS * (double)warps0))));
     F.chunk = std::min<int64_t>(32, std::max<int64_t>(1, (n0 + deal * warps0 - 1) / (deal * warps0)));
     F.seed_n = n0;
+    F.lo = 0;  // from the start, also after an attempt that overflowed in a later round
     float ms = 0.f;
     int64_t run_steps = 0, warps = 0;  // warps of the first launch
     for (bool more = true, first = true; more; first = false) {

@@ -65,3 +65,20 @@ def test_rows_and_best_rows(B, comb, length, budget):
             assert np.array_equal(again[0], best[0]) and np.array_equal(again[1], best[1])
         order = np.lexsort((np.arange(len(scores)), scores))[:50]
         assert np.array_equal(best[0], rows[order]) and np.array_equal(best[1], scores[order])
+
+
+def test_arena_that_overflows_in_a_later_round(B):
+    """61 M rows of 44 bytes in three rounds: two fit the first arena (rows in its half, 2 GB), the third does
+    not, and the joins begin again in a larger one."""
+    g, p = I.random_regular3(40000, 3), I.path(11)
+    ref = oracle.enumerate(g, p, threads=8, rows=False)
+    with B.Context(0) as c:
+        plan = c.plan(c.load(g), p)
+        B.dm_set_launch_limit(c.h, 1)
+        got = []
+        count, checksum = B.dm_match(c.h, plan.h, B.DM_ALL | B.DM_DEVICE_ROWS, lambda r, s, m, n: got.append((m, n)) or 0)
+        assert (count, checksum) == (ref.count, ref.checksum) and sum(m for m, _ in got) == ref.count
+        # the arena has grown: one attempt, three rounds
+        plan2 = c.plan(c.load(g), I.path(10))
+        B.dm_match(c.h, plan2.h, B.DM_ALL | B.DM_DEVICE_ROWS, lambda r, s, m, n: 0)
+        assert c.stats()["rows"][-1] == oracle.enumerate(g, I.path(10), threads=8, rows=False).count
