@@ -170,8 +170,8 @@ struct OrdSmem {
 };
 
 // Order the m rows of the bucket that starts at lo, by T threads (a warp or the block) that share the
-// places from `at` on (a multiple of 4), and write them out. LOCAL: the bucket's keys, less `base`, are
-// below 2^32 - 1 and decide alone.
+// places from `at` on (a multiple of 4), and write them out. LOCAL: the bucket's keys are not below `base`,
+// are below base + 2^32 - 1 and decide alone.
 template <int KW, int T, bool LOCAL>
 __device__ __forceinline__ void ord_bucket_out(const OrderArgs &a, OrdSmem<KW> &S, int at, int64_t lo, int m,
                                                unsigned long long base) {
@@ -275,13 +275,11 @@ __global__ void __launch_bounds__(ORD_BLK) k_ord_rank(const __grid_constant__ Or
   const int64_t n = ord_n(a);
   if (n == 0 || a.ctr[CTR_OVF]) return;
   const int nb = ord_buckets(n), wid = threadIdx.x >> 5;
-  // the keys of a bucket start at about range / nb * b: a bit below that, and their spread
-  const unsigned long long width = a.range / nb + 2;
-  const bool local = KW == 1 && a.packed == a.w && width < 0xFFFFFF00ull / 2;
-  auto base = [&](int b) {
-    const unsigned long long x = a.range / nb * (unsigned long long)b;
-    return x > width ? x - width : 0ull;
-  };
+  // bucket b holds the keys k with b <= k * scale * nb / 2^64 < b + 1: none below b * floor((2^64 - 1) / nb) /
+  // scale, which is at most ORD_MAX + 2 below the bucket's edge, and 2^64 / (nb * scale) + 1 of them at most
+  const unsigned long long cut = ~0ull / nb;
+  const bool local = KW == 1 && a.packed == a.w && cut / a.scale < 0xFFFFFFFFull - 2 * ORD_MAX;
+  auto base = [&](int b) { return cut * (unsigned long long)b / a.scale; };
   if (threadIdx.x == 0) s_large = 0;
   __syncthreads();
   for (int b = blockIdx.x * ORD_WARPS + wid; b < nb; b += gridDim.x * ORD_WARPS) {
