@@ -3692,12 +3692,12 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   // in the context's pinned buffer where it fits (a copy from other memory is made twice, and waited for)
   const int64_t per_epoch = (n + (int64_t)batch - 1) / batch, n_steps = per_epoch * epochs;
   if (n_steps > (int64_t)1 << 28) return DM_E_CAPACITY;
-  const size_t stage = sizeof(float) * ((size_t)n * (NFEAT + 1) + (size_t)n_steps + 1 + (size_t)n * epochs);
+  const size_t stage = sizeof(float) * ((size_t)n * (NFEAT + 1) + (size_t)n_steps + 2 + (size_t)n * epochs);
   const bool pinned = stage <= c->h_stage_bytes;
   std::vector<float> unpinned(pinned ? 0 : (stage + 3) / sizeof(float));
   float *hX = pinned ? (float *)c->h_stage : unpinned.data(), *hT = hX + (size_t)n * NFEAT, *hL = hT + n;
   unsigned *hE = (unsigned *)(hL + n_steps);
-  int32_t *hI = (int32_t *)(hE + 1);
+  int32_t *hI = (int32_t *)(hE + 2);
   normalise(c, feats, n, hX);
   memcpy(hT, targets, sizeof(float) * n);
   // one buffer for the call's tables, kept for the next call up to TRAIN_KEEP
@@ -3710,7 +3710,7 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   };
   const size_t atX = place(sizeof(float) * (size_t)n * NFEAT), atT = place(sizeof(float) * (size_t)n),
                atL = place(sizeof(float) * (size_t)n_steps), atI = place(sizeof(int32_t) * (size_t)n),
-               atE = place(sizeof(unsigned)), atW = place((size_t)dmk::mlp_train_bytes(rows));
+               atE = place(2 * sizeof(unsigned)), atW = place((size_t)dmk::mlp_train_bytes(rows));
   if (c->train_bytes < used) {
     dfree(c, c->train_buf);
     c->train_buf = nullptr;
@@ -3744,11 +3744,12 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   r = check(cudaMemcpyAsync(X, hX, sizeof(float) * (size_t)n * NFEAT, cudaMemcpyHostToDevice, c->stream));
   if (r == DM_OK) r = check(cudaMemcpyAsync(T, hT, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
   if (r == DM_OK) r = check(cudaMemsetAsync(L, 0, sizeof(float) * n_steps, c->stream));
-  if (r == DM_OK) r = check(cudaMemsetAsync(E, 0, sizeof(unsigned), c->stream));
+  if (r == DM_OK) r = check(cudaMemsetAsync(E, 0, 2 * sizeof(unsigned), c->stream));
   if (r == DM_OK) r = check(dmk::mlp_train_begin(A, c->stream));
   std::vector<int32_t> idx(n);
   for (int32_t i = 0; i < n; i++) idx[i] = i;
   uint64_t st = seed ^ 0xA5A5A5A5ull;
+  const int step0 = c->m_step;
   int64_t step = 0;
   for (int32_t ep = 0; ep < epochs && r == DM_OK; ep++) {
     for (int32_t i = n - 1; i > 0; i--) {  // Fisher-Yates with SplitMix64
@@ -3768,12 +3769,13 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
     }
   }
   if (r == DM_OK) r = check(cudaMemcpyAsync(hL, L, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, c->stream));
-  if (r == DM_OK) r = check(cudaMemcpyAsync(hE, E, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+  if (r == DM_OK) r = check(cudaMemcpyAsync(hE, E, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
   const cudaError_t se = cudaStreamSynchronize(c->stream);
   if (r == DM_OK) r = check(se);
   release(r);
   if (r != DM_OK) return r;
-  if (*hE) {
+  if (hE[0]) {  // the steps before it stand
+    c->m_step = step0 + (int)hE[1];
     c->last_error = "a tensor-core wait of the cardinality model timed out";
     return DM_E_TIMEOUT;
   }

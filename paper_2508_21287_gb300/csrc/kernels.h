@@ -376,7 +376,8 @@ unsigned *mlp_error_flag(void *work, int rows);
 cudaError_t mlp_forward_backward(const float *params, const float *X, const float *target, int rows, int n_valid,
                                  float *y, float *grads, float *loss, void *work, cudaStream_t s);
 // Training (mlp.cu): one Adam step on m samples (rows idx[0 .. m) of X and target) in two launches. The
-// launches before must be this stream's kernels or copies. err is raised as mlp_error_flag is; *loss is added to.
+// launches before must be this stream's kernels or copies. err[0] is raised as mlp_error_flag is, and no step is
+// taken once it is up; err[1] counts the steps taken. *loss is added to.
 struct MlpTrain {
   float *params, *m, *v;
   const float *X, *target;   // standardised samples, n x 32, and their targets

@@ -411,7 +411,7 @@ struct TrainSmemA {
   uint16_t h2[TR_M * (MLP_H + 8)];              // row-major, padded
   float b1[MLP_H], b2[MLP_H], w3[MLP_H], dy[TR_M];
   unsigned long long bar, load[2];              // products; the first and the second layer's weights
-  uint32_t tmem;
+  uint32_t tmem, stop;
 };
 
 // Block-wide wait for the MMAs committed to the barrier; false (and *err raised) when it ran out.
@@ -510,19 +510,21 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
   if (tid < MLP_H) S.b1[tid] = b1[tid];
   else if (tid < 2 * MLP_H) S.b2[tid - MLP_H] = b2[tid - MLP_H];
   else if (tid < 3 * MLP_H) S.w3[tid - 2 * MLP_H] = w3[tid - 2 * MLP_H];
+  else if (tid == 3 * MLP_H) S.stop = *(volatile unsigned *)T.err;  // a wait of an earlier step ran out: no more steps
   const float bias3 = b3[0];
   if (m0 + xr < rows) *(uint4 *)(T.Xb + tr_at(T.R, m0 + xr, xk)) = xin;  // kept for the weights of the first layer
   __syncthreads();
   const TrOp X{S.x, 128, 512, false}, L1{S.w1, 128, 512, false};
   const TrOp H1{S.h1, 128, 2048, false}, L2{S.w2, 128, 2048, false};  // h2 x h1, K = h1 ...
   const TrOp D2{S.d2, 128, 2048, false}, L2t{S.w2, 2048, 128, true};  // ... and backwards h1 x h2, K = h2
-  if (tid == 0 && tr_landed(tc_saddr(&S.load[0]), 0, T.err)) tr_mma(tmem, X, L1, MLP_H, MLP_IN, true, bar);
+  const bool stop = S.stop != 0;
+  if (tid == 0 && !stop && tr_landed(tc_saddr(&S.load[0]), 0, T.err)) tr_mma(tmem, X, L1, MLP_H, MLP_IN, true, bar);
   const int quad = warp & 3, c0 = 32 * (warp >> 2);  // a warp reads its lane quadrant (warp % 4)
   const int r = 32 * quad + lane;                    // this thread's row: columns c0 .. c0 + 31
   const bool live = m0 + r < rows;
   const uint32_t mine = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
   uint32_t v[32], on1 = 0, on2 = 0;  // signs of the pre-activations: the ReLU masks
-  bool ok = tr_wait(bar, phase, T.err);
+  bool ok = !stop && tr_wait(bar, phase, T.err);
   if (ok) {
     tr_ld32(mine, v);
 #pragma unroll
@@ -624,7 +626,10 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_rows(const MlpTrain T, 
       if (live) *(uint4 *)(T.dH1 + tr_at(T.R, m0 + r, (c0 >> 3) + q)) = make_uint4(h[0], h[1], h[2], h[3]);
     }
   }
-  else if (tid == 0) tr_landed(tc_saddr(&S.load[1]), 0, T.err);  // given up: its copy has still to land
+  else if (tid == 0) {  // given up: the copies have still to land
+    tr_landed(tc_saddr(&S.load[0]), 0, T.err);
+    tr_landed(tc_saddr(&S.load[1]), 0, T.err);
+  }
   tr_teardown(&S.bar, 3, tmem, COLS);
 }
 
@@ -643,7 +648,7 @@ struct TrainSmemB {
   float g[MLP_H * 33];                       // the block's gradient
   float part[256];
   unsigned long long bar, load;
-  uint32_t tmem;
+  uint32_t tmem, stop;
 };
 
 // Blocks 0 .. 3: columns 32 b .. of gW2; 4: gW1; then 4 blocks each for b1's, b2's and w3's gradients (32
@@ -663,6 +668,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
     griddep_launch_dependents();
     const int what = (b - 5) >> 2, c = 32 * ((b - 5) & 3) + (tid & 31);
     const bool sums = tid < 256;  // colsum32's eight warps; all threads take its barriers
+    const bool stop = *(volatile unsigned *)T.err != 0;
     float t = 0.f, u = 0.f;
     auto add = [&](const __nv_bfloat16 *M, const float *wrow) {
       float s = 0.f;
@@ -692,13 +698,17 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
       __syncthreads();
       if (tid == 0) {
         for (int k = 0; k < 8; k++) u += S.part[k * 32];
-        adam(ob3, u);
+        if (!stop) {
+          adam(ob3, u);
+          atomicAdd(T.err + 1, 1u);  // steps taken
+        }
       }
     }
-    if (tid < 32) adam((what == 0 ? ob1 : what == 1 ? ob2 : ow3) + c, t);
+    if (tid < 32 && !stop) adam((what == 0 ? ob1 : what == 1 ? ob2 : ow3) + c, t);
     return;
   }
   constexpr int COLS = 32;
+  if (tid == 0) S.stop = 0;
   tr_setup(&S.bar, 2, &S.tmem, COLS);
   const uint32_t tmem = S.tmem, bar = tc_saddr(&S.bar), load = tc_saddr(&S.load);
   griddep_wait();
@@ -734,9 +744,14 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_train_weights(const MlpTrain 
         am[j] = T.m[at];
         av[j] = T.v[at];
       }
-    if (tid == 0 && tr_landed(load, phase_l, T.err)) tr_mma(tmem, A, B, 32, kc, k0 == 0, bar);
+    if (tid == 0) {
+      if (k0 == 0) S.stop = *(volatile unsigned *)T.err;  // this step's activations are void, or an earlier step's were
+      const bool up = tr_landed(load, phase_l, T.err);
+      if (S.stop) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+      else if (up) tr_mma(tmem, A, B, 32, kc, k0 == 0, bar);
+    }
     phase_l ^= 1u;
-    ok = tr_wait(bar, phase, T.err);
+    ok = tr_wait(bar, phase, T.err) && !S.stop;
   }
   if (ok) {
     if (tid < 128) {
