@@ -351,7 +351,9 @@ int dm_model_init(dm_ctx *ctx, uint64_t seed);
 
 /* Train on n (features, log growth) samples with Adam (mini-batches of `batch` >= 16,
  * `epochs` passes, learning rate lr, shuffling seeded by `seed`), all on the GPU.
- * out_loss (nullable) receives the mean squared error of each epoch. */
+ * out_loss (nullable) receives the mean squared error of each epoch. The samples are on the device
+ * during the call where they take at most 64 MB or an eighth of the memory budget; of more samples
+ * every batch is brought by itself. Up to 64 MB of the call's tables stay with the context. */
 int dm_model_train(dm_ctx *ctx, const float *feats, const float *targets, int32_t n, int32_t epochs,
                    int32_t batch, float lr, uint64_t seed, float *out_loss);
 

@@ -2520,6 +2520,30 @@ void normalise(const dm_ctx *c, const float *x, int32_t n, std::vector<float> &o
   normalise(c, x, n, out.data());
 }
 
+// Training: bytes of device tables that a context keeps between calls, and steps whose losses wait on the
+// device before the host adds them up.
+constexpr size_t TRAIN_KEEP = 64ull << 20;
+constexpr int64_t TRAIN_LOSSES = 1 << 14;
+
+// Pieces of the context's pinned staging buffer, for copies of its stream. When the buffer is used up the
+// stream is waited for and the pieces begin again.
+struct Staging {
+  dm_ctx *c;
+  size_t used = 0;
+  size_t most() const { return c->h_stage_bytes / 4; }  // bytes of a piece
+  template <class T>
+  int take(size_t count, T **p) {
+    const size_t bytes = (count * sizeof(T) + 15) / 16 * 16;
+    if (used + bytes > c->h_stage_bytes) {
+      CK(cudaStreamSynchronize(c->stream));
+      used = 0;
+    }
+    *p = (T *)((unsigned char *)c->h_stage + used);
+    used += bytes;
+    return DM_OK;
+  }
+};
+
 // Predicted cost of a plan: bytes of every intermediate table it writes (rows from the chain
 // of predicted log growths, model or heuristic) plus 64 KiB per step for launch and barrier
 // overheads; and its largest predicted table.
@@ -3667,8 +3691,6 @@ int dm_model_grad(dm_ctx *c, const float *feats, const float *targets, int32_t n
   return DM_OK;
 }
 
-constexpr size_t TRAIN_KEEP = 64ull << 20;  // bytes of training tables that a context keeps between calls
-
 int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t n, int32_t epochs, int32_t batch,
                    float lr, uint64_t seed, float *out_loss) {
   if (!c || !feats || !targets || n < 1 || epochs < 1 || batch < 16) return DM_E_INVAL;
@@ -3688,29 +3710,22 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
       c->m_std[k] = var > 1e-12 ? (float)sqrt(var) : 1.f;
     }
   }
-  // everything the steps read is uploaded once; losses and the timeout flag come back in the end. Staged
-  // in the context's pinned buffer where it fits (a copy from other memory is made twice, and waited for)
+  // All samples go to the device once, standardised, where they take no more than TRAIN_KEEP or an eighth of the
+  // budget; otherwise every step brings its own. Everything passes through the pinned staging buffer (a copy
+  // from other memory is made twice, and waited for), and the host waits only when that or the losses' buffer is full.
   const int64_t per_epoch = (n + (int64_t)batch - 1) / batch, n_steps = per_epoch * epochs;
-  if (n_steps > (int64_t)1 << 28) return DM_E_CAPACITY;
-  const size_t stage = sizeof(float) * ((size_t)n * (NFEAT + 1) + (size_t)n_steps + 2 + (size_t)n * epochs);
-  const bool pinned = stage <= c->h_stage_bytes;
-  std::vector<float> unpinned(pinned ? 0 : (stage + 3) / sizeof(float));
-  float *hX = pinned ? (float *)c->h_stage : unpinned.data(), *hT = hX + (size_t)n * NFEAT, *hL = hT + n;
-  unsigned *hE = (unsigned *)(hL + n_steps);
-  int32_t *hI = (int32_t *)(hE + 2);
-  normalise(c, feats, n, hX);
-  memcpy(hT, targets, sizeof(float) * n);
-  // one buffer for the call's tables, kept for the next call up to TRAIN_KEEP
   const int rows = std::min(batch, n);
+  const bool resident = sizeof(float) * (NFEAT + 1) * (size_t)n <= std::max<size_t>(TRAIN_KEEP, (size_t)(c->budget / 8));
+  const size_t held = resident ? n : rows;  // samples, and indices, on the device
+  const size_t E_bytes = 2 * sizeof(unsigned) + sizeof(float) * (size_t)std::min(n_steps, TRAIN_LOSSES);
   size_t used = 0;
   auto place = [&](size_t bytes) {
     const size_t at = used;
     used += (bytes + 255) / 256 * 256;
     return at;
   };
-  const size_t atX = place(sizeof(float) * (size_t)n * NFEAT), atT = place(sizeof(float) * (size_t)n),
-               atL = place(sizeof(float) * (size_t)n_steps), atI = place(sizeof(int32_t) * (size_t)n),
-               atE = place(2 * sizeof(unsigned)), atW = place((size_t)dmk::mlp_train_bytes(rows));
+  const size_t atX = place(sizeof(float) * held * (NFEAT + 1)), atI = place(sizeof(int32_t) * held), atE = place(E_bytes),
+               atW = place((size_t)dmk::mlp_train_bytes(rows));
   if (c->train_bytes < used) {
     dfree(c, c->train_buf);
     c->train_buf = nullptr;
@@ -3719,19 +3734,10 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
     c->train_bytes = used;
   }
   unsigned char *buf = (unsigned char *)c->train_buf;
-  float *X = (float *)(buf + atX), *T = (float *)(buf + atT), *L = (float *)(buf + atL);
+  float *X = (float *)(buf + atX), *T = X + held * NFEAT;
   int32_t *I = (int32_t *)(buf + atI);
   unsigned *E = (unsigned *)(buf + atE);
-  void *work = buf + atW;
-  auto release = [&](int r) {
-    if (c->train_bytes > TRAIN_KEEP) {
-      dfree(c, c->train_buf);
-      c->train_buf = nullptr;
-      c->train_bytes = 0;
-    }
-    return r;
-  };
-  int r = DM_OK;
+  float *L = (float *)(E + 2);  // behind the flag and the count: they come back together
   dmk::MlpTrain A{};
   A.params = c->m_params;
   A.m = c->m_m;
@@ -3739,54 +3745,104 @@ int dm_model_train(dm_ctx *c, const float *feats, const float *targets, int32_t 
   A.X = X;
   A.target = T;
   A.err = E;
-  dmk::mlp_train_layout(A, work, rows);
-  auto check = [&](cudaError_t e) { return e == cudaSuccess ? DM_OK : cuda_fail(c, e, "model training"); };
-  r = check(cudaMemcpyAsync(X, hX, sizeof(float) * (size_t)n * NFEAT, cudaMemcpyHostToDevice, c->stream));
-  if (r == DM_OK) r = check(cudaMemcpyAsync(T, hT, sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
-  if (r == DM_OK) r = check(cudaMemsetAsync(L, 0, sizeof(float) * n_steps, c->stream));
-  if (r == DM_OK) r = check(cudaMemsetAsync(E, 0, 2 * sizeof(unsigned), c->stream));
-  if (r == DM_OK) r = check(dmk::mlp_train_begin(A, c->stream));
+  dmk::mlp_train_layout(A, buf + atW, rows);
+  Staging stage{c};
   std::vector<int32_t> idx(n);
   for (int32_t i = 0; i < n; i++) idx[i] = i;
-  uint64_t st = seed ^ 0xA5A5A5A5ull;
+  auto put_samples = [&](const int32_t *which, int32_t m) -> int {  // the first m of them, or those at which[0 .. m)
+    const int32_t per = (int32_t)(stage.most() / (sizeof(float) * (NFEAT + 1)));
+    for (int32_t lo = 0, k; lo < m; lo += k) {
+      k = std::min(per, m - lo);
+      float *h;
+      RET(stage.take((size_t)k * (NFEAT + 1), &h));
+      float *ht = h + (size_t)k * NFEAT;
+      if (!which) {
+        normalise(c, feats + (size_t)lo * NFEAT, k, h);
+        memcpy(ht, targets + lo, sizeof(float) * k);
+      } else {
+        for (int32_t i = 0; i < k; i++) {
+          normalise(c, feats + (size_t)which[lo + i] * NFEAT, 1, h + (size_t)i * NFEAT);
+          ht[i] = targets[which[lo + i]];
+        }
+      }
+      // the targets lie behind the samples on both sides: one copy where a piece is all there is room for
+      const size_t xs = (size_t)k * NFEAT + ((size_t)k == held ? k : 0);
+      CK(cudaMemcpyAsync(X + (size_t)lo * NFEAT, h, sizeof(float) * xs, cudaMemcpyHostToDevice, c->stream));
+      if ((size_t)k < held) CK(cudaMemcpyAsync(T + lo, ht, sizeof(float) * k, cudaMemcpyHostToDevice, c->stream));
+    }
+    return DM_OK;
+  };
+  auto put_indices = [&](int32_t m) -> int {  // idx[0 .. m)
+    for (int32_t lo = 0, k; lo < m; lo += k) {
+      k = std::min((int32_t)(stage.most() / sizeof(int32_t)), m - lo);
+      int32_t *h;
+      RET(stage.take((size_t)k, &h));
+      memcpy(h, idx.data() + lo, sizeof(int32_t) * k);
+      CK(cudaMemcpyAsync(I + lo, h, sizeof(int32_t) * k, cudaMemcpyHostToDevice, c->stream));
+    }
+    return DM_OK;
+  };
   const int step0 = c->m_step;
-  int64_t step = 0;
-  for (int32_t ep = 0; ep < epochs && r == DM_OK; ep++) {
-    for (int32_t i = n - 1; i > 0; i--) {  // Fisher-Yates with SplitMix64
-      st += 0x9E3779B97F4A7C15ull;
-      uint64_t z = st;
-      z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-      z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-      z ^= z >> 31;
-      std::swap(idx[i], idx[(int32_t)(z % (uint64_t)(i + 1))]);
+  int64_t step = 0, added = 0;  // steps queued, and those whose losses are added up
+  double sum = 0;
+  auto add_losses = [&]() -> int {
+    const int64_t k = step - added;
+    unsigned *he;
+    RET(stage.take((size_t)k + 2, &he));
+    const float *h = (const float *)(he + 2);
+    CK(cudaMemcpyAsync(he, E, sizeof(float) * (k + 2), cudaMemcpyDeviceToHost, c->stream));
+    if (step < n_steps) CK(cudaMemsetAsync(L, 0, sizeof(float) * k, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    stage.used = 0;
+    if (he[0]) {  // the steps before it stand
+      c->m_step = step0 + (int)he[1];
+      c->last_error = "a tensor-core wait of the cardinality model timed out";
+      return DM_E_TIMEOUT;
     }
-    int32_t *hi = hI + (size_t)ep * n;
-    memcpy(hi, idx.data(), sizeof(int32_t) * n);
-    r = check(cudaMemcpyAsync(I, hi, sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream));
-    for (int32_t b0 = 0; b0 < n && r == DM_OK; b0 += batch) {
-      c->m_step++;
-      r = check(dmk::mlp_train_step(A, I + b0, std::min(batch, n - b0), L + step++, lr, c->m_step, c->stream));
+    for (int64_t i = 0; i < k; i++, added++) {
+      const int64_t b = added % per_epoch;
+      sum += (double)h[i] * std::min<int64_t>(batch, n - b * batch);
+      if (b + 1 < per_epoch) continue;
+      if (out_loss) out_loss[added / per_epoch] = (float)(sum / n);
+      sum = 0;
     }
+    return DM_OK;
+  };
+  auto train = [&]() -> int {
+    if (resident) RET(put_samples(nullptr, n));
+    else RET(put_indices(rows));
+    CK(cudaMemsetAsync(E, 0, E_bytes, c->stream));
+    CK(dmk::mlp_train_begin(A, c->stream));
+    uint64_t st = seed ^ 0xA5A5A5A5ull;
+    for (int32_t ep = 0; ep < epochs; ep++) {
+      for (int32_t i = n - 1; i > 0; i--) {  // Fisher-Yates with SplitMix64
+        st += 0x9E3779B97F4A7C15ull;
+        uint64_t z = st;
+        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+        z ^= z >> 31;
+        std::swap(idx[i], idx[(int32_t)(z % (uint64_t)(i + 1))]);
+      }
+      if (resident) RET(put_indices(n));
+      for (int64_t b0 = 0; b0 < n; b0 += batch) {
+        const int32_t m = (int32_t)std::min<int64_t>(batch, n - b0);
+        if (!resident) RET(put_samples(idx.data() + b0, m));
+        c->m_step++;
+        CK(dmk::mlp_train_step(A, resident ? I + b0 : I, m, L + (step - added), lr, c->m_step, c->stream));
+        if (++step - added == TRAIN_LOSSES) RET(add_losses());
+      }
+    }
+    return step > added ? add_losses() : DM_OK;
+  };
+  const int r = train();
+  if (r != DM_OK) cudaStreamSynchronize(c->stream);  // what is queued still reads the staging buffer
+  if (c->train_bytes > TRAIN_KEEP) {
+    dfree(c, c->train_buf);
+    c->train_buf = nullptr;
+    c->train_bytes = 0;
   }
-  if (r == DM_OK) r = check(cudaMemcpyAsync(hL, L, sizeof(float) * n_steps, cudaMemcpyDeviceToHost, c->stream));
-  if (r == DM_OK) r = check(cudaMemcpyAsync(hE, E, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-  const cudaError_t se = cudaStreamSynchronize(c->stream);
-  if (r == DM_OK) r = check(se);
-  release(r);
-  if (r != DM_OK) return r;
-  if (hE[0]) {  // the steps before it stand
-    c->m_step = step0 + (int)hE[1];
-    c->last_error = "a tensor-core wait of the cardinality model timed out";
-    return DM_E_TIMEOUT;
-  }
-  for (int32_t ep = 0; ep < epochs && out_loss; ep++) {
-    double sum = 0;
-    for (int64_t k = 0; k < per_epoch; k++)
-      sum += (double)hL[ep * per_epoch + k] * std::min<int64_t>(batch, n - k * batch);
-    out_loss[ep] = (float)(sum / n);
-  }
-  c->m_trained = true;
-  return DM_OK;
+  if (r == DM_OK) c->m_trained = true;
+  return r;
 }
 
 int dm_model_predict(dm_ctx *c, const float *feats, int32_t n, float *out) {
