@@ -93,7 +93,8 @@ typedef struct dm_plan_opts {
  * dataframe library's memory pool): a context owns a stream, counters and the device memory
  * of its graphs and tables. mem_budget_bytes bounds the device memory the intermediate tables
  * of one dm_match may hold (0 = half of the free memory at creation); larger results are
- * streamed in chunks (depth-first over the join steps). Errors: DM_E_INVAL (out NULL),
+ * streamed in chunks (depth-first over the join steps). Tables of what a plan's candidates bring
+ * stay with the context beside that, at most an eighth of the budget and 256 MB. Errors: DM_E_INVAL (out NULL),
  * DM_E_CUDA (no such device, or stream/event creation failed), DM_E_NOMEM. */
 int dm_create(dm_ctx **out, int device, uint64_t mem_budget_bytes);
 

@@ -506,6 +506,9 @@ struct StepRT {
 constexpr int CHAIN_SM_BYTES = 224 * 1024;
 constexpr int CHAIN_WARPS = 16;
 constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20, CHAIN_TAB_MIN = 4ll << 20;
+// ... which a context keeps between calls, beside the arena: an eighth of its budget at most. A plan that needs
+// more runs a launch a step.
+int64_t chain_tab_limit(uint64_t budget) { return std::min<int64_t>(CHAIN_TAB_BYTES, (int64_t)(budget / 8)); }
 constexpr double CHAIN_LAUNCH_NS = 4000, CHAIN_ROW_NS = 0.03, CHAIN_BYTE_NS = 0.0002;
 // Rows of work that an item of a launch's input stands for at the least: each further item is a turn
 // at one counter that all warps share. A 7-vertex tree on 2640 vertices (31 656 first rows, 0.25 M
@@ -1349,12 +1352,12 @@ struct Exec {
         for (int q = 0; q < la.wo; q++) A.out_off[q] = off(at[S][la.src_col[q]]);
     }
     C.needs_arena = C.launch.size() > 1 || !count_mode;
-    return C.tab_bytes <= CHAIN_TAB_BYTES;
+    return C.tab_bytes <= chain_tab_limit(c->budget);
   }
 
   int ensure_tables(int64_t bytes) {
     if (c->tab_bytes >= bytes) return DM_OK;
-    bytes = std::max(bytes, CHAIN_TAB_MIN);  // so that the next plan finds room as well
+    bytes = std::max(bytes, std::min(CHAIN_TAB_MIN, chain_tab_limit(c->budget)));  // so that the next plan finds room as well
     dfree(c, c->tabs);  // in stream order: behind what still reads it
     c->tabs = nullptr;
     c->tab_bytes = 0;
@@ -2813,6 +2816,11 @@ int dm_set_budget(dm_ctx *c, uint64_t bytes) {
     bytes = fr / 2;
   }
   c->budget = bytes;
+  if (c->tab_bytes > chain_tab_limit(bytes)) {
+    dfree(c, c->tabs);
+    c->tabs = nullptr;
+    c->tab_bytes = 0;
+  }
   return DM_OK;
 }
 
