@@ -510,6 +510,8 @@ constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20, CHAIN_TAB_MIN = 4ll << 20;
 // more runs a launch a step.
 int64_t chain_tab_limit(uint64_t budget) { return std::min<int64_t>(CHAIN_TAB_BYTES, (int64_t)(budget / 8)); }
 constexpr double CHAIN_LAUNCH_NS = 4000, CHAIN_ROW_NS = 0.03, CHAIN_BYTE_NS = 0.0002;
+// The smallest arena that tables go into: the parts it is cut into then hold a block or a row of any width.
+constexpr size_t ARENA_MIN = 64 << 10;
 // Rows of work that an item of a launch's input stands for at the least: each further item is a turn
 // at one counter that all warps share. A 7-vertex tree on 2640 vertices (31 656 first rows, 0.25 M
 // embeddings) took 53 us in eight items a warp, 47 without the rounding to whole rows, 36.5 at 32 rows an
@@ -1590,7 +1592,7 @@ struct Exec {
       size_t want = std::max<size_t>(c->arena_bytes, (size_t)4 << 30);
       while (true) {
         want = std::min<size_t>(want, (size_t)c->budget);
-        if (ensure_arena(want) != DM_OK) break;
+        if (want < ARENA_MIN || ensure_arena(want) != DM_OK) break;
         bool fits = false;
         dm_stats saved = c->stats;
         RET(chain ? run_chain(C, &fits) : run_fast(&fits));

@@ -30,3 +30,18 @@ def test_candidate_tables_within_the_budget(B):
             launches.setdefault(budget, c.stats()["kernel_launches"])
             assert c.stats()["kernel_launches"] == launches[budget]
         assert launches[0] == launches[64 << 20] == 2 < launches[16 << 20]
+
+
+@pytest.mark.parametrize("budget", [1, 600, 1500, 6000, 20000, 65535, 65536, 70000])
+def test_budgets_below_a_table(B, budget):
+    # wide rows and tables between launches (the long paths), where not even one of them fits
+    for g, lengths in ((I.cycle(12), (5, 12)), (I.cycle(70), (31, 60)), (I.heavy_hex(2, 2), (6, 9))):
+        g = I.lognormal_weights(g, 4)
+        with B.Context(0, budget) as c:
+            gid = c.load(g)
+            for n in lengths:
+                plan, ref = c.plan(gid, I.path(n)), oracle.enumerate(g, I.path(n))
+                assert plan.count() == (ref.count, ref.checksum)
+                rows, _, cnt, cs = plan.all()
+                assert (cnt, cs) == (ref.count, ref.checksum) == (len(rows), ref.checksum)
+                assert sorted(map(tuple, rows)) == sorted(map(tuple, ref.rows))
