@@ -33,6 +33,7 @@ struct DevTable {
   int64_t n = 0;
   int32_t w = 0;
   bool borrowed = false;  // lives in the context's arena: never freed by its holder
+  bool even = false;      // rows of launches of several steps, whose keys spread (order.cu)
   int64_t held = 0;       // bytes counted against the memory budget while it lives
 };
 
@@ -478,8 +479,6 @@ struct Sink {
     int64_t spare_bytes;
     unsigned long long *ctr;          // CTR_N zeroed counters, which come back with the joins' own
     const unsigned long long *h_ctr;
-    const Plan *p;
-    DevGraph *g;
   };
   virtual int ahead(dm_ctx *, const Ahead &) { return DM_OK; }
   virtual bool counts() const { return true; }  // ahead() uses those counters
@@ -1493,8 +1492,6 @@ struct Exec {
         a.spare_bytes = (int64_t)half;
         a.ctr = c->d_ctr_steps + (size_t)S * CTR_N;
         a.h_ctr = c->h_ctr_steps + (size_t)S * CTR_N;
-        a.p = p;
-        a.g = g;
         RET(sink->ahead(c, a));
       }
       if (!C.launch.back().h_out)
@@ -1557,6 +1554,7 @@ struct Exec {
     t.n = (int64_t)hl[CTR_ROWS];
     t.w = A.wo;
     t.borrowed = true;
+    t.even = true;
     return sink->take(c, t);
   }
 
@@ -1704,24 +1702,94 @@ struct AllSink : Sink {
   float *final_scores = nullptr;
   bool final_done = false;
   int64_t final_n = 0;
-  // sort (checksum fused into the key packing), one synchronisation, delivery, then the top-k
-  // tap (which takes the table over). last: no table follows, nothing was flushed before.
+  const Plan *p = nullptr;
+  DevGraph *g = nullptr;
+  // the rows' keys crowd: too many in a bucket behind the joins (finer buckets are tried next), and in those
+  // as well (later tables are sorted by comparison at once)
+  bool crowded = false, very_crowded = false;
+  // order, checksum, one synchronisation, delivery, then the top-k tap (which takes the table over).
+  // last: no table follows, nothing was flushed before.
   int flush_one(dm_ctx *c, DevTable &t, bool last = false) {
     CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(unsigned long long) * CTR_N, c->stream));
-    RET(sort_canonical(c, t, bits, c->d_ctr));
+    DevTable o;
+    bool keyed = t.even && !very_crowded && t.n > dmk::msort_into_max_rows() && t.n <= dmk::ORD_ROWS && order_table(c, t, &o) == DM_OK;
+    if (!keyed) RET(sort_canonical(c, t, bits, c->d_ctr));
     const bool fast_topk = last && tap && final_rows && topk_small_enough(tap);
     const int64_t k = fast_topk ? topk_k(tap) : 0;
-    if (fast_topk && t.n > 0) RET(topk_enqueue(c, k, t, nullptr, true));
+    if (fast_topk && t.n > 0) RET(topk_enqueue(c, k, keyed ? o : t, nullptr, true));
     RET(read_ctr(c));
+    checksum += c->h_ctr[CTR_SUM];
+    if (keyed && c->h_ctr[CTR_OVF]) {
+      very_crowded = true;
+      free_table(c, o);
+      RET(sort_canonical(c, t, bits));
+      if (fast_topk) RET(topk_enqueue(c, k, t, nullptr, true));
+      CK(cudaStreamSynchronize(c->stream));
+    } else if (keyed) {
+      free_table(c, t);
+      t = o;
+    }
     if (fast_topk) {
       final_n = std::min(k, t.n);
       final_done = t.n == 0 || topk_enqueued(c, k, t.n, t.w, final_rows, final_scores);
     }
     count += (uint64_t)t.n;
-    checksum += c->h_ctr[CTR_SUM];
     int r = deliver(c, t, flags, cb, user, true);
     if (r == DM_OK && tap && !final_done) return topk_take(c, tap, t);  // the tap takes ownership
     free_table(c, t);
+    return r;
+  }
+  // The keys of table t in o (order.cu); returns their words, or a negative error.
+  int order_keys(dm_ctx *c, const DevTable &t, dmk::OrderArgs &o) {
+    o.rows = t.rows;
+    o.sc = t.score;
+    o.w = t.w;
+    o.adj4 = g->adj4;
+    // a column's code is its place among the neighbours of an earlier column's vertex, where that is short
+    const int place = std::max(2, g->max_deg);
+    for (int32_t col = 0; col < t.w; col++) {
+      o.ref[col] = dmk::ORD_NONE;
+      for (int32_t e = p->rp[col]; e < p->rp[col + 1] && g->adj4; e++)
+        if (p->ci[e] < col) o.ref[col] = (uint8_t)p->ci[e];
+    }
+    if (!c->ord_work) {
+      RET(dalloc(c, &c->ord_work, (size_t)dmk::order_work_bytes()));
+      CK(cudaMemsetAsync(c->ord_work, 0, (size_t)dmk::order_work_bytes(), c->stream));
+    }
+    o.work = (dmk::OrderWork *)c->ord_work;
+    return dmk::order_layout(o, (unsigned)std::max(2, g->V), (unsigned)place);
+  }
+  // Places of the keys, numbers and indices of o.cap rows from `at` on; returns what lies behind them.
+  static unsigned char *order_place(dmk::OrderArgs &o, int kw, void *at) {
+    o.key = (unsigned long long *)at;
+    o.num = (int32_t *)(o.key + kw * o.cap);
+    o.idx = o.num + o.cap;
+    return (unsigned char *)(o.idx + o.cap);
+  }
+  // t in canonical order as a table of its own, enqueued; its checksum and CTR_OVF (then *out is void) go to d_ctr.
+  int order_table(dm_ctx *c, const DevTable &t, DevTable *out) {
+    dmk::OrderArgs o{};
+    const int kw = order_keys(c, t, o);
+    if (kw < 0) return kw;
+    DevTable s;
+    s.n = o.n = o.cap = t.n;
+    if (crowded) o.log2_many = dmk::ORD_FINE;
+    s.w = t.w;
+    void *tmp = nullptr;
+    int r = dalloc(c, &tmp, (size_t)t.n * (8 * kw + 8));
+    if (r == DM_OK) r = dalloc_t(c, &s.rows, (size_t)t.n * t.w);
+    if (r == DM_OK && t.score) r = dalloc_t(c, &s.score, t.n);
+    if (r == DM_OK) {
+      order_place(o, kw, tmp);
+      o.out = s.rows;
+      o.outs = s.score;
+      o.ctr = c->d_ctr;
+      const cudaError_t e = dmk::order_rows(o, kw, c->num_sms, c->stream);
+      if (e != cudaSuccess) r = cuda_fail(c, e, "canonical order");
+    }
+    dfree(c, tmp);
+    if (r == DM_OK) *out = s;
+    else free_table(c, s);
     return r;
   }
   // The only table, put into canonical order on the device behind the joins (order.cu): the sorted rows,
@@ -1732,33 +1800,12 @@ struct AllSink : Sink {
   int ahead(dm_ctx *c, const Ahead &a) override {
     const int64_t w = a.t.w;
     dmk::OrderArgs o{};
-    o.rows = a.t.rows;
-    o.sc = a.t.score;
     o.n_dev = a.n_dev;
-    o.w = (int32_t)w;
-    o.adj4 = a.g->adj4;
-    // a column's code is its place among the neighbours of an earlier column's vertex, where that is short
-    const int place = std::max(2, a.g->max_deg);
-    for (int32_t col = 0; col < w; col++) {
-      o.ref[col] = dmk::ORD_NONE;
-      for (int32_t e = a.p->rp[col]; e < a.p->rp[col + 1] && a.g->adj4; e++)
-        if (a.p->ci[e] < col) o.ref[col] = (uint8_t)a.p->ci[e];
-    }
-    const int kw = dmk::order_layout(o, (unsigned)std::max(2, a.g->V), (unsigned)place);
-    o.cap = std::min<int64_t>(a.t.n, (a.spare_bytes - 2048) / (4 * w + 4 + 8 * kw + 8)) / 64 * 64;
+    const int kw = order_keys(c, a.t, o);
+    if (kw < 0) return kw;
+    o.cap = std::min({a.t.n, (a.spare_bytes - 2048) / (4 * w + 4 + 8 * kw + 8), dmk::ORD_ROWS}) / 64 * 64;
     if (o.cap < 64) return DM_OK;
-    if (!c->ord_work) {
-      RET(dalloc(c, &c->ord_work, (size_t)dmk::order_work_bytes()));
-      CK(cudaMemsetAsync(c->ord_work, 0, (size_t)dmk::order_work_bytes(), c->stream));
-    }
-    o.work = (dmk::OrderWork *)c->ord_work;
-    unsigned char *at = a.spare;
-    o.key = (unsigned long long *)at;
-    at += 8 * kw * o.cap;
-    o.num = (int32_t *)at;
-    at += 4 * o.cap;
-    o.idx = (int32_t *)at;
-    at += 4 * o.cap;
+    unsigned char *at = order_place(o, kw, a.spare);
     o.out = (int32_t *)at;
     at += 4 * w * o.cap;
     o.outs = a.t.score ? (float *)at : nullptr;
@@ -1790,6 +1837,7 @@ struct AllSink : Sink {
       if (r == DM_OK && tap && !final_done) r = topk_take(c, tap, sorted);
       return r;
     }
+    crowded = tried && h_ahead[CTR_OVF] && t.n <= sorted.n;
     if (!streaming && held_bytes + tb <= (int64_t)c->budget / 2) {
       held.push_back(t);
       held_bytes += tb;
@@ -3260,6 +3308,8 @@ int dm_match(dm_ctx *c, const dm_plan_t *pl, int mode, dm_chunk_cb cb, void *use
   sink.cb = cb;
   sink.user = user;
   sink.bits = graph_bits(g);
+  sink.p = &pl->p;
+  sink.g = g;
   ex.sink = &sink;
   int r = ex.run();
   uint64_t cnt = ex.count, cs = ex.checksum;
@@ -3621,6 +3671,8 @@ int dm_match_topk(dm_ctx *c, const dm_plan_t *pl, int mode, dm_chunk_cb cb, void
   sink.cb = cb;
   sink.user = user;
   sink.bits = graph_bits(g);
+  sink.p = &pl->p;
+  sink.g = g;
   sink.tap = &tk;
   sink.final_rows = out_rows;
   sink.final_scores = out_scores;

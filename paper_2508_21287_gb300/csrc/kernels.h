@@ -247,8 +247,12 @@ cudaError_t msort_rows(const int32_t *rows, int64_t n, int32_t w, int bits, void
 
 // Canonical order of a table of embeddings whose row count is on the device (order.cu). The counters
 // ctr[CTR_SUM] (zeroed by the caller) and ctr[CTR_OVF] receive the rows' checksum and whether the order
-// was given up (more than cap rows, or a bucket too full; nothing usable is written then).
-constexpr int ORD_KW = 4, ORD_MAX = 16384, ORD_BUCKET = 1024;  // words of a key, buckets, rows of one
+// was given up (more than cap rows, or a bucket too full; no rows are written then, and the checksum only in the
+// second case).
+constexpr int ORD_KW = 4, ORD_MAX = 1 << 20;             // words of a key, buckets
+constexpr int ORD_BUCKET = 1024, ORD_CROWDED = 4096;     // most rows of a bucket, with n_dev and without
+constexpr int64_t ORD_ROWS = (int64_t)ORD_MAX * ORD_BUCKET;
+constexpr int ORD_FINE = 2;                              // log2 rows a bucket, for keys that crowd
 constexpr uint8_t ORD_NONE = 255;
 struct OrderWork {
   uint32_t count[ORD_MAX];           // zero between calls
@@ -259,11 +263,12 @@ struct OrderArgs {
   const float *sc;                   // nullable
   int64_t n;                         // rows, unless n_dev says it
   const unsigned long long *n_dev;
-  int64_t cap;                       // rows key, num, idx, out and outs have room for
+  int64_t cap;                       // rows key, num, idx, out and outs have room for, at most ORD_ROWS
   int32_t w, packed;                 // packed: columns held in the key
+  int32_t log2_many;                 // rows a bucket of large tables (order_layout), fewer where keys crowd
   const uint2 *adj4;                 // neighbour lists of the data graph, for columns with ref
   int32_t radix_id, radix_place;     // of a column's id, and of its place among an earlier one's neighbours
-  unsigned long long range, scale;   // the first word is below range; times scale, its fraction of 2^64
+  unsigned long long scale;          // the first word times scale is its fraction of 2^64
   uint8_t ref[dmi::MAXW];            // an earlier column that is a pattern neighbour, or ORD_NONE
   uint8_t word[dmi::MAXW];
   OrderWork *work;

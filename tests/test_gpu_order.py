@@ -31,3 +31,58 @@ def test_wide_buckets(B, side):
         np.testing.assert_allclose(scores, oracle.scores(g, p, ref.rows), rtol=1.5e-6, atol=0)
         plan.count()
         assert launches <= c.stats()["kernel_launches"] + 6  # ordered behind the joins, not sorted afterwards
+
+
+# tables of more than 64 rows for each of the first 16 384 buckets (several turns of the scan), behind the
+# joins and, where the arena has no room for that, in memory of their own
+@pytest.mark.parametrize("length,budget", [(7, 0), (7, 128 << 20), (8, 0), (8, 200 << 20)])
+@pytest.mark.parametrize("weights", [False, True])
+def test_many_buckets(B, length, budget, weights):
+    g, p = I.random_regular3(20000, 3), I.path(length)
+    if weights:
+        g = I.lognormal_weights(g, 2)
+    ref = oracle.enumerate(g, p, threads=8)
+    with B.Context(0, budget) as c:
+        plan = c.plan(c.load(g, weights), p)
+        rows, scores, cnt, cs = plan.all()
+        assert (cnt, cs) == (ref.count, ref.checksum)
+        if c.stats()["chunks"] > c.stats()["n_steps"]:  # streamed: chunks are sorted one by one
+            rows = rows[np.lexsort(rows.T[::-1])]
+        assert np.array_equal(rows, ref.rows)
+        if weights:
+            top_rows, top, cnt, cs = B.dm_match_topk(c.h, plan.h, B.DM_ALL, None, 50, p.n)
+            assert (cnt, cs) == (ref.count, ref.checksum)
+            rows, scores, _, _ = plan.all()
+            order = np.lexsort((*rows.T[::-1], scores))[:50]
+            assert np.array_equal(top_rows, rows[order]) and np.array_equal(top, scores[order])
+
+
+def corner(m, n):
+    """An m x m grid with a path behind its first vertex, n vertices in all: squares lie in a few ids of many."""
+    e = [(r * m + c, r * m + c + 1) for r in range(m) for c in range(m - 1)]
+    e += [(r * m + c, r * m + c + m) for r in range(m - 1) for c in range(m)]
+    return I.from_edges(n, e + [(0, m * m)] + [(i, i + 1) for i in range(m * m, n - 1)])
+
+
+# a square with a tail of that many vertices, columns as they are and scrambled: rows of the fullest bucket
+# within 4096 (ordered at the second attempt) and beyond (sorted by comparison)
+@pytest.mark.parametrize("side,tail,within", [(16, 4, True), (12, 5, True), (12, 6, None), (8, 6, False)])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_crowded_keys(B, side, tail, within, seed):
+    g = I.lognormal_weights(corner(side, 60000), 2)
+    p = I.from_edges(4 + tail, [(0, 1), (1, 2), (2, 3), (0, 3), (3, 4)] + [(i, i + 1) for i in range(4, 3 + tail)])
+    if seed:
+        p = I.relabel(p, np.random.RandomState(seed).permutation(p.n))
+    ref = oracle.enumerate(g, p, threads=8)
+    with B.Context(0) as c:
+        plan = c.plan(c.load(g), p)
+        for _ in range(2):
+            rows, scores, cnt, cs = plan.all()
+            assert (cnt, cs) == (ref.count, ref.checksum) and np.array_equal(rows, ref.rows)
+            again = c.stats()["kernel_launches"]
+            top_rows, top, cnt, cs = B.dm_match_topk(c.h, plan.h, B.DM_ALL, None, 50, p.n)
+            assert (cnt, cs) == (ref.count, ref.checksum)
+            order = np.lexsort((np.arange(len(scores)), scores))[:50]
+            assert np.array_equal(top_rows, rows[order]) and np.array_equal(top, scores[order])
+        if within is not None:
+            assert (again <= 10) == within  # two attempts of four launches behind the joins, and no sort
