@@ -66,7 +66,7 @@ struct DevGraph {
   // girth, and whether every cycle is even
   int32_t girth = 3;
   bool bipartite = false;
-  uint2 *adj4 = nullptr;  // neighbour lists of 16-bit ids, where no degree is above 4
+  uint2 *adj4 = nullptr;  // neighbour lists of 16-bit ids, where no degree is above 4 (in row_ptr's allocation)
   double edge_deg = 0;  // mean degree of the vertices that edges lead to
   std::map<int, DevTable> motifs;
   std::map<std::tuple<int, int, int, int>, Index> indices;  // (motif, key position 0, 1, sort-merge)
@@ -228,44 +228,31 @@ int validate_csr(int32_t n, const int32_t *rp, const int32_t *ci, const float *e
   return DM_OK;
 }
 
-bool connected(const HostCSR &g, int32_t n) {
+// bipartite (nullable): whether the part that 0 is in has no odd cycle.
+bool connected(const HostCSR &g, int32_t n, bool *bipartite = nullptr) {
+  if (bipartite) *bipartite = true;
   if (n <= 1) return true;
-  std::vector<char> seen(n, 0);
+  std::vector<char> seen(n, 0);  // 1 or 2: colour of a vertex seen
   std::vector<int32_t> st{0};
   seen[0] = 1;
   int32_t cnt = 1;
+  bool odd = false;
   while (!st.empty()) {
     int32_t u = st.back();
     st.pop_back();
-    for (int32_t k = g.rp[u]; k < g.rp[u + 1]; k++)
-      if (!seen[g.ci[k]]) {
-        seen[g.ci[k]] = 1;
+    const char other = 3 - seen[u];
+    for (int32_t k = g.rp[u]; k < g.rp[u + 1]; k++) {
+      char &v = seen[g.ci[k]];
+      if (!v) {
+        v = other;
         cnt++;
         st.push_back(g.ci[k]);
       }
-  }
-  return cnt == n;
-}
-
-// Whether a connected graph has no odd cycle.
-bool two_colourable(const HostCSR &g, int32_t n) {
-  std::vector<signed char> col(n, -1);
-  std::vector<int32_t> st{0};
-  col[0] = 0;
-  while (!st.empty()) {
-    const int32_t u = st.back();
-    st.pop_back();
-    for (int32_t k = g.rp[u]; k < g.rp[u + 1]; k++) {
-      const int32_t v = g.ci[k];
-      if (col[v] < 0) {
-        col[v] = 1 - col[u];
-        st.push_back(v);
-      } else if (col[v] == col[u]) {
-        return false;
-      }
+      odd |= v != other;
     }
   }
-  return true;
+  if (bipartite) *bipartite = !odd;
+  return cnt == n;
 }
 
 // ------------------------------------------------------------------ sorting ------------
@@ -2782,7 +2769,6 @@ void free_graph(dm_ctx *c, DevGraph *g) {
     if (kv.second.slots) dfree(c, kv.second.slots);
     if (kv.second.keys) dfree(c, kv.second.keys);
   }
-  dfree(c, g->adj4);
   cudaFree(g->row_ptr);
   cudaFree(g->col_idx);
   cudaFree(g->eerr);
@@ -2939,8 +2925,10 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
       for (int32_t v = 0; v < n; v++)
         if (!(qubit_err[v] >= 0.f && qubit_err[v] < 1.f)) return DM_E_INVAL;
   }
-  if (!connected(h, n)) return DM_E_DISCONNECTED;
+  bool bipartite = false;
+  if (!connected(h, n, &bipartite)) return DM_E_DISCONNECTED;
   DevGraph *g = new DevGraph();
+  g->bipartite = bipartite;
   g->V = n;
   g->nnz = (int64_t)h.ci.size();
   int32_t md = 0;
@@ -2956,8 +2944,25 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
     if (bytes && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return DM_E_CUDA;
     return DM_OK;
   };
-  int r = up((void **)&g->row_ptr, h.rp.data(), sizeof(int32_t) * (n + 1));
+  const bool ids16 = n <= 65534;
+  const size_t rp_bytes = sizeof(int32_t) * (n + 1), adj4_at = (rp_bytes + 15) / 16 * 16;  // adj4 behind row_ptr
+  int r = DM_OK;
+  if (ids16 && md <= 4) {
+    if (cudaMalloc(&g->row_ptr, adj4_at + sizeof(uint2) * n) != cudaSuccess) r = DM_E_NOMEM;
+    else if (cudaMemcpy(g->row_ptr, h.rp.data(), rp_bytes, cudaMemcpyHostToDevice) != cudaSuccess) r = DM_E_CUDA;
+    else g->adj4 = (uint2 *)((unsigned char *)g->row_ptr + adj4_at);
+  } else {
+    r = up((void **)&g->row_ptr, h.rp.data(), rp_bytes);
+  }
   if (r == DM_OK) r = up((void **)&g->col_idx, h.ci.data(), sizeof(int32_t) * h.ci.size());
+  // launches of several steps (chain.cu) need the girth, which comes back through a counter slot that no other
+  // work of the context uses now, and short neighbour lists; both run beside the uploads and allocations below
+  if (r == DM_OK && ids16) {
+    int32_t *d = (int32_t *)c->d_ctr;
+    if (cudaMemsetAsync(d, 0x7f, sizeof(int32_t), c->stream) != cudaSuccess ||
+        dmk::launch_girth(g->row_ptr, g->col_idx, n, d, g->adj4, c->stream) != cudaSuccess)
+      r = DM_E_CUDA;
+  }
   if (r == DM_OK && edge_err) r = up((void **)&g->eerr, h.ee.data(), sizeof(float) * h.ee.size());
   if (r == DM_OK && qubit_err) r = up((void **)&g->qerr, qubit_err, sizeof(float) * n);
   if (r == DM_OK && score_form == DM_SCORE_LOG_FIDELITY) {  // weights -log(1 - e): scores add up
@@ -2972,21 +2977,10 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
     else if (dmk::launch_bitmap(g->row_ptr, g->col_idx, n, g->nnz, g->adj_words, g->adj, c->stream) != cudaSuccess)
       r = DM_E_CUDA;
   }
-  if (r == DM_OK) {  // the girth, through a counter slot that no other work of the context uses now
-    int32_t *d = (int32_t *)c->d_ctr, *h_girth = (int32_t *)c->h_ctr;
-    *h_girth = dmk::GIRTH_MAX;
-    if (cudaMemcpyAsync(d, h_girth, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
-        dmk::launch_girth(g->row_ptr, g->col_idx, n, d, c->stream) != cudaSuccess ||
-        cudaMemcpyAsync(h_girth, d, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
-      r = DM_E_CUDA;
-    g->bipartite = two_colourable(h, n);
-    if (r == DM_OK && md <= 4 && n <= 65534) {
-      r = dalloc_t(c, &g->adj4, (size_t)n);
-      if (r == DM_OK && dmk::launch_adj4(g->row_ptr, g->col_idx, n, g->adj4, c->stream) != cudaSuccess) r = DM_E_CUDA;
-    }
-  }
+  if (r == DM_OK && ids16 && cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
+    r = DM_E_CUDA;
   if (r == DM_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) r = DM_E_CUDA;
-  if (r == DM_OK) g->girth = *(int32_t *)c->h_ctr;
+  if (r == DM_OK && ids16) g->girth = std::min(dmk::GIRTH_MAX, *(int32_t *)c->h_ctr);
   if (r == DM_OK) r = ensure_motif(c, g, 2);
   if (r != DM_OK) {  // a graph that failed to load is neither registered nor kept
     cudaGetLastError();

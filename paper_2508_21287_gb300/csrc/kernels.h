@@ -163,11 +163,12 @@ cudaError_t launch_chain_tables(const ChainTables &r, cudaStream_t s);
 // Data-graph preparation.
 cudaError_t launch_csr_to_m2(const int32_t *row_ptr, const int32_t *col_idx, const float *eerr,
                              int32_t V, int64_t nnz, int32_t *rows, float *score, cudaStream_t s);
-// *girth = min(*girth, a lower bound of the graph's girth); the caller sets it to GIRTH_MAX before.
+// *girth = min(*girth, a lower bound of the graph's girth); the caller sets it to GIRTH_MAX or more before.
+// adj4 (nullable): the neighbours of every vertex, ascending, 16 bits each, 0xFFFF past its degree (at most
+// 4; V <= 65 534).
 constexpr int GIRTH_MAX = 32;
-cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth, cudaStream_t s);
-// adj4[v]: the neighbours of v, ascending, 16 bits each, 0xFFFF past its degree (at most 4; V <= 65 534).
-cudaError_t launch_adj4(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, uint2 *adj4, cudaStream_t s);
+cudaError_t launch_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int32_t *girth, uint2 *adj4,
+                         cudaStream_t s);
 cudaError_t launch_vertex_table(int32_t V, int32_t *rows, float *score, cudaStream_t s);
 cudaError_t launch_bitmap(const int32_t *row_ptr, const int32_t *col_idx, int32_t V, int64_t nnz,
                           int32_t words, unsigned long long *adj, cudaStream_t s);
