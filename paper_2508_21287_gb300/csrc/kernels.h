@@ -269,7 +269,7 @@ struct OrderArgs {
   int32_t log2_many;                 // rows a bucket of large tables (order_layout), fewer where keys crowd
   const uint2 *adj4;                 // neighbour lists of the data graph, for columns with ref
   int32_t radix_id, radix_place;     // of a column's id, and of its place among an earlier one's neighbours
-  unsigned long long scale;          // the first word times scale is its fraction of 2^64
+  unsigned long long scale, unit;    // the first word times scale is its fraction of 2^64; 2^64 - 1 over scale
   uint8_t ref[dmi::MAXW];            // an earlier column that is a pattern neighbour, or ORD_NONE
   uint8_t word[dmi::MAXW];
   OrderWork *work;

@@ -319,11 +319,12 @@ __global__ void __launch_bounds__(ORD_BLK) k_ord_rank(const __grid_constant__ Or
   const int64_t n = ord_n(a);
   if (n == 0 || a.ctr[CTR_OVF]) return;
   const int nb = ord_buckets(a, n), wid = threadIdx.x >> 5;
-  // bucket b holds the keys k with b <= k * scale * nb / 2^64 < b + 1: none below b * floor((2^64 - 1) / nb) /
-  // scale, which is at most ORD_MAX + 2 below the bucket's edge, and 2^64 / (nb * scale) + 1 of them at most
-  const unsigned long long cut = ~0ull / nb;
-  const bool local = KW == 1 && a.packed == a.w && cut / a.scale < 0xFFFFFFFFull - 2 * ORD_MAX;
-  auto base = [&](int b) { return cut * (unsigned long long)b / a.scale; };
+  // bucket b holds the keys k with b <= k * scale * nb / 2^64 < b + 1, at most 2^64 / (nb * scale) + 1 of them:
+  // none below b * width, and width less than b + 2 short of a bucket (a division for each bucket instead took
+  // 2 us of 20 here, and 8 of a call)
+  const unsigned long long width = a.unit / nb;  // floor((2^64 - 1) / (nb * scale))
+  const bool local = KW == 1 && a.packed == a.w && width < 0xFFFFFFFFull - 2 * ORD_MAX;
+  auto base = [&](int b) { return width * (unsigned long long)b; };
   if (threadIdx.x == 0) s_large = 0;
   __syncthreads();
   for (int b = blockIdx.x * ORD_WARPS + wid; b < nb; b += gridDim.x * ORD_WARPS) {
@@ -368,6 +369,7 @@ int order_layout(OrderArgs &a, unsigned radix_id, unsigned radix_place) {
     skewed |= c && word == 0 && a.ref[c] == ORD_NONE;
   }
   a.scale = ~0ull / range[0];
+  a.unit = ~0ull / a.scale;
   a.log2_many = skewed && !a.n_dev ? ORD_FINE : 6;
   return word + 1;
 }
