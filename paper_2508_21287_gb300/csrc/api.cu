@@ -2339,7 +2339,7 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
       cudaGetLastError();
       return DM_E_NOMEM;
     }
-    cudaError_t e = bytes ? cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
+    cudaError_t e = bytes ? cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, c->stream) : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(c, e, "batch upload");
     return DM_OK;
   };
@@ -2390,6 +2390,7 @@ int batch_build(dm_ctx *c, DevGraph *g, const dm_plan_t *const *plans, int32_t n
   P.sigs = (const uint32_t *const *)b->d_sigs;
   P.sig_units = sig_units;
   P.scratch = (unsigned char *)b->scratch;
+  CK(cudaStreamSynchronize(c->stream));  // the uploads' sources end here
   *out = b.release();
   return DM_OK;
 }
@@ -2503,9 +2504,9 @@ int model_alloc(dm_ctx *c) {
     cudaGetLastError();
     return DM_E_NOMEM;
   }
-  CK(cudaMemset(c->m_grads, 0, b));
-  CK(cudaMemset(c->m_m, 0, b));
-  CK(cudaMemset(c->m_v, 0, b));
+  CK(cudaMemsetAsync(c->m_grads, 0, b, c->stream));
+  CK(cudaMemsetAsync(c->m_m, 0, b, c->stream));
+  CK(cudaMemsetAsync(c->m_v, 0, b, c->stream));
   return DM_OK;
 }
 
@@ -2939,9 +2940,11 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
   for (int32_t u = 0; u < n; u++) deg2 += (double)(h.rp[u + 1] - h.rp[u]) * (h.rp[u + 1] - h.rp[u]);
   g->edge_deg = g->nnz ? deg2 / (double)g->nnz : 0.0;
   g->nonneg_weights = nonneg;
+  // in stream order: a copy outside it returns once its source is staged, and the context's stream, which does
+  // not wait for the default one, could read the arrays before they are there
   auto up = [&](void **dst, const void *src, size_t bytes) -> int {
     if (cudaMalloc(dst, std::max<size_t>(bytes, 16)) != cudaSuccess) return DM_E_NOMEM;
-    if (bytes && cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return DM_E_CUDA;
+    if (bytes && cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) return DM_E_CUDA;
     return DM_OK;
   };
   const bool ids16 = n <= 65534;
@@ -2949,7 +2952,7 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
   int r = DM_OK;
   if (ids16 && md <= 4) {
     if (cudaMalloc(&g->row_ptr, adj4_at + sizeof(uint2) * n) != cudaSuccess) r = DM_E_NOMEM;
-    else if (cudaMemcpy(g->row_ptr, h.rp.data(), rp_bytes, cudaMemcpyHostToDevice) != cudaSuccess) r = DM_E_CUDA;
+    else if (cudaMemcpyAsync(g->row_ptr, h.rp.data(), rp_bytes, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) r = DM_E_CUDA;
     else g->adj4 = (uint2 *)((unsigned char *)g->row_ptr + adj4_at);
   } else {
     r = up((void **)&g->row_ptr, h.rp.data(), rp_bytes);
@@ -3554,7 +3557,8 @@ int dm_load_directed_errors(dm_ctx *c, dm_graph gh, const float *e_dir) {
     cudaGetLastError();
     return DM_E_NOMEM;
   }
-  if (cudaMemcpy(d, e_dir, sizeof(float) * g->nnz, cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (cudaMemcpyAsync(d, e_dir, sizeof(float) * g->nnz, cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess) {
     const cudaError_t e = cudaGetLastError();
     cudaFree(d);
     return cuda_fail(c, e, "directed errors upload");
@@ -3727,7 +3731,8 @@ int dm_model_set_weights(dm_ctx *c, const float *w, int64_t n) {
   if (!c || !w || n != P + 2 * NFEAT) return DM_E_INVAL;
   cudaSetDevice(c->device);
   RET(model_alloc(c));
-  CK(cudaMemcpy(c->m_params, w, sizeof(float) * P, cudaMemcpyHostToDevice));
+  CK(cudaMemcpyAsync(c->m_params, w, sizeof(float) * P, cudaMemcpyHostToDevice, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
   for (int k = 0; k < NFEAT; k++) {
     c->m_mean[k] = w[P + k];
     c->m_std[k] = w[P + NFEAT + k] > 0.f ? w[P + NFEAT + k] : 1.f;
@@ -3741,7 +3746,7 @@ int dm_model_grad(dm_ctx *c, const float *feats, const float *targets, int32_t n
   if (!c || !feats || n < 1 || !c->m_params) return DM_E_INVAL;
   cudaSetDevice(c->device);
   const int64_t P = dmk::mlp_param_count();
-  if (targets) CK(cudaMemset(c->m_grads, 0, sizeof(float) * P));
+  if (targets) CK(cudaMemsetAsync(c->m_grads, 0, sizeof(float) * P, c->stream));
   RET(model_run(c, feats, targets, n, out_pred, targets ? c->m_grads : nullptr, out_loss));
   if (targets && out_grads) CK(cudaMemcpy(out_grads, c->m_grads, sizeof(float) * P, cudaMemcpyDeviceToHost));
   return DM_OK;
