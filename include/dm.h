@@ -285,6 +285,12 @@ int dm_set_fusion(dm_ctx *ctx, int on);
  * value. DM_E_INVAL if negative. */
 int dm_set_launch_limit(dm_ctx *ctx, int32_t candidates);
 
+/* Most rows of a table that is put in order or selected from (no counterpart in the paper; 0 = the
+ * default, 2^31 - 1: rows have 32-bit numbers there). Larger results are streamed in chunks of at most
+ * that many rows, as results beyond the memory budget are; dm_images and motif tables, which are one table,
+ * give DM_E_CAPACITY. DM_E_INVAL if negative. */
+int dm_set_table_limit(dm_ctx *ctx, int32_t rows);
+
 /* Block shape of dm_match_batch when autotuning is off (no counterpart in the paper):
  * threads_per_cta 128 or 256 (every CTA walks its work items through the plan's steps in
  * tiles of the tuned row count), or 32 (every warp walks its own work items in 32-row tiles,

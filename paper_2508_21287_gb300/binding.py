@@ -120,6 +120,7 @@ _SIGS = {
     "dm_set_batch_shape": (ctypes.c_int, [_vp, _i32, _i32]),
     "dm_set_fusion": (ctypes.c_int, [_vp, ctypes.c_int]),
     "dm_set_launch_limit": (ctypes.c_int, [_vp, _i32]),
+    "dm_set_table_limit": (ctypes.c_int, [_vp, _i32]),
     "dm_batch_latency": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_double), _i32]),
     "dm_set_tuning": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_double, ctypes.c_double]),
     "dm_model_init": (ctypes.c_int, [_vp, _u64]),
@@ -489,6 +490,10 @@ def dm_set_fusion(ctx, on: bool = True) -> None:
 
 def dm_set_launch_limit(ctx, candidates: int = 0) -> None:
     _check(_lib.dm_set_launch_limit(ctx, int(candidates)), "dm_set_launch_limit", ctx)
+
+
+def dm_set_table_limit(ctx, rows: int = 0) -> None:
+    _check(_lib.dm_set_table_limit(ctx, int(rows)), "dm_set_table_limit", ctx)
 
 
 def dm_batch_latency(ctx, n: int) -> np.ndarray:

@@ -114,6 +114,7 @@ struct dm_ctx {
   double heavy_rows = 1e300;          // plans predicted to hold more rows run step by step
   int batch_threads = 256, batch_ctas = 0;  // block shape of dm_match_batch without autotuning
   uint32_t launch_limit = 1u << 20;  // a warp's candidates (dm_set_launch_limit): about 2.5e9 a launch, tens of ms
+  int64_t table_rows = INT32_MAX;    // of a table that is put in order or selected from: its rows have 32-bit numbers
   bool fuse_last = false;  // counted plans: the last two joins in one launch when they qualify
   std::vector<double> batch_latency;  // per plan, ms from the start of the last dm_match_batch
 };
@@ -708,7 +709,7 @@ struct Exec {
 
   int64_t limit_rows(int j) const {
     int64_t avail = (int64_t)c->budget - c->inflight;
-    int64_t lim = std::max<int64_t>(1, avail / row_bytes(j));
+    int64_t lim = std::min(std::max<int64_t>(1, avail / row_bytes(j)), c->table_rows);
     if (chunk_rows > 0) lim = std::min(lim, chunk_rows);
     return lim;
   }
@@ -877,6 +878,7 @@ struct Exec {
       const int64_t ows = a.rs_out ? a.rs_out : a.wo;  // output row stride in words
       int64_t rb = 4ll * ows + (a.scored ? 4 : 0);
       int64_t cap = std::max<int64_t>(1, ((int64_t)half - 512) / rb);
+      if (j + 1 == S) cap = std::min(cap, c->table_rows);
       int32_t *orows = (int32_t *)buf[j & 1];
       float *oscore = (float *)(buf[j & 1] + ((size_t)cap * ows * 4 + 255) / 256 * 256);
       a.out = a.mode == 0 ? orows : nullptr;
@@ -1396,7 +1398,7 @@ struct Exec {
       if (A.out_kind == 1) {
         unsigned char *buf = c->arena + (i & 1) * half;
         const int64_t rb = 4ll * A.wo + (A.scored ? 4 : 0);
-        A.out_cap = std::max<int64_t>(1, ((int64_t)half - 512) / rb);
+        A.out_cap = std::min(std::max<int64_t>(1, ((int64_t)half - 512) / rb), c->table_rows);
         A.out = (int32_t *)buf;
         A.outs = A.scored ? (float *)(buf + ((size_t)A.out_cap * A.wo * 4 + 255) / 256 * 256) : nullptr;
       }
@@ -1620,6 +1622,11 @@ struct CollectSink : Sink {
   int concat(dm_ctx *c, int32_t w, bool scored, DevTable *out) {
     int64_t n = 0;
     for (auto &p : parts) n += p.n;
+    if (n > c->table_rows) {
+      for (auto &p : parts) free_table(c, p);
+      parts.clear();
+      return DM_E_CAPACITY;
+    }
     DevTable o;
     o.n = n;
     o.w = w;
@@ -1680,7 +1687,7 @@ struct AllSink : Sink {
   void *user;
   int bits;
   std::vector<DevTable> held;
-  int64_t held_bytes = 0;
+  int64_t held_bytes = 0, held_rows = 0;
   bool streaming = false;
   uint64_t count = 0, checksum = 0;
   // host buffers of the caller's top-k: when the whole result is one table, its top-k is
@@ -1825,9 +1832,10 @@ struct AllSink : Sink {
       return r;
     }
     crowded = tried && h_ahead[CTR_OVF] && t.n <= sorted.n;
-    if (!streaming && held_bytes + tb <= (int64_t)c->budget / 2) {
+    if (!streaming && held_bytes + tb <= (int64_t)c->budget / 2 && held_rows + t.n <= c->table_rows) {
       held.push_back(t);
       held_bytes += tb;
+      held_rows += t.n;
       return DM_OK;
     }
     streaming = true;
@@ -3480,6 +3488,12 @@ int dm_set_batch_shape(dm_ctx *c, int32_t threads_per_cta, int32_t ctas_per_sm) 
 int dm_set_launch_limit(dm_ctx *c, int32_t candidates) {
   if (!c || candidates < 0) return DM_E_INVAL;
   c->launch_limit = candidates ? (uint32_t)candidates : 1u << 20;
+  return DM_OK;
+}
+
+int dm_set_table_limit(dm_ctx *c, int32_t rows) {
+  if (!c || rows < 0) return DM_E_INVAL;
+  c->table_rows = rows ? rows : INT32_MAX;
   return DM_OK;
 }
 
