@@ -532,8 +532,8 @@ def measure_queries(args, kind: str, with_e2e: bool, with_cpu: bool, fuse: bool 
     achieved = racc["join_bytes"] / (racc["join_ms"] / 1e3) / 1e9 if racc["join_ms"] > 0 else 0.0
     digest = join_kernel_digest()
     traffic = JOIN_TRAFFIC_BYTES_PER_LAUNCH.get((workload_key(args, kind), digest))
-    roofline = {"bound": "hbm", "kernel": "k_chain", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "peak_source": "measured (burst copy)" if "hbm_gbs" in peaks else "fallback",
+    roofline = {"bound": "instructions", "kernel": "k_chain", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "frac_of": "hbm", "peak_source": "measured (burst copy)" if "hbm_gbs" in peaks else "fallback",
                 "traffic": traffic, "kernel_digest": digest,
                 "algorithmic_bytes_per_launch": racc["join_bytes"] / max(1, racc["join_launches"]),
                 "avg_launch_us": 1e3 * racc["join_ms"] / max(1, racc["join_launches"]),

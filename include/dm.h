@@ -94,7 +94,8 @@ typedef struct dm_plan_opts {
  * of its graphs and tables. mem_budget_bytes bounds the device memory the intermediate tables
  * of one dm_match may hold (0 = half of the free memory at creation); larger results are
  * streamed in chunks (depth-first over the join steps). Tables of what a plan's candidates bring
- * stay with the context beside that, at most an eighth of the budget and 256 MB. Errors: DM_E_INVAL (out NULL),
+ * stay with the context beside that, at most an eighth of the budget and 256 MB, and so do work buffers
+ * of the order of results (8.4 MB), of the selection of best rows (1 MB) and of training (64 MB). Errors: DM_E_INVAL (out NULL),
  * DM_E_CUDA (no such device, or stream/event creation failed), DM_E_NOMEM. */
 int dm_create(dm_ctx **out, int device, uint64_t mem_budget_bytes);
 
