@@ -2966,16 +2966,16 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
     r = up((void **)&g->row_ptr, h.rp.data(), rp_bytes);
   }
   if (r == DM_OK) r = up((void **)&g->col_idx, h.ci.data(), sizeof(int32_t) * h.ci.size());
+  if (r == DM_OK && edge_err) r = up((void **)&g->eerr, h.ee.data(), sizeof(float) * h.ee.size());
+  if (r == DM_OK && qubit_err) r = up((void **)&g->qerr, qubit_err, sizeof(float) * n);
   // launches of several steps (chain.cu) need the girth, which comes back through a counter slot that no other
-  // work of the context uses now, and short neighbour lists; both run beside the uploads and allocations below
+  // work of the context uses now, and short neighbour lists; both run beside the allocations below
   if (r == DM_OK && ids16) {
     int32_t *d = (int32_t *)c->d_ctr;
     if (cudaMemsetAsync(d, 0x7f, sizeof(int32_t), c->stream) != cudaSuccess ||
         dmk::launch_girth(g->row_ptr, g->col_idx, n, d, g->adj4, c->stream) != cudaSuccess)
       r = DM_E_CUDA;
   }
-  if (r == DM_OK && edge_err) r = up((void **)&g->eerr, h.ee.data(), sizeof(float) * h.ee.size());
-  if (r == DM_OK && qubit_err) r = up((void **)&g->qerr, qubit_err, sizeof(float) * n);
   if (r == DM_OK && score_form == DM_SCORE_LOG_FIDELITY) {  // weights -log(1 - e): scores add up
     if (g->eerr && dmk::launch_neg_log1m(g->eerr, (int64_t)h.ee.size(), c->stream) != cudaSuccess) r = DM_E_CUDA;
     if (g->qerr && dmk::launch_neg_log1m(g->qerr, n, c->stream) != cudaSuccess) r = DM_E_CUDA;

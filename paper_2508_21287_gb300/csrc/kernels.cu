@@ -85,10 +85,10 @@ cudaError_t launch_bitmap(const int32_t *row_ptr, const int32_t *col_idx, int32_
 // length met over all v is the girth. A warp whose search outgrows GIRTH_LIST vertices reports what it has
 // seen in full, plus one: the result never exceeds the girth (up to GIRTH_MAX, which stands for "at least
 // that"). On lattices a search ends within 40 vertices, six levels of two dependent loads each: what bounds it.
-// A lane a vertex of the level, all lanes looking for their neighbours in the list at once; and started before
-// the weights and the bitmap are uploaded. Loading a graph of 159 vertices took 154 us with a thread a vertex
-// (most of it this kernel), 70 so and 55 without the girth (64 so with the uploads in stream order); 16 082
-// vertices 654, 564 and 547.
+// A lane a vertex of the level, all lanes looking for their neighbours in the list at once; started before the
+// bitmap's memory is asked for (ahead of the weights' uploads in the same stream instead, 16 082 vertices took
+// 650 us). Loading a graph of 159 vertices took 154 us with a thread a vertex (most of it this kernel), 63 so and
+// 55 without the girth; 16 082 vertices 654, 578 and 547.
 constexpr int GIRTH_LIST = 96, GIRTH_WARPS = 4;
 __global__ void __launch_bounds__(32 * GIRTH_WARPS) k_girth(const int32_t *row_ptr, const int32_t *col_idx, int32_t V,
                                                             int32_t *girth, uint2 *adj4) {
