@@ -66,6 +66,7 @@ struct DevGraph {
   // girth, and whether every cycle is even
   int32_t girth = 3;
   bool bipartite = false;
+  float uneven = 1.f;  // how many times the mean the largest neighbourhood is (uneven_walks)
   uint2 *adj4 = nullptr;  // neighbour lists of 16-bit ids, where no degree is above 4 (in row_ptr's allocation)
   double edge_deg = 0;  // mean degree of the vertices that edges lead to
   std::map<int, DevTable> motifs;
@@ -254,6 +255,34 @@ bool connected(const HostCSR &g, int32_t n, bool *bipartite = nullptr) {
   }
   if (bipartite) *bipartite = !odd;
   return cnt == n;
+}
+
+// Walks of UNEVEN_STEPS edges that do not turn back, from the vertex that has most over the mean of all. Lattices
+// stay below 1.7 (borders) and count as even: 1; random trees with a few more edges have 2.3 to 4.2.
+constexpr int UNEVEN_STEPS = 3;
+constexpr double UNEVEN_FROM = 2.0;
+float uneven_walks(const HostCSR &g, int32_t n) {
+  bool regular = true;
+  for (int32_t u = 1; u < n; u++) regular &= g.rp[u + 1] - g.rp[u] == g.rp[1];
+  if (regular) return 1.f;
+  std::vector<float> a(n), b(n), d(n);  // walks of k - 1 and k edges
+  for (int32_t u = 0; u < n; u++) b[u] = d[u] = (float)(g.rp[u + 1] - g.rp[u]);
+  for (int k = 1; k < UNEVEN_STEPS; k++) {
+    for (int32_t u = 0; u < n; u++) {  // walks on from each neighbour, less those that come back to u
+      float x = k == 1 ? -d[u] : -(d[u] - 1.f) * a[u];
+      for (int32_t e = g.rp[u]; e < g.rp[u + 1]; e++) x += b[g.ci[e]];
+      a[u] = x;  // (k - 1 edges are not needed any more)
+    }
+    a.swap(b);
+  }
+  double sum = 0;
+  float most = 0;
+  for (int32_t u = 0; u < n; u++) {
+    sum += b[u];
+    most = std::max(most, b[u]);
+  }
+  const double r = sum > 0 ? most * (double)n / sum : 1.0;
+  return r > UNEVEN_FROM ? (float)r : 1.f;
 }
 
 // ------------------------------------------------------------------ sorting ------------
@@ -474,6 +503,7 @@ struct Sink {
   // k > 0: only the k best rows are wanted, and rows whose partial score is above the k-th best of those
   // seen may be dropped; hist receives where the joins count the scores of what they write
   virtual int64_t best_only(dm_ctx *, dmk::SelHist **) { return 0; }
+  virtual bool few() const { return false; }  // whether best_only() will say so
 };
 
 struct StepRT {
@@ -497,6 +527,13 @@ constexpr int64_t CHAIN_TAB_BYTES = 256ll << 20, CHAIN_TAB_MIN = 4ll << 20;
 // more runs a launch a step.
 int64_t chain_tab_limit(uint64_t budget) { return std::min<int64_t>(CHAIN_TAB_BYTES, (int64_t)(budget / 8)); }
 constexpr double CHAIN_LAUNCH_NS = 4000, CHAIN_ROW_NS = 0.03, CHAIN_BYTE_NS = 0.0002;
+// ... and of a row to the warp that joins it: all rows that come from one row of a launch's first table are one
+// warp's, so a launch lasts at least as long as the largest of them. A 7-vertex path in a clique of 11: 1.7 M
+// rows from 110, 158 us in one launch. On graphs whose neighbourhoods are uneven (above) the largest has many
+// times the mean: its size is taken to grow by a factor for each new vertex, but for best rows, whose bound cuts
+// it short. An end shorter than CHAIN_TAIL_NS costs less than dealing the rows out anew. A 16-vertex tree on a
+// random tree of 474 vertices with 60 edges more: 1070 us in one launch (150 a step a launch), 152 so.
+constexpr double CHAIN_WARP_NS = 36, CHAIN_TAIL_NS = 20000;
 // The smallest arena that tables go into: the parts it is cut into then hold a block or a row of any width.
 constexpr size_t ARENA_MIN = 64 << 10;
 // Rows of work that an item of a launch's input stands for at the least: each further item is a turn
@@ -1173,18 +1210,28 @@ struct Exec {
       C.work += r;
       C.most = std::max(C.most, r);
     }
+    std::vector<double> grow(S, 1.0);  // the largest of a first table's rows against the mean, by a step
+    const bool few = sink && sink->few();
+    for (int j = 1; j < S && g->uneven > 1.f && !few; j++) grow[j] = pow((double)g->uneven, (double)p->steps[j].n_new / UNEVEN_STEPS);
     std::vector<double> cost(S + 1, 1e300);  // steps 1 .. j done, tile j + 1 written
     std::vector<int> from(S + 1, -1);
     cost[0] = 0;
     for (int j = 1; j < S; j++) {
-      double work = 0;
+      double work = 0, largest = 1;
       for (int i = j - 1; i >= 0; i--) {  // one launch of steps i + 1 .. j
         const bool end = j == S - 1;
         const int need_smem = bytes(i + 1, end ? last_tile : j + 1) * dmk::CH_CTA_WARPS;
         work += rows[i + 1];
+        largest *= grow[i + 1];
         if (j - i > dmk::CH_STEPS || need_smem > dmk::CH_SMEM_MAX) break;
         const double warps = std::min(CHAIN_WARPS, CHAIN_SM_BYTES / need_smem * dmk::CH_CTA_WARPS);
-        const double x = cost[i] + CHAIN_LAUNCH_NS + CHAIN_ROW_NS * work * CHAIN_WARPS / warps +
+        // rows of the first table that one warp takes at a time (run_chain, k_chain)
+        const double all = warps * c->num_sms, blocks = std::max(rows[i] / 32, std::min(rows[i], all));
+        const double take = i ? std::max(1.0, rows[i] / (blocks * (blocks >= 8 * all ? 1 : blocks < 4 * all ? 4 : 2)))
+                              : std::max(2 * rows[0] > all ? 1.0 : 4 * rows[0] > all ? 0.5 : 0.25, rows[0] / (8 * all));
+        const double item = take * work / std::max(1.0, rows[i]) * largest;
+        const double x = cost[i] + CHAIN_LAUNCH_NS +
+                         std::max(CHAIN_ROW_NS * work * CHAIN_WARPS / warps, CHAIN_WARP_NS * item - CHAIN_TAIL_NS) +
                          (end ? 0.0 : CHAIN_BYTE_NS * 16.0 * (nc[j + 1] + 1) * rows[j]);
         if (x < cost[j]) {
           cost[j] = x;
@@ -2012,8 +2059,9 @@ struct TopkSink : Sink {
   bool counts() const override { return false; }
   void forget() override { tried = false; }
   bool counted = false;       // the joins count the scores and lower the bound (best_only)
+  bool few() const override { return prune_ptr && !input_sorted && !have && k <= dmk::SEL_K; }
   int64_t best_only(dm_ctx *c, dmk::SelHist **hist) override {
-    if (!prune_ptr || input_sorted || have || k > dmk::SEL_K) return 0;
+    if (!few()) return 0;
     RET(select_work(c));
     *hist = (dmk::SelHist *)c->sel_work;
     c->sel_dirty = true;  // until the selection that follows has run
@@ -2988,6 +3036,7 @@ int dm_load_data_graph_ex(dm_ctx *c, int32_t n, const int32_t *row_ptr, const in
     else if (dmk::launch_bitmap(g->row_ptr, g->col_idx, n, g->nnz, g->adj_words, g->adj, c->stream) != cudaSuccess)
       r = DM_E_CUDA;
   }
+  if (ids16) g->uneven = uneven_walks(h, n);  // while the device is busy
   if (r == DM_OK && ids16 && cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess)
     r = DM_E_CUDA;
   if (r == DM_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) r = DM_E_CUDA;
