@@ -1753,7 +1753,12 @@ struct AllSink : Sink {
   int flush_one(dm_ctx *c, DevTable &t, bool last = false) {
     CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(unsigned long long) * CTR_N, c->stream));
     DevTable o;
-    bool keyed = t.even && !very_crowded && t.n > dmk::msort_into_max_rows() && t.n <= dmk::ORD_ROWS && order_table(c, t, &o) == DM_OK;
+    // keys that crowded behind the joins: finer buckets, or at once the sort. On graphs of uneven neighbourhoods most
+    // keys are a hub's and finer buckets crowd, too: trees with hubs, 53 000 rows 284 us so and 220 sorted, 149 000
+    // 1072 and 327, 574 000 2586 and 724, 6.1 M 6705 and 5883. On lattices they spread them where the table is
+    // large (rows of scrambled paths: 655 000 835 to 1120 and 708, 3.5 M 2260 to 2660 and 3200 to 3310).
+    const bool sort = very_crowded || (crowded && t.n < (g->uneven > 1.f ? 1 << 23 : 1 << 20));
+    bool keyed = t.even && !sort && t.n > dmk::msort_into_max_rows() && t.n <= dmk::ORD_ROWS && order_table(c, t, &o) == DM_OK;
     if (!keyed) RET(sort_canonical(c, t, bits, c->d_ctr));
     const bool fast_topk = last && tap && final_rows && topk_small_enough(tap);
     const int64_t k = fast_topk ? topk_k(tap) : 0;

@@ -16,7 +16,7 @@
 // k_ord_keys packs the keys, sums the rows' checksum and takes every row's number in its bucket,
 // k_ord_scan finds the buckets' places, k_ord_deal puts the rows' indices there, and k_ord_rank orders
 // each bucket's rows in shared memory (a warp a bucket; a block for the few large ones) and copies rows and
-// scores to their final places. A bucket of more than ORD_BUCKET rows is reported. The caller tries again with
+// scores to their final places. A bucket of more than ORD_BUCKET rows is reported. The caller tries large tables again with
 // the row count in hand, buckets of ORD_FINE and blocks that order up to ORD_CROWDED rows by keys they leave
 // in memory, and sorts another way where that is not enough.
 //
